@@ -127,23 +127,25 @@ __device__ inline T warp_sum(T v) {
   return v;
 }
 
-// Four sums over the warp in 6 additions per lane instead of 20 (FP64 additions issue at one
-// per 16 cycles here): the halves of the warp first split the four values among themselves,
-// then every group of 8 lanes reduces one of them.
-__device__ inline void warp_sum4(double& a, double& b, double& c, double& d) {
+// Total mass and centre-of-mass velocity from the lanes' masses and momenta: four sums over the
+// warp in 6 additions per lane instead of 20 (FP64 additions issue at one per 16 cycles here):
+// the halves of the warp first split the four values among themselves, then every group of 8
+// lanes reduces one of them and divides it by the mass (a true division: a group of one atom
+// has no relative velocity).
+__device__ inline void warp_centre(double sm, double& px, double& py, double& pz) {
   const int lane = threadIdx.x & 31;
   const bool hi = lane & 16, mid = lane & 8;
-  double k0 = hi ? c : a, k1 = hi ? d : b;
-  k0 += __shfl_xor_sync(0xffffffffu, hi ? a : c, 16);
-  k1 += __shfl_xor_sync(0xffffffffu, hi ? b : d, 16);
+  double k0 = hi ? py : sm, k1 = hi ? pz : px;
+  k0 += __shfl_xor_sync(0xffffffffu, hi ? sm : py, 16);
+  k1 += __shfl_xor_sync(0xffffffffu, hi ? px : pz, 16);
   double k = mid ? k1 : k0;
   k += __shfl_xor_sync(0xffffffffu, mid ? k0 : k1, 8);
 #pragma unroll
   for (int o = 4; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
-  a = __shfl_sync(0xffffffffu, k, 0);
-  b = __shfl_sync(0xffffffffu, k, 8);
-  c = __shfl_sync(0xffffffffu, k, 16);
-  d = __shfl_sync(0xffffffffu, k, 24);
+  k = k / __shfl_sync(0xffffffffu, k, 0);
+  px = __shfl_sync(0xffffffffu, k, 8);
+  py = __shfl_sync(0xffffffffu, k, 16);
+  pz = __shfl_sync(0xffffffffu, k, 24);
 }
 
 // Member test for row entry t of atom i: a mobile atom other than i that, with DEDUP, does
@@ -261,9 +263,8 @@ __global__ void __launch_bounds__(32) k_th_rescale(
         spz += mq * v[3 * q + 2];
       }
     }
-    warp_sum4(sm, spx, spy, spz);
-    const double inv_m = 1.0 / sm;
-    const double vcx = spx * inv_m, vcy = spy * inv_m, vcz = spz * inv_m;
+    double vcx = spx, vcy = spy, vcz = spz;
+    warp_centre(sm, vcx, vcy, vcz);
     // relative kinetic energy
     double k = 0.0;
     if (lane == 0) {
