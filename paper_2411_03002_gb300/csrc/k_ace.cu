@@ -17,9 +17,9 @@
 //   k_ace_nu3      one lane per precise atom: the nu = 3 energy and gradient with A
 //                  and dE/dA in registers, straight-line code over the merged
 //                  monomials generated from the basis (ace_nu3.inc);
-//   k_ace_adjoint  one warp per precise atom: u = W^T dE/dA / N0; lanes recompute g,
-//                  g', Y, grad Y per in-range neighbour, contract with u, and scatter
-//                  -w_i p_ij to neighbour j and +w_i sum p to i.
+//   k_ace_adjoint  8 or 16 lanes per precise atom: u = W^T dE/dA / N0; each lane evaluates
+//                  the pair force of one neighbour at a time from u (pair_force) and
+//                  scatters -w_i p_ij to neighbour j; +w_i sum p goes to i.
 #include <complex>
 #include <algorithm>
 #include <cstring>
@@ -78,33 +78,24 @@ __device__ inline typename V<R>::R4 ld4(const R* p) {
 
 __device__ inline int l_of(int lm) { return lm >= 16 ? 4 : lm >= 9 ? 3 : lm >= 4 ? 2 : lm >= 1 ? 1 : 0; }
 
-// Radial functions g_k and (optionally) dg_k/dr for r < rc.
-template <typename R, bool D>
-__device__ inline void radial(R r, R inv_rc, int mode, R g[8], R dg[8]) {
+// Radial functions g_k = T_k(c) f_cut, c = 2 r/rc - 1, for r < rc.
+template <typename R>
+__device__ inline void radial(R r, R inv_rc, int mode, R g[8]) {
   R x = r * inv_rc;
   R t = mode == 1 ? R(2) * x - R(1) : x;
   R t2 = t * t;
   R poly = R(1) - R(1.875) * t + R(1.25) * t2 * t - R(0.375) * t2 * t2 * t;
   R fc = mode == 1 ? R(0.5) * poly : poly;
-  R dfc = (R(-1.875) + R(3.75) * t2 - R(1.875) * t2 * t2) * inv_rc;
   R c = R(2) * x - R(1);
-  R T0 = R(1), T1 = c, dT0 = R(0), dT1 = R(1);
+  R T0 = R(1), T1 = c;
   g[0] = fc;
   g[1] = c * fc;
-  if (D) {
-    dg[0] = dfc;
-    dg[1] = R(2) * inv_rc * fc + c * dfc;
-  }
 #pragma unroll
   for (int k = 2; k < 8; ++k) {
     R T2 = R(2) * c * T1 - T0;
-    R dT2 = R(2) * T1 + R(2) * c * dT1 - dT0;
     g[k] = T2 * fc;
-    if (D) dg[k] = dT2 * R(2) * inv_rc * fc + T2 * dfc;
     T0 = T1;
     T1 = T2;
-    dT0 = dT1;
-    dT1 = dT2;
   }
 }
 
@@ -138,65 +129,6 @@ __device__ inline void sh_values(R x, R y, R z, R Y[25]) {
   Y[22] = R(0.47308734787878004) * (x2 - y2) * (R(6) * z2 - rho);
   Y[23] = R(1.7701307697799304) * x * z * (x2 - R(3) * y2);
   Y[24] = R(0.6258357354491761) * (x2 * x2 - R(6) * x2 * y2 + y2 * y2);
-}
-
-// Block l of the homogeneous solid harmonics Z_lm (= Y_lm on the unit sphere) and
-// their Cartesian gradients; the tangential gradient is grad Z - l Z u.
-template <typename R, int L>
-__device__ inline void sh_block(R x, R y, R z, R* Y, R* gx, R* gy, R* gz) {
-  const R x2 = x * x, y2 = y * y, z2 = z * z;
-  if constexpr (L == 0) {
-    Y[0] = R(0.28209479177387814);
-    gx[0] = gy[0] = gz[0] = R(0);
-  } else if constexpr (L == 1) {
-    const R c = R(0.4886025119029199);
-    Y[0] = c * y; gx[0] = R(0); gy[0] = c; gz[0] = R(0);
-    Y[1] = c * z; gx[1] = R(0); gy[1] = R(0); gz[1] = c;
-    Y[2] = c * x; gx[2] = c; gy[2] = R(0); gz[2] = R(0);
-  } else if constexpr (L == 2) {
-    const R a = R(1.0925484305920792), b = R(0.31539156525252005), e = R(0.5462742152960396);
-    Y[0] = a * x * y; gx[0] = a * y; gy[0] = a * x; gz[0] = R(0);
-    Y[1] = a * y * z; gx[1] = R(0); gy[1] = a * z; gz[1] = a * y;
-    Y[2] = b * (R(2) * z2 - x2 - y2); gx[2] = R(-2) * b * x; gy[2] = R(-2) * b * y; gz[2] = R(4) * b * z;
-    Y[3] = a * x * z; gx[3] = a * z; gy[3] = R(0); gz[3] = a * x;
-    Y[4] = e * (x2 - y2); gx[4] = R(2) * e * x; gy[4] = R(-2) * e * y; gz[4] = R(0);
-  } else if constexpr (L == 3) {
-    const R c3 = R(0.5900435899266435), c2 = R(2.890611442640554), c1 = R(0.4570457994644658);
-    const R c0 = R(0.3731763325901154), c2h = R(1.445305721320277);
-    Y[0] = c3 * y * (R(3) * x2 - y2); gx[0] = c3 * R(6) * x * y; gy[0] = c3 * (R(3) * x2 - R(3) * y2); gz[0] = R(0);
-    Y[1] = c2 * x * y * z; gx[1] = c2 * y * z; gy[1] = c2 * x * z; gz[1] = c2 * x * y;
-    Y[2] = c1 * y * (R(4) * z2 - x2 - y2); gx[2] = c1 * R(-2) * x * y;
-    gy[2] = c1 * (R(4) * z2 - x2 - R(3) * y2); gz[2] = c1 * R(8) * y * z;
-    Y[3] = c0 * z * (R(2) * z2 - R(3) * x2 - R(3) * y2); gx[3] = c0 * R(-6) * x * z; gy[3] = c0 * R(-6) * y * z;
-    gz[3] = c0 * (R(6) * z2 - R(3) * x2 - R(3) * y2);
-    Y[4] = c1 * x * (R(4) * z2 - x2 - y2); gx[4] = c1 * (R(4) * z2 - R(3) * x2 - y2);
-    gy[4] = c1 * R(-2) * x * y; gz[4] = c1 * R(8) * x * z;
-    Y[5] = c2h * z * (x2 - y2); gx[5] = c2h * R(2) * x * z; gy[5] = c2h * R(-2) * y * z; gz[5] = c2h * (x2 - y2);
-    Y[6] = c3 * x * (x2 - R(3) * y2); gx[6] = c3 * (R(3) * x2 - R(3) * y2); gy[6] = c3 * R(-6) * x * y; gz[6] = R(0);
-  } else {
-    const R a = R(2.5033429417967046), b = R(1.7701307697799304), c = R(0.9461746957575601);
-    const R d = R(0.6690465435572892), e = R(0.10578554691520431), f = R(0.47308734787878004);
-    const R g = R(0.6258357354491761);
-    const R rho = x2 + y2;
-    Y[0] = a * x * y * (x2 - y2); gx[0] = a * (R(3) * x2 * y - y2 * y); gy[0] = a * (x2 * x - R(3) * x * y2); gz[0] = R(0);
-    Y[1] = b * y * z * (R(3) * x2 - y2); gx[1] = b * R(6) * x * y * z; gy[1] = b * (R(3) * x2 * z - R(3) * y2 * z);
-    gz[1] = b * (R(3) * x2 * y - y2 * y);
-    Y[2] = c * x * y * (R(6) * z2 - rho); gx[2] = c * (R(6) * y * z2 - R(3) * x2 * y - y2 * y);
-    gy[2] = c * (R(6) * x * z2 - x2 * x - R(3) * x * y2); gz[2] = c * R(12) * x * y * z;
-    Y[3] = d * y * z * (R(4) * z2 - R(3) * rho); gx[3] = d * R(-6) * x * y * z;
-    gy[3] = d * (R(4) * z2 * z - R(3) * x2 * z - R(9) * y2 * z); gz[3] = d * (R(12) * y * z2 - R(3) * x2 * y - R(3) * y2 * y);
-    Y[4] = e * (R(8) * z2 * z2 - R(24) * z2 * rho + R(3) * rho * rho);
-    gx[4] = e * x * (R(12) * rho - R(48) * z2); gy[4] = e * y * (R(12) * rho - R(48) * z2);
-    gz[4] = e * (R(32) * z2 * z - R(48) * z * rho);
-    Y[5] = d * x * z * (R(4) * z2 - R(3) * rho); gx[5] = d * (R(4) * z2 * z - R(9) * x2 * z - R(3) * y2 * z);
-    gy[5] = d * R(-6) * x * y * z; gz[5] = d * (R(12) * x * z2 - R(3) * x2 * x - R(3) * x * y2);
-    Y[6] = f * (x2 - y2) * (R(6) * z2 - rho); gx[6] = f * (R(12) * x * z2 - R(4) * x2 * x);
-    gy[6] = f * (R(-12) * y * z2 + R(4) * y2 * y); gz[6] = f * (R(12) * x2 * z - R(12) * y2 * z);
-    Y[7] = b * x * z * (x2 - R(3) * y2); gx[7] = b * (R(3) * x2 * z - R(3) * y2 * z); gy[7] = b * R(-6) * x * y * z;
-    gz[7] = b * (x2 * x - R(3) * x * y2);
-    Y[8] = g * (x2 * x2 - R(6) * x2 * y2 + y2 * y2); gx[8] = g * (R(4) * x2 * x - R(12) * x * y2);
-    gy[8] = g * (R(-12) * x2 * y + R(4) * y2 * y); gz[8] = R(0);
-  }
 }
 
 template <typename R>
@@ -247,46 +179,184 @@ __device__ inline void add_force(float4* facc32, double* facc64, unsigned long l
   }
 }
 
-// Block l of the force contraction for one neighbour: with S_m = sum_k u_k,lm g_k and
-// S'_m = sum_k u_k,lm g'_k, accumulates pr += sum_m S'_m Z_m and the tangential part
-// sum_m S_m (grad Z_m - l Z_m u) as (ptx, pty, ptz) += sum_m S_m grad Z_m and
-// pz_l += l sum_m S_m Z_m (the caller subtracts pz_l u once).
-template <typename R, int L>
-__device__ inline void force_block(const R* __restrict__ U, R ux, R uy, R uz, const R g[8], const R dg[8], R& pr,
-                                   R& ptx, R& pty, R& ptz, R& pzl) {
-  R Y[2 * L + 1], gx[2 * L + 1], gy[2 * L + 1], gz[2 * L + 1];
-  sh_block<R, L>(ux, uy, uz, Y, gx, gy, gz);
-  R q = R(0);
+// Real harmonics in the factored form Y_lm = N_lm Pi_lm(z) {A_m | B_m}(x, y) of a unit vector:
+// A_m + i B_m = (x + i y)^m (A for m >= 0, B for m < 0) and Pi_lm the monic polynomial
+// proportional to d^m P_l/dz^m.  kNorm[l^2 + l + m] = N_lm = sqrt((2l + 1)/(4 pi) (l - m)!/(l + m)!)
+// (sqrt 2 if m > 0) (2l)!/(2^l l! (l - m)!).  The adjoint keeps its u rows in the order of
+// evaluation, by m, cosine before sine, l ascending: kSlot[l^2 + l + m].
+__constant__ double kNorm[25] = {
+    0.28209479177387814, 0.48860251190291998, 0.48860251190291992, 0.48860251190291998, 0.54627421529603959,
+    1.0925484305920792,  0.94617469575756008, 1.0925484305920792,  0.54627421529603959, 0.59004358992664363,
+    1.4453057213202771,  2.2852289973223292,  1.865881662950577,   2.2852289973223292,  1.4453057213202771,
+    0.59004358992664363, 0.62583573544917637, 1.7701307697799304,  3.3116114351514598,  4.6833258049010249,
+    3.7024941420321507,  4.6833258049010249,  3.3116114351514598,  1.7701307697799304,  0.62583573544917637};
+__constant__ unsigned char kSlot[25] = {0,  9,  1,  5,  16, 10, 2,  6,  13, 21, 17, 11, 3,
+                                        7,  14, 19, 24, 22, 18, 12, 4,  8,  15, 20, 23};
+
+// Force of one pair, p = dE_i/dr_ij, from the atom's coefficients U[slot][k] = N_lm u_klm:
+//   E = f_cut(r) sum_lm P_lm(c) Pi_lm {A_m | B_m},  P_lm = sum_k U_k T_k(c),  Q_lm = dP_lm/dc.
+// The sums over l are taken first, per m and for cosine and sine: C = sum_l P Pi, Cq = sum_l Q Pi,
+// D = sum_l P dPi/dz.  Then V = sum C A, Vq = sum Cq A, and the gradient t of the (not
+// homogeneous) extension needs x and y parts once per m instead of once per (l, m), with
+// d(A_m + i B_m) = m (A_{m-1} + i B_{m-1}) d(x + i y).  Only its tangential part t - (t.u) u
+// counts:  p = (f_cut' V + 2 f_cut/rc Vq) u + f_cut/r (t - (t.u) u).
+// About 490 FP operations a pair; contracting g and g' with u and adding Y and grad Y per
+// (l, m) took about 800.  These operations are what the kernel is bound by, in FP32 (issue)
+// and above all in FP64 (one warp instruction per 16 cycles and SM).  Kernel times before and
+// after, with the lane rule below: FP64 2.63 -> 1.47 ms (12,700 atoms), FP32 1.28 -> 0.89 ms
+// (255,840 atoms).
+template <typename R>
+__device__ inline void pair_force(const R* __restrict__ U, R x, R y, R z, R r, R ir, R inv_rc, int mode, R& px, R& py,
+                                  R& pz) {
+  const R rr = r * inv_rc;
+  const R c = fma(R(2), rr, R(-1)), c2 = c + c;
+  R T[8], D[8];   // T_k and dT_k/dc
+  T[1] = c;
+  T[2] = fma(c2, c, R(-1));
+  D[2] = c2 + c2;
+  D[1] = R(1);
 #pragma unroll
-  for (int m = 0; m < 2 * L + 1; ++m) {
-    const int lm = L * L + m;
-    auto ua = ld4<R>(&U[lm * 8]);
-    auto ub = ld4<R>(&U[lm * 8 + 4]);
-    R S = ua.x * g[0];
-    S = fma(ua.y, g[1], S);
-    S = fma(ua.z, g[2], S);
-    S = fma(ua.w, g[3], S);
-    S = fma(ub.x, g[4], S);
-    S = fma(ub.y, g[5], S);
-    S = fma(ub.z, g[6], S);
-    S = fma(ub.w, g[7], S);
-    R Sp = ua.x * dg[0];
-    Sp = fma(ua.y, dg[1], Sp);
-    Sp = fma(ua.z, dg[2], Sp);
-    Sp = fma(ua.w, dg[3], Sp);
-    Sp = fma(ub.x, dg[4], Sp);
-    Sp = fma(ub.y, dg[5], Sp);
-    Sp = fma(ub.z, dg[6], Sp);
-    Sp = fma(ub.w, dg[7], Sp);
-    pr = fma(Sp, Y[m], pr);
-    if (L > 0) {
-      q = fma(S, Y[m], q);
-      ptx = fma(S, gx[m], ptx);
-      pty = fma(S, gy[m], pty);
-      ptz = fma(S, gz[m], ptz);
-    }
+  for (int k = 3; k < 8; ++k) {
+    T[k] = fma(c2, T[k - 1], -T[k - 2]);
+    D[k] = fma(c2, D[k - 1], fma(R(2), T[k - 1], -D[k - 2]));
   }
-  if (L > 0) pzl = fma(R(L), q, pzl);
+  auto pq = [&](int slot, R& P, R& Q) {
+    const auto ua = ld4<R>(U + slot * 8);
+    const auto ub = ld4<R>(U + slot * 8 + 4);
+    P = fma(ua.y, T[1], ua.x);
+    P = fma(ua.z, T[2], P);
+    P = fma(ua.w, T[3], P);
+    P = fma(ub.x, T[4], P);
+    P = fma(ub.y, T[5], P);
+    P = fma(ub.z, T[6], P);
+    P = fma(ub.w, T[7], P);
+    Q = fma(ua.z, D[2], ua.y);
+    Q = fma(ua.w, D[3], Q);
+    Q = fma(ub.x, D[4], Q);
+    Q = fma(ub.y, D[5], Q);
+    Q = fma(ub.z, D[6], Q);
+    Q = fma(ub.w, D[7], Q);
+  };
+  const R w = z * z, z2 = z + z;
+  R V, Vq, tx, ty, tz, P, Q;
+  {   // m = 0
+    const R q2 = w - R(1.0 / 3.0), q3 = z * (w - R(0.6)), q4 = fma(w, w - R(6.0 / 7.0), R(3.0 / 35.0));
+    pq(0, V, Vq);
+    pq(1, P, Q);
+    V = fma(P, z, V);
+    Vq = fma(Q, z, Vq);
+    tz = P;
+    pq(2, P, Q);
+    V = fma(P, q2, V);
+    Vq = fma(Q, q2, Vq);
+    tz = fma(P, z2, tz);
+    pq(3, P, Q);
+    V = fma(P, q3, V);
+    Vq = fma(Q, q3, Vq);
+    tz = fma(P, fma(R(3), w, R(-0.6)), tz);
+    pq(4, P, Q);
+    V = fma(P, q4, V);
+    Vq = fma(Q, q4, Vq);
+    tz = fma(P, z * fma(R(4), w, R(-12.0 / 7.0)), tz);
+  }
+  R C, Cq, E;   // per m and parity: sum_l P Pi, sum_l Q Pi, sum_l P dPi/dz
+  {             // m = 1
+    const R p3 = w - R(0.2), p4 = z * (w - R(3.0 / 7.0)), d4 = fma(R(3), w, R(-3.0 / 7.0));
+    auto sum1 = [&](int s) {
+      pq(s, C, Cq);
+      pq(s + 1, P, Q);
+      C = fma(P, z, C);
+      Cq = fma(Q, z, Cq);
+      E = P;
+      pq(s + 2, P, Q);
+      C = fma(P, p3, C);
+      Cq = fma(Q, p3, Cq);
+      E = fma(P, z2, E);
+      pq(s + 3, P, Q);
+      C = fma(P, p4, C);
+      Cq = fma(Q, p4, Cq);
+      E = fma(P, d4, E);
+    };
+    sum1(5);
+    V = fma(C, x, V);
+    Vq = fma(Cq, x, Vq);
+    tx = C;
+    tz = fma(E, x, tz);
+    sum1(9);
+    V = fma(C, y, V);
+    Vq = fma(Cq, y, Vq);
+    ty = C;
+    tz = fma(E, y, tz);
+  }
+  // A_m, B_m and the next lower ones times m (the x and y derivatives)
+  auto cosine = [&](R A, R mA, R mB) {
+    V = fma(C, A, V);
+    Vq = fma(Cq, A, Vq);
+    tx = fma(C, mA, tx);
+    ty = fma(-C, mB, ty);
+  };
+  auto sine = [&](R B, R mA, R mB) {
+    V = fma(C, B, V);
+    Vq = fma(Cq, B, Vq);
+    tx = fma(C, mB, tx);
+    ty = fma(C, mA, ty);
+  };
+  const R A2 = fma(x, x, -y * y), B2 = R(2) * x * y;
+  {   // m = 2
+    const R p4 = w - R(1.0 / 7.0);
+    auto sum2 = [&](int s) {
+      pq(s, C, Cq);
+      pq(s + 1, P, Q);
+      C = fma(P, z, C);
+      Cq = fma(Q, z, Cq);
+      E = P;
+      pq(s + 2, P, Q);
+      C = fma(P, p4, C);
+      Cq = fma(Q, p4, Cq);
+      E = fma(P, z2, E);
+    };
+    const R mA = x + x, mB = y + y;
+    sum2(13);
+    cosine(A2, mA, mB);
+    tz = fma(E, A2, tz);
+    sum2(16);
+    sine(B2, mA, mB);
+    tz = fma(E, B2, tz);
+  }
+  const R A3 = fma(x, A2, -y * B2), B3 = fma(x, B2, y * A2);
+  {   // m = 3
+    const R mA = R(3) * A2, mB = R(3) * B2;
+    pq(19, C, Cq);
+    pq(20, P, Q);
+    C = fma(P, z, C);
+    Cq = fma(Q, z, Cq);
+    cosine(A3, mA, mB);
+    tz = fma(P, A3, tz);
+    pq(21, C, Cq);
+    pq(22, P, Q);
+    C = fma(P, z, C);
+    Cq = fma(Q, z, Cq);
+    sine(B3, mA, mB);
+    tz = fma(P, B3, tz);
+  }
+  {   // m = 4
+    const R mA = R(4) * A3, mB = R(4) * B3;
+    pq(23, C, Cq);
+    cosine(fma(x, A3, -y * B3), mA, mB);
+    pq(24, C, Cq);
+    sine(fma(x, B3, y * A3), mA, mB);
+  }
+  const R t = mode == 1 ? c : rr;   // the f_cut argument (mode 1: 2 r/rc - 1)
+  const R t2 = t * t;
+  R fc = R(1) - R(1.875) * t + R(1.25) * t2 * t - R(0.375) * t2 * t2 * t;
+  if (mode == 1) fc *= R(0.5);
+  const R dfc = (R(-1.875) + R(3.75) * t2 - R(1.875) * t2 * t2) * inv_rc;
+  const R ft = fc * ir;
+  const R tu = fma(tx, x, fma(ty, y, tz * z));
+  const R a = fma(dfc, V, fma(R(2) * fc * inv_rc, Vq, -ft * tu));
+  px = fma(a, x, ft * tx);
+  py = fma(a, y, ft * ty);
+  pz = fma(a, z, ft * tz);
 }
 
 template <typename T>
@@ -294,6 +364,20 @@ __device__ inline T warp_sum(T v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
+}
+
+template <typename T, int L>
+__device__ inline T lane_sum(T v) {   // over groups of L lanes
+#pragma unroll
+  for (int o = L / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// The warp's next work item: items below `first` were dealt out statically.
+__device__ inline int next_item(int* counter, int step, int first) {
+  int q = 0;
+  if ((threadIdx.x & 31) == 0) q = atomicAdd(counter, step);
+  return first + __shfl_sync(0xffffffffu, q, 0);
 }
 
 // ---- 3xTF32 on warp-level tensor cores (FP32 path).  An FP32 value x is carried as
@@ -475,11 +559,8 @@ __global__ void __launch_bounds__(kWarps<R> * 32, sizeof(R) == 4 ? AP_ACE_MINB :
   const int kq = lane & 7, grp = lane >> 3;
   const unsigned lt_mask = (1u << lane) - 1u;
   unsigned long long cnt_pairs = 0, cnt_atoms = 0, cnt_mma = 0;   // profiling counts of this warp
-  while (true) {
-    int q = 0;
-    if (lane == 0) q = atomicAdd(a.counter, 1);
-    q = __shfl_sync(0xffffffffu, q, 0);
-    if (q >= m) break;
+  const int q_first = warp * gridDim.x + blockIdx.x, q_all = kWarps<R> * gridDim.x;
+  for (int q = q_first; q < m; q = next_item(a.counter, 1, q_all)) {
     const int i = a.queue[q];
     const SysInfo& S = a.sys[a.atom_sys ? a.atom_sys[i] : 0];
     const auto si = a.sh[i];
@@ -546,7 +627,7 @@ __global__ void __launch_bounds__(kWarps<R> * 32, sizeof(R) == 4 ? AP_ACE_MINB :
           const auto en = slot < kListCap ? ld4<R>(&list[4 * slot]) : a.list4[(size_t)q * a.rec + slot];
           float r2 = en.x * en.x + en.y * en.y + en.z * en.z;
           float ir = rsqrt_(r2);
-          radial<float, false>(r2 * ir, a.inv_rc, a.mode, g, nullptr);
+          radial<float>(r2 * ir, a.inv_rc, a.mode, g);
           sh_values<float>(en.x * ir, en.y * ir, en.z * ir, Y);
         } else {
 #pragma unroll
@@ -647,7 +728,7 @@ __global__ void __launch_bounds__(kWarps<R> * 32, sizeof(R) == 4 ? AP_ACE_MINB :
           const auto en = slot < kListCap ? ld4<R>(&list[4 * slot]) : a.list4[(size_t)q * a.rec + slot];
           R r2 = en.x * en.x + en.y * en.y + en.z * en.z;
           R ir = rsqrt_(r2);
-          radial<R, false>(r2 * ir, a.inv_rc, a.mode, g, nullptr);
+          radial<R>(r2 * ir, a.inv_rc, a.mode, g);
           sh_values<R>(en.x * ir, en.y * ir, en.z * ir, Y);
         } else {
 #pragma unroll
@@ -832,85 +913,91 @@ __global__ void AP_NU3_BOUNDS k_ace_nu3(AceArgs<R> a, const Nu3Coef<R> P,
   }
 }
 
-// Kernel 3, one warp per precise atom (persistent): E_i = E12 + E3 -> e_prec, then
-// u_klm = (1/N0) sum_n W[l][n][k] dE/dA_nlm and the forces: lanes recompute g, g',
-// Y, grad Y per in-range neighbour (from the kept row positions), contract with u
-// and scatter -w_i p_ij to neighbour j, +w_i sum_j p_ij to i.
-template <typename R, bool FORCES, bool FS>
+// Energies alone: E_i = E12 + E3 (+ F), one thread per precise atom.
+template <typename R, bool FS>
+__global__ void k_ace_energy(AceArgs<R> a) {
+  const int m = *a.count;
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < m; q += gridDim.x * blockDim.x)
+    a.e_prec[a.queue[q]] = a.e12[q] + a.e3[q] + (FS ? a.fs[2 * (size_t)q] : 0.0);
+}
+
+// Kernel 3, L lanes per precise atom: E_i = E12 + E3 -> e_prec, then
+// u_klm = (1/N0) sum_n W[l][n][k] dE/dA_nlm (times N_lm, in the order of pair_force), and the
+// pair forces: each lane takes every L-th record of its atom, scatters -w_i p_ij to neighbour
+// j, and +w_i sum_j p_ij goes to i.  Persistent warps: every warp starts at its own position
+// (block-major, so short queues spread over all SMs) and continues by an atomic work counter.
+// L = 8 fills 98 % of the lanes with the about 134 neighbours of a bulk atom, L = 32 84 % of
+// 5 turns, but short queues need the warps (adjoint_lanes has the figures).
+template <typename R, bool FS, int L>
 __global__ void __launch_bounds__(kWarps3<R> * 32, sizeof(R) == 4 ? AP_ACE3_MINB : 1) k_ace_adjoint(AceArgs<R> a) {
-  // Shared memory: W [320] | per warp: dA [200] | U [200]
+  constexpr int NA = 32 / L;   // atoms per warp
+  // Shared memory: W [320] | per warp: dA [NA][200] | U [NA][200]
   extern __shared__ __align__(128) unsigned char smem_raw[];
   R* Ws = reinterpret_cast<R*>(smem_raw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  R* dA = Ws + 320 + warp * 400;
-  R* U = dA + 200;
+  R* dA = Ws + 320 + warp * (400 * NA);
+  R* U = dA + 200 * NA;
   for (int t = threadIdx.x; t < 320; t += blockDim.x) Ws[t] = a.W[t];
   __syncthreads();
   const int m = *a.count;
-  while (true) {
-    int q = 0;
-    if (lane == 0) q = atomicAdd(a.counter2, 1);
-    q = __shfl_sync(0xffffffffu, q, 0);
-    if (q >= m) break;
-    const int i = a.queue[q];
-    if (lane == 0) a.e_prec[i] = a.e12[q] + a.e3[q] + (FS ? a.fs[2 * (size_t)q] : 0.0);
-    if (!FORCES) continue;
-    if (FS) {
-      const R fp = (R)a.fs[2 * (size_t)q + 1];
-      for (int o = lane; o < 200; o += 32) dA[o] = fma(fp, a.dAb[(size_t)q * 200 + o], a.dA[(size_t)q * 200 + o]);
-    } else {
-      for (int o = lane; o < 200; o += 32) dA[o] = a.dA[(size_t)q * 200 + o];
+  const int g = lane / L, sub = lane & (L - 1);
+  const int q_first = NA * (warp * gridDim.x + blockIdx.x), q_all = NA * kWarps3<R> * gridDim.x;
+  for (int q0 = q_first; q0 < m; q0 = next_item(a.counter2, NA, q_all)) {
+    const int q = q0 + g;
+    const bool on = q < m;
+    const int i = on ? a.queue[q] : 0;
+    if (on && sub == 0) a.e_prec[i] = a.e12[q] + a.e3[q] + (FS ? a.fs[2 * (size_t)q] : 0.0);
+    const int na = min(NA, m - q0);
+    for (int t = 0; t < na; ++t) {
+      const size_t qt = (size_t)(q0 + t);
+      R* dst = dA + 200 * t;
+      const R fp = FS ? (R)a.fs[2 * qt + 1] : R(0);
+      for (int o = lane; o < 200; o += 32) {
+        const int n = o / 25, lm = o - 25 * n;
+        R v = a.dA[qt * 200 + o];
+        if (FS) v = fma(fp, a.dAb[qt * 200 + o], v);
+        if (n < 3 && lm < 16) v += a.de3[qt * 48 + n * 16 + lm];
+        dst[o] = v;
+      }
     }
-    __syncwarp();
-    for (int v = lane; v < 48; v += 32) dA[(v >> 4) * 25 + (v & 15)] += a.de3[(size_t)q * 48 + v];
     __syncwarp();
     for (int o = lane; o < 200; o += 32) {
       const int lm = o >> 3, k = o & 7, l = l_of(lm);
-      R s = R(0);
+      const R nrm = (R)kNorm[lm] * a.inv_n0;
+      R* dst = U + kSlot[lm] * 8 + k;
+      for (int t = 0; t < na; ++t) {
+        R s = R(0);
 #pragma unroll
-      for (int n = 0; n < 8; ++n) s += Ws[(l * 8 + n) * 8 + k] * dA[n * 25 + lm];
-      U[o] = s * a.inv_n0;
+        for (int n = 0; n < 8; ++n) s = fma(Ws[(l * 8 + n) * 8 + k], dA[200 * t + n * 25 + lm], s);
+        dst[200 * t] = s * nrm;
+      }
     }
     __syncwarp();
-    const int nin = a.nin[q];
-    const R wgt = (R)(a.wgt ? a.wgt[i] : 1.0 - (a.lam ? a.lam[i] : 0.0));
+    const int nin = on ? a.nin[q] : 0;
+    const R wgt = on ? (R)(a.wgt ? a.wgt[i] : 1.0 - (a.lam ? a.lam[i] : 0.0)) : R(0);
     R pix = R(0), piy = R(0), piz = R(0);
-    // the pair records kernel 1 kept (displacement and j, coalesced), the lane's next
-    // one loaded an iteration ahead
+    // the pair records kernel 1 kept (displacement and j), the lane's next one loaded a turn ahead
     const typename V<R>::R4* lst = a.list4 + (size_t)q * a.rec;
     typename V<R>::R4 e_n = make_r4(R(0), R(0), R(0), R(0));
-    if (lane < nin) e_n = lst[lane];
-    for (int base = 0; base < nin; base += 32) {
-      const int slot = base + lane;
+    if (sub < nin) e_n = lst[sub];
+    for (int slot = sub; slot < nin; slot += L) {
       const auto e = e_n;
-      if (slot + 32 < nin) e_n = lst[slot + 32];
-      if (slot >= nin) continue;
+      if (slot + L < nin) e_n = lst[slot + L];
       const int j = unpack_j(e.w);
-      const R d[3] = {e.x, e.y, e.z};
-      R r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-      R ir = rsqrt_(r2);
-      R ux = d[0] * ir, uy = d[1] * ir, uz = d[2] * ir;
-      R g[8], dg[8];
-      radial<R, true>(r2 * ir, a.inv_rc, a.mode, g, dg);
-      R pr = R(0), ptx = R(0), pty = R(0), ptz = R(0), pzl = R(0);
-      force_block<R, 0>(U, ux, uy, uz, g, dg, pr, ptx, pty, ptz, pzl);
-      force_block<R, 1>(U, ux, uy, uz, g, dg, pr, ptx, pty, ptz, pzl);
-      force_block<R, 2>(U, ux, uy, uz, g, dg, pr, ptx, pty, ptz, pzl);
-      force_block<R, 3>(U, ux, uy, uz, g, dg, pr, ptx, pty, ptz, pzl);
-      force_block<R, 4>(U, ux, uy, uz, g, dg, pr, ptx, pty, ptz, pzl);
-      ptx = fma(-pzl, ux, ptx);
-      pty = fma(-pzl, uy, pty);
-      ptz = fma(-pzl, uz, ptz);
-      R px = pr * ux + ptx * ir, py = pr * uy + pty * ir, pz = pr * uz + ptz * ir;
+      const R r2 = e.x * e.x + e.y * e.y + e.z * e.z;
+      const R ir = rsqrt_(r2);
+      R px, py, pz;
+      pair_force<R>(U + 200 * g, e.x * ir, e.y * ir, e.z * ir, r2 * ir, ir, a.inv_rc, a.mode, px, py, pz);
       pix += px;
       piy += py;
       piz += pz;
       add_force<R>(a.facc32, a.facc64, a.faccfix, j, -wgt * px, -wgt * py, -wgt * pz);
     }
-    pix = warp_sum<R>(pix);
-    piy = warp_sum<R>(piy);
-    piz = warp_sum<R>(piz);
-    if (lane == 0) add_force<R>(a.facc32, a.facc64, a.faccfix, i, wgt * pix, wgt * piy, wgt * piz);
+    __syncwarp();
+    pix = lane_sum<R, L>(pix);
+    piy = lane_sum<R, L>(piy);
+    piz = lane_sum<R, L>(piz);
+    if (on && sub == 0) add_force<R>(a.facc32, a.facc64, a.faccfix, i, wgt * pix, wgt * piy, wgt * piz);
     __syncwarp();
   }
 }
@@ -944,8 +1031,25 @@ size_t basis_smem() {
 }
 
 template <typename R>
-size_t adjoint_smem() {
-  return sizeof(R) * (320 + kWarps3<R> * 400);
+size_t adjoint_smem(int lanes) {
+  return sizeof(R) * (320 + kWarps3<R> * 400 * (32 / lanes));
+}
+
+// Grid of a persistent kernel over `items` (one warp each) with up to `resident` blocks per SM:
+// a whole number of blocks per SM, no more than the items need.
+inline int persistent_grid(int num_sms, int resident, int warps, int64_t items) {
+  const int64_t per_sm = (items + (int64_t)num_sms * warps - 1) / ((int64_t)num_sms * warps);
+  return num_sms * (int)std::max<int64_t>(1, std::min<int64_t>(resident, per_sm));
+}
+
+// Lanes per atom of the adjoint for a queue of m atoms: 8 where that still fills every SM
+// (FP32: all 24 resident warps twice; FP64: 4 warps per scheduler), a whole warp otherwise.
+// Whole force evaluations, 8 against 32 lanes: FP32 3.62 / 3.77 ms (255,840 atoms), 57.8 / 60.0 ms
+// (10 steps with 240,000), 3.17 / 3.09 ms (10 steps with 12,700); FP64 4.60 / 4.75 ms (12,700
+// atoms), 2.29 / 2.19 ms (energy and gradient, 1,365).
+template <typename R>
+inline int adjoint_lanes(int num_sms, int64_t m) {
+  return m >= (int64_t)num_sms * (sizeof(R) == 4 ? 192 : 64) ? 8 : 32;
 }
 
 template <typename K>
@@ -1015,12 +1119,18 @@ void run_ace(ap_ctx* c, const double* d_lam, const double* d_wgt, const int* d_q
   const bool fs = c->cfg.ace_fs_on != 0;
 
   const int pi = sizeof(R) == 4 ? 0 : 1;
+  // the queue's length as of the last synchronisation (its rows were built after it): sizes the
+  // grids only, the kernels read the device's own count
+  int m = 0;
+  std::memcpy(&m, (const char*)c->h_sc + ((const char*)a.count - (const char*)c->d_sc), sizeof(int));
+  const int lanes = adjoint_lanes<R>(c->num_sms, m);
   static int b1[2] = {0, 0}, b3[2][2][2] = {};
-  const size_t s1 = basis_smem<R>(), s3 = adjoint_smem<R>();
+  const size_t s1 = basis_smem<R>(), s3 = adjoint_smem<R>(lanes);
   if (!b1[pi]) b1[pi] = resident_blocks(k_ace_basis<R>, kWarps<R> * 32, s1);
-  auto k3 = forces ? (fs ? k_ace_adjoint<R, true, true> : k_ace_adjoint<R, true, false>)
-                   : (fs ? k_ace_adjoint<R, false, true> : k_ace_adjoint<R, false, false>);
-  if (!b3[pi][forces][fs]) b3[pi][forces][fs] = resident_blocks(k3, kWarps3<R> * 32, s3);
+  auto k3 = lanes == 8 ? (fs ? k_ace_adjoint<R, true, 8> : k_ace_adjoint<R, false, 8>)
+                       : (fs ? k_ace_adjoint<R, true, 32> : k_ace_adjoint<R, false, 32>);
+  int& r3 = b3[pi][lanes == 8][fs];
+  if (forces && !r3) r3 = resident_blocks(k3, kWarps3<R> * 32, s3);
   if (forces) {
     if (a.faccfix)
       cudaMemsetAsync(c->d_faccfix, 0, sizeof(unsigned long long) * 3 * (size_t)c->n, s);
@@ -1031,17 +1141,22 @@ void run_ace(ap_ctx* c, const double* d_lam, const double* d_wgt, const int* d_q
   }
   cudaMemsetAsync(a.counter, 0, 2 * sizeof(int), s);   // work_counter and work_counter2
   const int tb = prof_mark(c, s);
-  k_ace_basis<R><<<c->num_sms * b1[pi], kWarps<R> * 32, s1, s>>>(a);
+  k_ace_basis<R><<<persistent_grid(c->num_sms, b1[pi], kWarps<R>, m), kWarps<R> * 32, s1, s>>>(a);
   prof_add(c, AP_PHASE_ACE_BASIS, tb, prof_mark(c, s));
   const int t2 = sizeof(R) == 4 ? 128 : 64;
   if (fs)
     k_ace_nu3<R, true><<<c->num_sms * (sizeof(R) == 4 ? 8 : 16), t2, 0, s>>>(a, P, Q);
   else
     k_ace_nu3<R, false><<<c->num_sms * (sizeof(R) == 4 ? 8 : 16), t2, 0, s>>>(a, P, Q);
-  const int t0 = prof_mark(c, s);
-  k3<<<c->num_sms * b3[pi][forces][fs], kWarps3<R> * 32, s3, s>>>(a);
-  prof_add(c, AP_PHASE_ACE_ADJOINT, t0, prof_mark(c, s));
   c->kernels += 3;
+  if (!forces) {
+    auto ke = fs ? k_ace_energy<R, true> : k_ace_energy<R, false>;
+    ke<<<std::max(1, std::min(c->num_sms * 8, (m + 127) / 128)), 128, 0, s>>>(a);
+    return;
+  }
+  const int t0 = prof_mark(c, s);
+  k3<<<persistent_grid(c->num_sms, r3, kWarps3<R>, ((int64_t)m * lanes + 31) / 32), kWarps3<R> * 32, s3, s>>>(a);
+  prof_add(c, AP_PHASE_ACE_ADJOINT, t0, prof_mark(c, s));
 }
 
 }  // namespace
