@@ -120,6 +120,16 @@ ap_status set_systems(ap_ctx* c, int n_sys, const int64_t* offsets, const ap_box
       for (int k = 0; k < I.nc[d]; ++k) org.push_back(std::fma((double)k, I.h[d], I.lo[d]));
     }
   }
+  // Groups of 2^3 cells per block of the EAM row build (8 warps and about 44 atoms each) where
+  // these are at least two blocks per SM, else a block per cell, its warps sharing the atoms
+  const int group = base >= 16 * c->num_sms ? 2 : 1;
+  int n_groups = 0;
+  for (SysInfo& I : sys) {
+    I.grp_base = n_groups;
+    int g = 1;
+    for (int d = 0; d < 3; ++d) g *= (I.nc[d] + group - 1) / group;
+    n_groups += g;
+  }
   bool same = (n_sys == c->n_sys) && c->h_offsets.size() == (size_t)n_sys + 1 &&
               std::equal(offsets, offsets + n_sys + 1, c->h_offsets.begin()) &&
               std::memcmp(sys.data(), c->h_sys.data(), sizeof(SysInfo) * n_sys) == 0;
@@ -128,6 +138,8 @@ ap_status set_systems(ap_ctx* c, int n_sys, const int64_t* offsets, const ap_box
   c->h_offsets.assign(offsets, offsets + n_sys + 1);
   c->n_sys = n_sys;
   c->n_cells = base;
+  c->build_group = group;
+  c->n_groups = n_groups;
   c->stored_off = stored;
   for (int d = 0; d < 3; ++d) {
     c->sten_spread[d] = spread[d];

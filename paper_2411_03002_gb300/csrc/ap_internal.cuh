@@ -22,6 +22,7 @@ struct SysInfo {
   int nc[3];         // cells per dimension (<= 1023)
   int periodic[3];
   int cell_base;     // first global cell id of this system
+  int grp_base;      // first cell group of this system (blocks of the EAM row build)
   int org[3];        // offsets of this system's cell origins lo + c h in the origin table, per dimension
 };
 
@@ -181,6 +182,7 @@ struct ap_ctx {
   ap::SysInfo* d_sys = nullptr;
   int* d_atom_sys = nullptr;     // null when n_sys == 1
   int n_cells = 0;
+  int build_group = 1, n_groups = 0;   // EAM row build: cells per edge of a block's group, groups in all
   bool stored_off = false;
   bool lim_valid = false;        // d_lim_eam holds the prefixes of an EAM pass on the current rows
   float split_rpf2 = 0.f;        // r_c^2 (FP32) at which the EAM rows were split

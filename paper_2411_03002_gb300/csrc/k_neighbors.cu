@@ -295,131 +295,383 @@ __device__ inline int build_row_warp(int i, const double* __restrict__ x, const 
   return cnt;
 }
 
-#ifndef AP_BUILD_MINB
-#define AP_BUILD_MINB 9   // resident 128-thread blocks per SM the EAM row build is compiled for (<= 56 registers)
-#endif
-// Unroll depth of the per-cell candidate loop of the EAM row build (compile-time tuning).
-#ifndef AP_BUILD_UNROLL
-#define AP_BUILD_UNROLL 2
-#endif
-constexpr int kBuildUnroll = AP_BUILD_UNROLL;
+// ---- EAM rows, one block per group of cells (2 x 2 x 2, or a single one in small systems).
+//   * The block stages the candidates of the whole group once, in shared memory: the stencil is
+//     walked as pencils of cells along x, contiguous in cell order and cut to the reach of the
+//     group's box; of their atoms those within reach of the box are kept, in stencil order.
+//   * Each warp takes one cell of the group (or a share of the single cell's atoms) and lists the
+//     staged candidates within reach of the box around its atoms (about 250 of the 560 in a
+//     cell's 5^3 stencil in FCC copper, of which each atom takes 85 to 110).
+//   * Each lane tests a block of consecutive listed candidates against the warp's atoms, three
+//     at a time, and keeps a bit per candidate and atom; a scan over the lanes' counts gives
+//     every accepted candidate its place in the row.
+// A thread per row walked all 560 candidates in one dependent chain and wrote 32 rows at once,
+// 4 bytes each: 999,180 atoms at 6.5 A 1.48 -> 1.30 ms, 32,000 atoms 206 -> 75 us, 237 atoms
+// 160 -> 25 us (the dependent chain was the cost there).  What binds it now is instruction
+// issue: the tests (about 35 % of the instructions) and the writes of the accepted entries.
+//
+// Row order: first the entries whose FP32 distance lies inside the potential cutoff
+// (rpf2 = r_c^2), in stencil order, then the skin entries, last of the stencil first; nin
+// receives the length of the first part.  The EAM density pass records, per atom, where the
+// in-range entries end at the current positions (it re-tests every entry), so the force pass
+// walks only that prefix; the split at build time only makes the prefix short.  The CSP on
+// rows built at its own positions may stop after the first part.
+constexpr int kBuildWarps = 8;     // warps per block
+constexpr int kStage = 1024;       // staged candidates per block; a fuller stage is used up in rounds
+constexpr int kList = 416;         // listed candidates per warp (13 per lane), used up in turns likewise
+constexpr int kCentres = 3;        // atoms tested together against a listed candidate
 
-// One thread builds one row (EAM rows of all atoms): scan the 5x5x5 stencil around atom i and keep the
-// accepted (j, offset).  The row is ordered in two parts: first the entries whose FP32 distance
-// lies inside the potential cutoff (rpf2 = r_c^2), in stencil order, then the skin entries;
-// n_in_out receives the length of the first part.  The EAM density pass records, per atom,
-// where the in-range entries end at the current positions (it re-tests every entry), so the
-// force pass walks only that prefix; the split at build time only makes the prefix short.
-// The CSP on rows built at its own positions may stop after the first part.  Candidates are
-// read from s32c, the shadows in cell order; t_self is atom i's own position in that order.
-__device__ inline int build_row(int i, int t_self, const double* __restrict__ x, const SysInfo& S,
-                                const float4* __restrict__ s32, const float4* __restrict__ s32c,
-                                const int4* __restrict__ cunw, const int* __restrict__ cstart,
-                                const int* __restrict__ catoms, float rcf2, double rc2, float rpf2, float band,
-                                int cap, int* __restrict__ row, int* __restrict__ offrow, int& n_in_out) {
-  const float4 si = s32[i];
-  const int4 ci = cunw[i];
-  const int cw[3] = {cell_x(ci.w), cell_y(ci.w), cell_z(ci.w)};
-  const float sv[3] = {si.x, si.y, si.z};
-  const float rmax2 = rcf2 + band;
-  int n_in = 0, n_skin = 0;   // in-range entries fill the row from the front, skin entries from the back
-  for (int dz = -kStencil; dz <= kStencil; ++dz) {
-    int tz = cw[2] + dz, iz = 0;
-    if (S.periodic[2]) {
-      iz = floor_div(tz, S.nc[2]);
-      tz -= iz * S.nc[2];
-    } else if (tz < 0 || tz >= S.nc[2]) {
-      continue;
+struct BuildArgs {
+  const double* x;
+  const SysInfo* sys;
+  int n_sys, group;         // cells per edge of a block's group: 2 or 1
+  const float4* s32c;       // shadows in cell order
+  const int4* cunw;
+  const int* cstart;
+  const int* catoms;
+  float rcf2;
+  double rc2;
+  float rpf2, band;
+  int cap;
+  int* nbr;
+  int* off;
+  int* cnt;
+  int* nin;
+  DevScalars* sc;
+};
+
+// The exact decision for a candidate in the guard band around the cutoff, at cell offset o
+// (pack_off) of atom i if `stored`, else at the one that follows from the two atoms' cells.
+// Out of line: hardly any pair comes here.
+__device__ __noinline__ bool decide(const BuildArgs& A, const SysInfo& S, int i, int j, int o, bool stored) {
+  const int4 ci = A.cunw[i], cj = A.cunw[j];
+  const int cw[3] = {cell_x(ci.w), cell_y(ci.w), cell_z(ci.w)}, cv[3] = {cell_x(cj.w), cell_y(cj.w), cell_z(cj.w)};
+  const int ko[3] = {off_x(o), off_y(o), off_z(o)};
+  int img[3];
+  for (int d = 0; d < 3; ++d) {
+    const int k = stored ? ko[d] : wrap_off(cv[d] - cw[d], S.nc[d], S.periodic[d]);
+    img[d] = S.periodic[d] ? floor_div(cw[d] + k, S.nc[d]) : 0;
+  }
+  return exact_within(A.x, S, i, j, ci, cj, img, A.rc2);
+}
+
+__device__ inline float warp_min(float v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+__device__ inline float warp_max(float v) { return -warp_min(-v); }
+
+#ifndef AP_BUILD_MINB
+#define AP_BUILD_MINB 4   // resident blocks per SM the row build is compiled for (registers)
+#endif
+// STORED: the box is narrower than five cells in a periodic dimension and rows carry the cell
+// offsets; otherwise they follow from the two atoms' cells.
+template <bool STORED>
+__global__ void __launch_bounds__(kBuildWarps * 32, AP_BUILD_MINB)
+    k_build_eam(const __grid_constant__ BuildArgs A) {
+  constexpr int T = kBuildWarps * 32;
+  __shared__ float4 s_pos[kStage];                      // position relative to the group's first cell, atom index
+  __shared__ int s_cell[STORED ? kStage : 1];           // cell relative to the group's first cell (pack_off)
+  __shared__ unsigned short s_list[kBuildWarps][kList];
+  __shared__ int s_beg[T], s_pre[T + 1], s_run[T];      // runs: first slot, candidates before, cell (pack_off) and image
+  __shared__ int s_sum[kBuildWarps + 1];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned lt = (1u << lane) - 1u;
+  // the block's system and group of cells
+  int sys = 0;
+  for (int lo = 0, hi = A.n_sys - 1; lo <= hi;) {
+    const int mid = (lo + hi) >> 1;
+    if (A.sys[mid].grp_base <= (int)blockIdx.x) {
+      sys = mid;
+      lo = mid + 1;
+    } else {
+      hi = mid - 1;
     }
-    float gz = fmaxf(0.f, fmaxf((float)dz * S.hf[2] - sv[2], sv[2] - (float)(dz + 1) * S.hf[2]));
-    for (int dy = -kStencil; dy <= kStencil; ++dy) {
-      int ty = cw[1] + dy, iy = 0;
-      if (S.periodic[1]) {
-        iy = floor_div(ty, S.nc[1]);
-        ty -= iy * S.nc[1];
-      } else if (ty < 0 || ty >= S.nc[1]) {
+  }
+  const SysInfo& S = A.sys[sys];
+  const int nx = S.nc[0], ny = S.nc[1], nz = S.nc[2];
+  const float hx = S.hf[0], hy = S.hf[1], hz = S.hf[2];
+  const int gx = (nx + A.group - 1) / A.group, gy = (ny + A.group - 1) / A.group;
+  const int gid = blockIdx.x - S.grp_base;
+  const int x0 = gid % gx * A.group, y0 = gid / gx % gy * A.group, z0 = gid / (gx * gy) * A.group;
+  const int mx = min(A.group, nx - x0), my = min(A.group, ny - y0), mz = min(A.group, nz - z0);
+  const float reach2 = A.rcf2 + A.band, r_sure = A.rcf2 - A.band;
+  // this warp's cell of the group, or its share of the single cell's atoms
+  const int parts = A.group == 1 ? kBuildWarps : 1, part = A.group == 1 ? warp : 0;
+  const int wx = warp & 1, wy = (warp >> 1) & 1, wz = warp >> 2;
+  int b = 0, own = 0, ux = 0, uy = 0, uz = 0;
+  if (A.group == 1 || (wx < mx && wy < my && wz < mz)) {
+    if (A.group != 1) {
+      ux = wx;
+      uy = wy;
+      uz = wz;
+    }
+    const int cell = S.cell_base + ((z0 + uz) * ny + y0 + uy) * nx + x0 + ux;
+    b = A.cstart[cell];
+    own = max(0, (A.cstart[cell + 1] - b - part + parts - 1) / parts);   // atoms part, part + parts, ...
+  }
+  // ---- the runs of the group's stencil: pencil (dy, dz), periodic image ix along x
+  const int py = my + 2 * kStencil, pz = mz + 2 * kStencil;
+  const int ix_lo = S.periodic[0] ? floor_div(x0 - kStencil, nx) : 0;
+  const int n_im = S.periodic[0] ? floor_div(x0 + mx - 1 + kStencil, nx) - ix_lo + 1 : 1;
+  const int n_runs = py * pz * n_im;   // <= 36 * 2, or 25 * 5 for a single cell
+  const float gxh = (float)mx * hx + 1e-3f, gyh = (float)my * hy + 1e-3f, gzh = (float)mz * hz + 1e-3f;
+  int len = 0;
+  if (threadIdx.x < n_runs) {
+    const int pen = threadIdx.x / n_im, ix = ix_lo + threadIdx.x - pen * n_im;
+    const int dz = pen / py - kStencil, dy = pen % py - kStencil;
+    int ty = y0 + dy, tz = z0 + dz;
+    bool valid = true;
+    if (S.periodic[1]) ty -= floor_div(ty, ny) * ny;
+    else valid = valid && ty >= 0 && ty < ny;
+    if (S.periodic[2]) tz -= floor_div(tz, nz) * nz;
+    else valid = valid && tz >= 0 && tz < nz;
+    const float ay = fmaxf(0.f, fmaxf((float)dy * hy - gyh, -1e-3f - (float)(dy + 1) * hy));
+    const float az = fmaxf(0.f, fmaxf((float)dz * hz - gzh, -1e-3f - (float)(dz + 1) * hz));
+    const float left = reach2 - ay * ay - az * az;
+    if (valid && left >= 0.f) {
+      const float ax = sqrtf(left) + 2e-3f;   // cells that the reach along x touches, slack for the division
+      const int c0 = max(max(-kStencil, (int)floorf(-ax / hx)) + x0 - ix * nx, 0);
+      const int c1 = min(min(mx - 1 + kStencil, (int)floorf((gxh + ax) / hx)) + x0 - ix * nx, nx - 1);
+      if (c0 <= c1) {
+        const int row0 = S.cell_base + (tz * ny + ty) * nx;
+        const int beg = A.cstart[row0 + c0];
+        len = A.cstart[row0 + c1 + 1] - beg;
+        s_beg[threadIdx.x] = beg;
+        s_run[threadIdx.x] = pack_off(0, dy, dz) | (ix - ix_lo) << 24;
+      }
+    }
+  }
+  int pre = len;   // inclusive scan of the lengths over the block
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, pre, o);
+    if (lane >= o) pre += v;
+  }
+  if (lane == 31) s_sum[warp] = pre;
+  __syncthreads();
+  if (warp == 0) {
+    int v = lane < kBuildWarps ? s_sum[lane] : 0;
+#pragma unroll
+    for (int o = 1; o < kBuildWarps; o <<= 1) {
+      const int w = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += w;
+    }
+    if (lane < kBuildWarps) s_sum[lane] = v;
+  }
+  __syncthreads();
+  const int total = s_sum[kBuildWarps - 1];
+  s_pre[threadIdx.x + 1] = pre + (warp ? s_sum[warp - 1] : 0);
+  if (threadIdx.x == 0) s_pre[0] = 0;
+  __syncthreads();
+  if (total == 0) return;   // no atom in the group either
+
+  // ---- rounds: stage candidates (ordered), then test them against every warp's atoms
+  int at = 0, staged = 0;   // uniform over the block
+  bool first_round = true;
+  while (true) {
+    bool full = false;
+    while (at < total) {
+      const int f = at + threadIdx.x;
+      bool keep = false;
+      float px = 0.f, py_ = 0.f, pz_ = 0.f;
+      int j = 0, ko = 0;
+      if (f < total) {
+        int lo = 0, hi = n_runs - 1;   // the run of candidate f: the last one with s_pre <= f
+        while (lo < hi) {
+          const int mid = (lo + hi + 1) >> 1;
+          if (s_pre[mid] <= f) lo = mid;
+          else hi = mid - 1;
+        }
+        const int slot = s_beg[lo] + f - s_pre[lo], o = s_run[lo];
+        const float4 sj = A.s32c[slot];
+        j = A.catoms[slot];
+        const int kx = cell_x(__float_as_int(sj.w)) + (ix_lo + (o >> 24)) * nx - x0;
+        ko = (o & 0xffffff) + kx;
+        px = fmaf((float)kx, hx, sj.x);
+        py_ = fmaf((float)off_y(o), hy, sj.y);
+        pz_ = fmaf((float)off_z(o), hz, sj.z);
+        const float ax = fmaxf(0.f, fmaxf(-1e-3f - px, px - gxh)), ay = fmaxf(0.f, fmaxf(-1e-3f - py_, py_ - gyh)),
+                    az = fmaxf(0.f, fmaxf(-1e-3f - pz_, pz_ - gzh));
+        keep = ax * ax + ay * ay + az * az <= reach2;
+      }
+      const unsigned mk = __ballot_sync(0xffffffffu, keep);
+      __syncthreads();
+      if (lane == 0) s_sum[warp] = __popc(mk);
+      __syncthreads();
+      int before = 0, sum = 0;
+#pragma unroll
+      for (int w = 0; w < kBuildWarps; ++w) {
+        const int v = s_sum[w];
+        before += w < warp ? v : 0;
+        sum += v;
+      }
+      if (staged + sum > kStage) {   // uniform: no room, test what is staged first
+        full = true;
+        break;
+      }
+      if (keep) {
+        const int q = staged + before + __popc(mk & lt);
+        s_pos[q] = make_float4(px, py_, pz_, __int_as_float(j));
+        if (STORED) s_cell[q] = ko;
+      }
+      staged += sum;
+      at += T;
+    }
+    __syncthreads();
+    for (int c0 = 0; c0 < own; c0 += 32) {   // up to 32 of the warp's atoms, one per lane
+      const int nc = min(32, own - c0);
+      const int slot = b + part + (c0 + min(lane, nc - 1)) * parts;
+      const float4 sm = A.s32c[slot];
+      const int me_i = A.catoms[slot];
+      const float mex = fmaf((float)ux, hx, sm.x), mey = fmaf((float)uy, hy, sm.y), mez = fmaf((float)uz, hz, sm.z);
+      int n_in = 0, n_skin = 0;   // entries found so far for this lane's atom
+      if (!first_round) {
+        n_in = A.nin[me_i];
+        n_skin = A.cnt[me_i];
+      }
+      const float xlo = warp_min(mex), xhi = warp_max(mex), ylo = warp_min(mey), yhi = warp_max(mey),
+                  zlo = warp_min(mez), zhi = warp_max(mez);
+      unsigned short* const list = s_list[warp];
+      int from = 0;
+      bool first = first_round && !full, direct = false;
+      do {
+        // list the staged candidates within reach of this warp's atoms
+        int listed = 0;
+        while (from < staged) {
+          const int t = from + lane;
+          bool keep = false;
+          if (t < staged) {
+            const float4 p = s_pos[t];
+            const float ax = fmaxf(0.f, fmaxf(xlo - p.x, p.x - xhi)), ay = fmaxf(0.f, fmaxf(ylo - p.y, p.y - yhi)),
+                        az = fmaxf(0.f, fmaxf(zlo - p.z, p.z - zhi));
+            keep = fmaf(ax, ax, fmaf(ay, ay, az * az)) <= reach2;
+          }
+          const unsigned mk = __ballot_sync(0xffffffffu, keep);
+          if (listed + __popc(mk) > kList) break;
+          if (keep) list[listed + __popc(mk & lt)] = (unsigned short)t;
+          listed += __popc(mk);
+          from += 32;
+        }
+        __syncwarp();
+        direct = first && from >= staged;   // all candidates are in the list: rows are written in place
+        first = false;
+        // lane t takes candidates K t .. K t + K - 1 of the list
+        const int K = (listed + 31) >> 5, base = K * lane, nk = min(K, listed - base);
+        for (int u0 = 0; u0 < nc; u0 += kCentres) {
+          float cx[kCentres], cy[kCentres], cz[kCentres];
+          int ci[kCentres];
+          unsigned m[kCentres];   // bit k: candidate k is inside r_c; bit 16 + k: in the skin
+#pragma unroll
+          for (int u = 0; u < kCentres; ++u) {
+            const int src = min(u0 + u, nc - 1);
+            cx[u] = __shfl_sync(0xffffffffu, mex, src);
+            cy[u] = __shfl_sync(0xffffffffu, mey, src);
+            cz[u] = __shfl_sync(0xffffffffu, mez, src);
+            ci[u] = __shfl_sync(0xffffffffu, me_i, src);
+            m[u] = 0;
+          }
+          for (int k = 0; k < nk; ++k) {
+            const float4 p = s_pos[list[base + k]];
+            const unsigned b_in = 1u << k, b_sk = 0x10000u << k;
+#pragma unroll
+            for (int u = 0; u < kCentres; ++u) {
+              const float dx = p.x - cx[u], dy = p.y - cy[u], dz = p.z - cz[u];
+              const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+              const unsigned bit = r2 < A.rpf2 ? b_in : b_sk;
+              if (r2 < r_sure) m[u] |= bit;
+              if (fabsf(r2 - A.rcf2) <= A.band || r2 < 1e-6f) {
+                const int j = __float_as_int(p.w);
+                const int o = STORED ? s_cell[list[base + k]] - (pack_off(ux, uy, uz) - pack_off(0, 0, 0)) : 0;
+                if (r2 < 1e-6f && j == ci[u] && (!STORED || o == pack_off(0, 0, 0))) {
+                  m[u] &= ~bit;   // the atom itself
+                } else if (fabsf(r2 - A.rcf2) <= A.band) {
+                  m[u] &= ~bit;
+                  if (decide(A, S, ci[u], j, o, STORED)) m[u] |= bit;
+                }
+              }
+            }
+          }
+          __syncwarp();
+#pragma unroll
+          for (int u = 0; u < kCentres; ++u) {
+            if (u0 + u >= nc) break;
+            const int cnt = __popc(m[u] & 0xffffu) | (__popc(m[u] >> 16) << 16);
+            int sum = cnt;   // inclusive scan of both counts
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+              const int v = __shfl_up_sync(0xffffffffu, sum, o);
+              if (lane >= o) sum += v;
+            }
+            const int tot = __shfl_sync(0xffffffffu, sum, 31);
+            const int ni = __shfl_sync(0xffffffffu, n_in, u0 + u), ns = __shfl_sync(0xffffffffu, n_skin, u0 + u);
+            sum -= cnt;
+            // in-range entries fill the row from the front; skin entries from the row's end, or,
+            // while more candidates are to come, from the end of its capacity
+            int q_in = ni + (sum & 0xffff);
+            int q_sk = (direct ? ni + (tot & 0xffff) + ns + (tot >> 16) : A.cap) - 1 - ns - (sum >> 16);
+            int* const row = A.nbr + (size_t)ci[u] * A.cap;
+            unsigned bits = m[u];
+            while (bits) {
+              const int k = __ffs(bits) - 1;
+              bits &= bits - 1;
+              const int q = k < 16 ? q_in++ : q_sk--;
+              if (q >= 0 && q < A.cap) {
+                const int t = list[base + (k & 15)];
+                row[q] = __float_as_int(s_pos[t].w);
+                if (STORED)
+                  A.off[(size_t)ci[u] * A.cap + q] = s_cell[t] - (pack_off(ux, uy, uz) - pack_off(0, 0, 0));
+              }
+            }
+            if (lane == u0 + u) {
+              n_in = ni + (tot & 0xffff);
+              n_skin = ns + (tot >> 16);
+            }
+          }
+        }
+        __syncwarp();
+      } while (from < staged);
+      if (full) {   // another round follows
+        if (lane < nc) {
+          A.nin[me_i] = n_in;
+          A.cnt[me_i] = n_skin;
+        }
         continue;
       }
-      float gy = fmaxf(0.f, fmaxf((float)dy * S.hf[1] - sv[1], sv[1] - (float)(dy + 1) * S.hf[1]));
-      if (gz * gz + gy * gy > rmax2) continue;
-      for (int dx = -kStencil; dx <= kStencil; ++dx) {
-        int tx = cw[0] + dx, ix = 0;
-        if (S.periodic[0]) {
-          ix = floor_div(tx, S.nc[0]);
-          tx -= ix * S.nc[0];
-        } else if (tx < 0 || tx >= S.nc[0]) {
-          continue;
-        }
-        float gx = fmaxf(0.f, fmaxf((float)dx * S.hf[0] - sv[0], sv[0] - (float)(dx + 1) * S.hf[0]));
-        if (gz * gz + gy * gy + gx * gx > rmax2) continue;
-        int cid = S.cell_base + (tz * S.nc[1] + ty) * S.nc[0] + tx;
-        int b = cstart[cid], e = cstart[cid + 1];
-        const float ox = (float)dx * S.hf[0] - si.x;
-        const float oy = (float)dy * S.hf[1] - si.y;
-        const float oz = (float)dz * S.hf[2] - si.z;
-#if AP_BUILD_UNROLL > 1
-#pragma unroll kBuildUnroll
-#endif
-        for (int a = b; a < e; ++a) {
-          // the shadows in cell order: the candidate's shadow and index load independently
-          if (a == t_self && dx == 0 && dy == 0 && dz == 0) continue;
-          const float4 sj = s32c[a];
-          const int j = catoms[a];
-          float ddx = ox + sj.x, ddy = oy + sj.y, ddz = oz + sj.z;
-          float r2f = ddx * ddx + ddy * ddy + ddz * ddz;
-          if (r2f > rcf2 + band) continue;
-          bool take = r2f < rcf2 - band;
-          if (!take) {
-            int img[3] = {ix, iy, iz};
-            take = exact_within(x, S, i, j, ci, cunw[j], img, rc2);
-          }
-          if (take) {
-            const bool in = r2f < rpf2;
-            if (n_in + n_skin < cap) {
-              const int pos = in ? n_in : cap - 1 - n_skin;
-              row[pos] = j;
-              if (offrow) offrow[pos] = pack_off(dx, dy, dz);
-            }
-            if (in)
-              ++n_in;
-            else
-              ++n_skin;
+      // rows of more than one turn: the skin entries move from [cap - n_skin, cap) to [n_in, cnt),
+      // each run of 32 read in full before it is written; its destinations lie below every source
+      // of the later runs.  An overflowing row holds cap valid entries (the capacity error makes
+      // the caller rebuild or fail before any result is used).
+      const int cnt = n_in + n_skin;
+      for (int u = 0; !direct && u < nc; ++u) {
+        const int i = __shfl_sync(0xffffffffu, me_i, u), ni = __shfl_sync(0xffffffffu, n_in, u),
+                  ns = __shfl_sync(0xffffffffu, n_skin, u);
+        if (ni + ns >= A.cap) continue;
+        for (int which = 0; which < (STORED ? 2 : 1); ++which) {
+          int* r = (which ? A.off : A.nbr) + (size_t)i * A.cap;
+          for (int k0 = 0; k0 < ns; k0 += 32) {
+            const int k = k0 + lane;
+            const int v = k < ns ? r[A.cap - ns + k] : 0;
+            __syncwarp();
+            if (k < ns) r[ni + k] = v;
           }
         }
       }
-    }
-  }
-  const int cnt = n_in + n_skin;
-  n_in_out = n_in;
-  if (cnt < cap) {
-    // Close the gap: the skin entries move from [cap - n_skin, cap) to [n_in, cnt) in
-    // chunks of 8, each chunk read in full before it is written.  A chunk's
-    // destinations lie below every source of the later chunks (n_in + n_skin < cap),
-    // so no entry is overwritten before it is read.  (A full row has no gap.)
-    int* src = row + cap - n_skin;
-    int* dst = row + n_in;
-    for (int k0 = 0; k0 < n_skin; k0 += 8) {
-      int v[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) v[u] = k0 + u < n_skin ? src[k0 + u] : 0;
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (k0 + u < n_skin) dst[k0 + u] = v[u];
-    }
-    if (offrow) {
-      int* osrc = offrow + cap - n_skin;
-      int* odst = offrow + n_in;
-      for (int k0 = 0; k0 < n_skin; k0 += 8) {
-        int v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = k0 + u < n_skin ? osrc[k0 + u] : 0;
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-          if (k0 + u < n_skin) odst[k0 + u] = v[u];
+      if (lane < nc) {
+        A.cnt[me_i] = min(cnt, A.cap);
+        A.nin[me_i] = min(n_in, A.cap);   // the in-range part (read by the CSP on rows built at its positions)
+        if (cnt > A.cap) {
+          atomicMax(&A.sc->need_eam, cnt);
+          atomicOr(&A.sc->err, kErrCapacity);
+        }
       }
     }
+    if (!full) break;
+    first_round = false;
+    staged = 0;
+    __syncthreads();   // the stage is refilled
   }
-  return cnt;
 }
 
 // FP32 shadows in cell order (s32c[a] = s32[catoms[a]]), for the EAM row build.
@@ -427,32 +679,6 @@ __global__ void k_shadow_cells(int n, const int* __restrict__ catoms, const floa
                                float4* __restrict__ s32c) {
   const int a = blockIdx.x * blockDim.x + threadIdx.x;
   if (a < n) s32c[a] = s32[catoms[a]];
-}
-
-__global__ void __launch_bounds__(128, AP_BUILD_MINB) k_build_eam(int n, const double* __restrict__ x, const SysInfo* __restrict__ sys,
-                            const int* __restrict__ atom_sys, const float4* __restrict__ s32,
-                            const float4* __restrict__ s32c,
-                            const int4* __restrict__ cunw, const int* __restrict__ cstart,
-                            const int* __restrict__ catoms, float rcf2, double rc2, float rpf2, float band,
-                            int cap, int* __restrict__ nbr, int* __restrict__ off, int* __restrict__ cnt,
-                            int* __restrict__ nin, DevScalars* sc) {
-  // Threads take the atoms in cell order: the atoms of one cell walk the same stencil
-  // cells with the same atom counts, so a warp diverges only on the per-atom gap test.
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  const int i = catoms[t];
-  const SysInfo& S = sys_of(sys, atom_sys, i);
-  int a = 0;
-  int c = build_row(i, t, x, S, s32, s32c, cunw, cstart, catoms, rcf2, rc2, rpf2, band, cap, nbr + (size_t)i * cap,
-                    off ? off + (size_t)i * cap : nullptr, a);
-  // an overflowing row holds cap valid entries (the capacity error makes the caller
-  // rebuild or fail before any result is used)
-  cnt[i] = c < cap ? c : cap;
-  nin[i] = a < cap ? a : cap;   // the in-range part (read by the CSP on rows built at its positions)
-  if (c > cap) {
-    atomicMax(&sc->need_eam, c);
-    atomicOr(&sc->err, kErrCapacity);
-  }
 }
 
 __global__ void __launch_bounds__(256) k_build_ace(const int* __restrict__ queue, const int* __restrict__ nq,
@@ -587,12 +813,27 @@ void launch_build_eam(ap_ctx* c, const double* d_x, cudaStream_t s) {
   c->split_rpf2 = (float)(rp * rp);
   k_shadow_cells<<<nblk(c->n, 256), 256, 0, s>>>((int)c->n, c->d_cell_atoms, c->d_sh32, c->d_sh32c);
   c->kernels += 1;
-  k_build_eam<<<nblk(c->n, 128), 128, 0, s>>>((int)c->n, d_x, c->d_sys, c->d_atom_sys, c->d_sh32, c->d_sh32c,
-                                              c->d_cunw,
-                                              c->d_cell_start, c->d_cell_atoms, (float)rc2, rc2, c->split_rpf2,
-                                              kBand, c->cap_eam, c->d_nbr_eam,
-                                              c->stored_off ? c->d_off_eam : nullptr, c->d_cnt_eam, c->d_lim_eam,
-                                              c->d_sc);
+  BuildArgs A;
+  A.x = d_x;
+  A.sys = c->d_sys;
+  A.n_sys = c->n_sys;
+  A.group = c->build_group;
+  A.s32c = c->d_sh32c;
+  A.cunw = c->d_cunw;
+  A.cstart = c->d_cell_start;
+  A.catoms = c->d_cell_atoms;
+  A.rcf2 = (float)rc2;
+  A.rc2 = rc2;
+  A.rpf2 = c->split_rpf2;
+  A.band = kBand;
+  A.cap = c->cap_eam;
+  A.nbr = c->d_nbr_eam;
+  A.off = c->stored_off ? c->d_off_eam : nullptr;
+  A.cnt = c->d_cnt_eam;
+  A.nin = c->d_lim_eam;
+  A.sc = c->d_sc;
+  auto build = c->stored_off ? k_build_eam<true> : k_build_eam<false>;
+  build<<<c->n_groups, kBuildWarps * 32, 0, s>>>(A);
   c->kernels += 1;
 }
 
