@@ -104,7 +104,8 @@ struct DevScalars {
   int n_precise;      // |P| (int32 copy used by kernels)
   int work_counter;   // persistent-kernel work counter
   int work_counter2;  // second persistent-kernel work counter (right after work_counter)
-  int n_csp_slow;     // atoms handed from the FP32 CSP kernel to the exact one
+  int n_csp_slow;     // atoms handed from k_csp_sort to k_csp_exact
+  int n_csp_list;     // atoms handed on by k_csp_near
   int ace_row_max;    // longest ACE row of the last ACE row build
   int n_stale_bad;    // atoms whose CSP the rows of an earlier build cannot decide (stale rows)
   int n_det1;         // detected atoms the lambda spread's second pass visits
@@ -232,7 +233,7 @@ struct ap_ctx {
 
   // lambda state (FP64)
   double* d_csp = nullptr;       // sample
-  int* d_csp_slow = nullptr;     // [n] atoms whose CSP needs the exact selection
+  int* d_csp_slow = nullptr;     // [n] atoms handed on by k_csp_near
   double* d_csp_avg = nullptr;
   double* d_lam0 = nullptr;
   double* d_lam_min = nullptr;

@@ -119,28 +119,53 @@ __device__ inline bool entry_less(const double* __restrict__ x, const SysInfo& S
   return cand_less(ra, ja, sa, rb, jb, sb);
 }
 
+// Ascending FP64 sum of the six pair values (non-negative: their bit patterns order them, in
+// integer instructions).
+__device__ inline double sum_ascending(double v[kHalf]) {
+#pragma unroll
+  for (int a = 1; a < kHalf; ++a)
+#pragma unroll
+    for (int p = a; p > 0; --p)
+      if (__double_as_longlong(v[p]) < __double_as_longlong(v[p - 1])) {
+        const double t = v[p];
+        v[p] = v[p - 1];
+        v[p - 1] = t;
+      }
+  double sum = v[0];
+#pragma unroll
+  for (int a = 1; a < kHalf; ++a) sum = __dadd_rn(sum, v[a]);
+  return sum;
+}
+
 // ------------------------------------------------------------------ CSP
 #ifndef AP_CSP_PREFETCH
 #define AP_CSP_PREFETCH 1   // software-pipelined row walk in the CSP selection (compile-time tuning)
 #endif
 
-// One thread per atom.  All selection arrays are indexed with compile-time
-// indices (fully unrolled insertion), so they live in registers.
-// FAST: every atom, FP32 selections only; an atom whose selection the FP32 values
-// cannot decide (an r_search band hit, an ambiguous 12/13 or 6/7 boundary) is
-// appended to `slow`.  !FAST: the atoms of `slow`, with the exact FP64 selections.
+// Three kernels share the atoms (launch_csp):
+//   k_csp_near   one thread per atom: the 12 nearest and the six smallest pair values found by
+//                thresholds, without sorting; in a crystal they stand apart.  Atoms where they
+//                do not (surfaces, defects, strong disorder) are handed on.
+//   k_csp_sort   one thread per atom: sorted FP32 selections (insertion), for long lists only;
+//                what FP32 cannot decide is handed on again.
+//   k_csp_exact  one warp per atom, exact selections: what is left, short lists, small systems.
+// FP64 arithmetic issues one warp instruction per 16 cycles and SM: a warp per atom for all
+// atoms would take 4 ms on 4,000,000 of them, the 89 FP64 operations of a thread 0.57 ms.
+
+// csp_atom: all selection arrays are indexed with compile-time indices (fully unrolled
+// insertion), so they live in registers.  An atom whose selection the FP32 values cannot
+// decide (an r_search band hit, an ambiguous 12/13 or 6/7 boundary) is appended to `slow`.
 // CSP of atom i (128-thread blocks: the shared arrays are indexed by threadIdx.x).
-// nin (FAST, rows built at these positions, else null): the row's first nin[i] entries
+// nin (rows built at these positions, else null): the row's first nin[i] entries
 // are the ones inside r_c^2 = rpf2 at the build (FP32), the rest lie beyond it.  When the
 // 13th smallest r^2 of that part lies more than two guard bands inside rpf2, no skin
 // entry can enter the 13 nearest or come within a band of the 12/13 boundary, and the
 // skin part is skipped; otherwise it is walked too.
-template <bool FAST>
 __device__ __forceinline__ void csp_atom(int i, const double* __restrict__ x, const uint8_t* __restrict__ ch,
                                          const SysInfo* __restrict__ sys, const int* __restrict__ atom_sys,
                                          const float4* __restrict__ s32, const int4* __restrict__ cunw,
                                          const int* __restrict__ nbr, const int* __restrict__ off,
-                                         const int* __restrict__ cnt, int cap, float rsf2, double rs2,
+                                         const int* __restrict__ cnt, int cap, float rsf2,
                                          double* __restrict__ csp, int* __restrict__ slow, int* __restrict__ n_slow,
                                          const int* __restrict__ nin = nullptr, float rpf2 = 0.f,
                                          float stale2 = 0.f, int* __restrict__ n_stale = nullptr) {
@@ -164,7 +189,7 @@ __device__ __forceinline__ void csp_atom(int i, const double* __restrict__ x, co
     tq[a] = -1;
   }
   int n_in = 0;
-  int q_end = (FAST && nin) ? nin[i] : c;
+  int q_end = nin ? nin[i] : c;
 #if AP_CSP_PREFETCH
   // loads run ahead of the selection: the next entry's shadow and the entry after it
   int j_a = c > 0 ? nbr[row] : 0;
@@ -172,19 +197,17 @@ __device__ __forceinline__ void csp_atom(int i, const double* __restrict__ x, co
   int j_b = c > 1 ? nbr[row + 1] : 0;
 #endif
   for (int q = 0; q < c; ++q) {
-    if (q == q_end) {   // end of the in-range part (FAST with nin only)
+    if (q == q_end) {   // end of the in-range part
       if (tr[kNN] + 2.f * kBand < rpf2) break;
       q_end = c;
     }
 #if AP_CSP_PREFETCH
-    const int j = j_a;
     const float4 sj = s_a;
     j_a = j_b;
     if (q + 1 < c) s_a = s32[j_a];
     if (q + 2 < c) j_b = nbr[row + q + 2];
 #else
-    const int j = nbr[row + q];
-    const float4 sj = s32[j];
+    const float4 sj = s32[nbr[row + q]];
 #endif
     int k[3];
     entry_offset(off, row + q, S, ci.w, __float_as_int(sj.w), k);
@@ -194,13 +217,8 @@ __device__ __forceinline__ void csp_atom(int i, const double* __restrict__ x, co
     const float r2 = dx * dx + dy * dy + dz * dz;
     if (r2 > rsf2 + kBand) continue;
     if (r2 >= rsf2 - kBand) {
-      if constexpr (FAST) {
-        slow[atomicAdd(n_slow, 1)] = i;
-        return;
-      }
-      double d[3];
-      exact_disp(x, S, i, j, ci, cunw[j], k, d);
-      if (!(norm2_exact(d) < rs2)) continue;
+      slow[atomicAdd(n_slow, 1)] = i;
+      return;
     }
     ++n_in;
     if (r2 < tr[kNN]) {
@@ -229,42 +247,10 @@ __device__ __forceinline__ void csp_atom(int i, const double* __restrict__ x, co
     csp[i] = INFINITY;
     return;
   }
-  // 2. exact (r2, j, s) selection when the 12/13 boundary lies within the guard band
+  // 2. FP32 decides the 12 nearest unless the 12/13 boundary lies within the guard band
   if (n_in > kNN && tr[kNN] - tr[kNN - 1] <= 2.f * kBand) {
-    if constexpr (FAST) {
-      slow[atomicAdd(n_slow, 1)] = i;
-      return;
-    }
-    double br[kNN];
-    int bq[kNN];
-#pragma unroll
-    for (int a = 0; a < kNN; ++a) {
-      br[a] = INFINITY;
-      bq[a] = -1;
-    }
-    for (int q = 0; q < c; ++q) {
-      double d[3];
-      int j, s[3];
-      exact_entry(x, S, i, ci, nbr, off, cunw, row, q, d, j, s);
-      const double r2 = norm2_exact(d);
-      if (!(r2 < rs2)) continue;
-      if (!entry_less(x, S, i, ci, nbr, off, cunw, row, r2, q, br[kNN - 1], bq[kNN - 1])) continue;
-      br[kNN - 1] = r2;
-      bq[kNN - 1] = q;
-#pragma unroll
-      for (int p = kNN - 1; p > 0; --p) {
-        if (entry_less(x, S, i, ci, nbr, off, cunw, row, br[p], bq[p], br[p - 1], bq[p - 1])) {
-          const double t = br[p];
-          br[p] = br[p - 1];
-          br[p - 1] = t;
-          const int u = bq[p];
-          bq[p] = bq[p - 1];
-          bq[p - 1] = u;
-        }
-      }
-    }
-#pragma unroll
-    for (int a = 0; a < kNN; ++a) tq[a] = bq[a];
+    slow[atomicAdd(n_slow, 1)] = i;
+    return;
   }
   // 3. FP32 vectors of the 12 and the 7 smallest pair values |r_a + r_b|^2.  The 12
   // vectors and row positions live in shared memory, component-major (thread index
@@ -315,7 +301,7 @@ __device__ __forceinline__ void csp_atom(int i, const double* __restrict__ x, co
       }
     }
   }
-  // 4. exact values of the six smallest pairs (all 66 in FP64 if the 6/7 boundary is ambiguous)
+  // 4. exact values of the six smallest pairs, unless the 6/7 boundary is ambiguous
   double chosen[kHalf];
   if (pv[kHalf] - pv[kHalf - 1] > 2.f * kBand) {
 #pragma unroll
@@ -328,80 +314,346 @@ __device__ __forceinline__ void csp_atom(int i, const double* __restrict__ x, co
       chosen[t] = norm2_exact(s3);
     }
   } else {
-    if constexpr (FAST) {
-      slow[atomicAdd(n_slow, 1)] = i;
-      return;
+    slow[atomicAdd(n_slow, 1)] = i;
+    return;
+  }
+  csp[i] = sum_ascending(chosen);
+}
+
+struct CspArgs {
+  int n;
+  const double* x;
+  const uint8_t* ch;
+  const SysInfo* sys;
+  const int* atom_sys;
+  const float4* s32;
+  const int4* cunw;
+  const int* nbr;
+  const int* off;
+  const int* cnt;
+  int cap;
+  float rsf2;
+  double rs2;
+  double* csp;
+  const int* nin;
+  float rpf2, stale2;
+  int* n_stale;
+};
+
+// Atoms on k_csp_near's list up to which k_csp_exact takes them all (a warp each, about 2 ns);
+// beyond, k_csp_sort's threads (0.7 ns each, but 60 to 100 us however few).
+constexpr int kSortFrom = 48000;   // 965,000 atoms: 45,000 on the list took 0.43 ms sorted, 17,000 0.10 ms exactly
+
+__global__ void __launch_bounds__(128) k_csp_sort(const CspArgs A, const int* __restrict__ list,
+                                                  const int* __restrict__ n_list, int* __restrict__ slow,
+                                                  int* __restrict__ n_slow) {
+  const int m = *n_list;
+  if (m <= kSortFrom) return;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < m; t += gridDim.x * blockDim.x)
+    csp_atom(list[t], A.x, A.ch, A.sys, A.atom_sys, A.s32, A.cunw, A.nbr, A.off, A.cnt, A.cap, A.rsf2, A.csp, slow,
+             n_slow, A.nin, A.rpf2, A.stale2, A.n_stale);
+}
+
+// Thread per atom, FP32 screening by thresholds.  The number of entries walked gives the density
+// and that the first shell's r^2 in an FCC crystal, r1^2 = R^2 (4 sqrt(2) pi/3 / N)^(2/3).  Entries
+// below 1.6 r1^2 go to a short list in shared memory; a threshold (1.6 r1^2 or a little less)
+// that leaves exactly 12 of them is looked for (the second shell lies at twice the first one's
+// r^2), and the next entry must lie more than two guard bands further out.  Likewise the six
+// pairs below r1^2/4 (opposite neighbours; other pairs leave about r1^2 or more), if they are six
+// and stand apart.  Sorting networks over 13 entries and 7 pairs, which this replaces for the
+// atoms of a crystal, were 4 of 5 instructions: 4,000,000 atoms 2.74 -> 1.98 ms,
+// and 0.25 ms less for the exact selections.
+constexpr int kNear = 24;
+#ifndef AP_CSP_MINB
+#define AP_CSP_MINB 8   // resident blocks per SM k_csp_near is compiled for
+#endif
+__global__ void __launch_bounds__(128, AP_CSP_MINB) k_csp_near(const CspArgs A, int* __restrict__ list, int* __restrict__ n_list) {
+  __shared__ float s_r2[kNear][128];
+  __shared__ unsigned short s_q[kNear][128];
+  const int i = blockIdx.x * 128 + threadIdx.x, tx = threadIdx.x;
+  if (i >= A.n) return;
+  if (A.ch && !A.ch[i]) {
+    A.csp[i] = 0.0;
+    return;
+  }
+  const SysInfo& S = sys_of(A.sys, A.atom_sys, i);
+  const float4 si = A.s32[i];
+  const int wi = __float_as_int(si.w);
+  // with nin only the in-range part is walked: the rest lies beyond rpf2
+  const int c = A.nin ? A.nin[i] : A.cnt[i];
+  const size_t row = (size_t)i * A.cap;
+  const float r1 = (A.nin ? A.rpf2 : A.rsf2) * exp2f((2.f / 3.f) * log2f(5.924f / (float)(c + 1)));   // r1^2
+  float top = 1.6f * r1, rest = INFINITY;
+  int n = 0;
+  {
+    // loads run ahead of their use: the next entry's shadow and the entry after it
+    int j_a = c > 0 ? A.nbr[row] : 0;
+    float4 s_a = A.s32[j_a];
+    int j_b = c > 1 ? A.nbr[row + 1] : 0;
+    for (int q = 0; q < c; ++q) {
+      const float4 sj = s_a;
+      j_a = j_b;
+      if (q + 1 < c) s_a = A.s32[j_a];
+      if (q + 2 < c) j_b = A.nbr[row + q + 2];
+      int k[3];
+      entry_offset(A.off, row + q, S, wi, __float_as_int(sj.w), k);
+      const float dx = (float)k[0] * S.hf[0] + sj.x - si.x;
+      const float dy = (float)k[1] * S.hf[1] + sj.y - si.y;
+      const float dz = (float)k[2] * S.hf[2] + sj.z - si.z;
+      const float r2 = dx * dx + dy * dy + dz * dz;
+      if (r2 < top) {
+        if (n < kNear) {
+          s_r2[n][tx] = r2;
+          s_q[n][tx] = (unsigned short)q;
+        }
+        ++n;
+      } else {
+        rest = fminf(rest, r2);
+      }
     }
-#pragma unroll
-    for (int t = 0; t < kHalf; ++t) chosen[t] = INFINITY;
-    double ex[kNN][3];
+  }
+  // the threshold that leaves 12 of the list
+  bool ok = n <= kNear;
+  int m = 0;
+  float far = 0.f;
+  for (int turn = 0; ok && turn < 4; ++turn, top *= 0.92f) {
+    float out = INFINITY;   // the nearest entry of the list beyond the threshold
+    m = 0;
+    far = 0.f;
+    for (int k = 0; k < n; ++k) {
+      const float r2 = s_r2[k][tx];
+      const bool in = r2 < top;
+      m += in ? 1 : 0;
+      far = in ? fmaxf(far, r2) : far;
+      out = in ? out : fminf(out, r2);
+    }
+    if (m <= kNN) {
+      rest = fminf(rest, out);
+      break;
+    }
+  }
+  m = 0;
+  for (int k = 0; ok && k < n; ++k)
+    if (s_r2[k][tx] <= far && m < kNear) s_q[m++][tx] = s_q[k][tx];
+  // the 12 nearest, surely inside r_search, and surely nearer than what was not walked or what
+  // rows older than the positions may miss
+  ok = ok && m == kNN && rest - far > 2.f * kBand && far < A.rsf2 - kBand && (!A.nin || far + 2.f * kBand < A.rpf2) &&
+       (!(A.stale2 > 0.f) || far + 2.f * kBand < A.stale2);
+  unsigned lo = 0, hi = 0;   // the pairs found, a | b << 4, the last one in the low byte
+  if (ok) {
+    float v[kNN][3];
 #pragma unroll
     for (int a = 0; a < kNN; ++a) {
-      int j, s[3];
-      exact_entry(x, S, i, ci, nbr, off, cunw, row, s_tq[a][tx], ex[a], j, s);
+      const int q = s_q[a][tx];
+      const float4 sj = A.s32[A.nbr[row + q]];
+      int k[3];
+      entry_offset(A.off, row + q, S, wi, __float_as_int(sj.w), k);
+      v[a][0] = (float)k[0] * S.hf[0] + sj.x - si.x;
+      v[a][1] = (float)k[1] * S.hf[1] + sj.y - si.y;
+      v[a][2] = (float)k[2] * S.hf[2] + sj.z - si.z;
     }
+    const float lim = 0.25f * r1;
+    float big = 0.f, next = INFINITY;
+    int pairs = 0;
 #pragma unroll
     for (int a = 0; a < kNN; ++a)
 #pragma unroll
       for (int b = a + 1; b < kNN; ++b) {
-        const double s3[3] = {__dadd_rn(ex[a][0], ex[b][0]), __dadd_rn(ex[a][1], ex[b][1]),
-                              __dadd_rn(ex[a][2], ex[b][2])};
-        const double v = norm2_exact(s3);
-        if (v < chosen[kHalf - 1]) {
-          chosen[kHalf - 1] = v;
-#pragma unroll
-          for (int p = kHalf - 1; p > 0; --p) {
-            if (chosen[p] < chosen[p - 1]) {
-              const double t = chosen[p];
-              chosen[p] = chosen[p - 1];
-              chosen[p - 1] = t;
-            }
-          }
+        const float sx = v[a][0] + v[b][0], sy = v[a][1] + v[b][1], sz = v[a][2] + v[b][2];
+        const float p = sx * sx + sy * sy + sz * sz;
+        if (p < lim) {
+          hi = __funnelshift_l(lo, hi, 8);
+          lo = lo << 8 | (unsigned)(a | b << 4);
+          ++pairs;
+          big = fmaxf(big, p);
+        } else {
+          next = fminf(next, p);
         }
       }
+    ok = pairs == kHalf && next - big > 2.f * kBand;
   }
-  // 5. ascending sum of the six values
+  if (!ok) {
+    list[atomicAdd(n_list, 1)] = i;
+    return;
+  }
+  // exact values of the six pairs, summed in ascending order
+  const int4 ci = A.cunw[i];
+  double chosen[kHalf];
 #pragma unroll
-  for (int a = 1; a < kHalf; ++a)
+  for (int t = 0; t < kHalf; ++t) {
+    const unsigned ab = t < 4 ? lo >> (8 * t) : hi >> (8 * (t - 4));
+    double d[2][3];
 #pragma unroll
-    for (int p = a; p > 0; --p)
-      if (chosen[p] < chosen[p - 1]) {
-        const double t = chosen[p];
-        chosen[p] = chosen[p - 1];
-        chosen[p - 1] = t;
+    for (int e = 0; e < 2; ++e) {
+      const int q = s_q[(e ? ab >> 4 : ab) & 15][tx];
+      int j, s[3];
+      exact_entry(A.x, S, i, ci, A.nbr, A.off, A.cunw, row, q, d[e], j, s);
+    }
+    const double s3[3] = {__dadd_rn(d[0][0], d[1][0]), __dadd_rn(d[0][1], d[1][1]), __dadd_rn(d[0][2], d[1][2])};
+    chosen[t] = norm2_exact(s3);
+  }
+  A.csp[i] = sum_ascending(chosen);
+}
+
+template <typename K>
+__device__ inline K warp_min_key(K v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const K u = __shfl_xor_sync(0xffffffffu, v, o);
+    v = u < v ? u : v;
+  }
+  return v;
+}
+
+// One warp per atom: the atoms of list[0, *n_list) or, with a null list, all n atoms.  The 13
+// nearest in FP32 by 13 warp minima over the row (key: r^2 bits, row position); the exact
+// (r^2, j, image) selection instead where FP32 cannot decide the 12/13 boundary.  Then all 66
+// pair values in FP64, two or three per lane, and six minima of their bit patterns.
+// list2: what k_csp_sort handed on, when it ran.
+__global__ void __launch_bounds__(128) k_csp_exact(const CspArgs A, const int* __restrict__ list,
+                                                   const int* __restrict__ n_list, const int* __restrict__ list2,
+                                                   const int* __restrict__ n_list2) {
+  const int lane = threadIdx.x & 31, warps = (gridDim.x * blockDim.x) >> 5;
+  const bool sorted = list && *n_list > kSortFrom;
+  const int m = !list ? A.n : sorted ? *n_list2 : *n_list;
+  const unsigned long long none = ~0ull;
+  for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < m; w += warps) {
+    const int i = !list ? w : sorted ? list2[w] : list[w];
+    if (A.ch && !A.ch[i]) {
+      if (lane == 0) A.csp[i] = 0.0;
+      continue;
+    }
+    const SysInfo& S = sys_of(A.sys, A.atom_sys, i);
+    const float4 si = A.s32[i];
+    const int4 ci = A.cunw[i];
+    const int c = A.cnt[i];
+    const size_t row = (size_t)i * A.cap;
+    // FP32 key of row position t; none outside r_search (decided exactly in its guard band)
+    auto key = [&](int t) -> unsigned long long {
+      const int j = A.nbr[row + t];
+      const float4 sj = A.s32[j];
+      int k[3];
+      entry_offset(A.off, row + t, S, ci.w, __float_as_int(sj.w), k);
+      const float dx = (float)k[0] * S.hf[0] + sj.x - si.x;
+      const float dy = (float)k[1] * S.hf[1] + sj.y - si.y;
+      const float dz = (float)k[2] * S.hf[2] + sj.z - si.z;
+      const float r2 = dx * dx + dy * dy + dz * dz;
+      if (r2 > A.rsf2 + kBand) return none;
+      if (r2 >= A.rsf2 - kBand) {
+        double d[3];
+        exact_disp(A.x, S, i, j, ci, A.cunw[j], k, d);
+        if (!(norm2_exact(d) < A.rs2)) return none;
       }
-  double sum = chosen[0];
+      return (unsigned long long)__float_as_uint(r2) << 32 | (unsigned)t;
+    };
+    constexpr int kKeep = 5;   // keys of the first 160 row positions stay in registers
+    unsigned long long ks[kKeep];
+    int n_in = 0;
 #pragma unroll
-  for (int a = 1; a < kHalf; ++a) sum = __dadd_rn(sum, chosen[a]);
-  csp[i] = sum;
-}
-
-__global__ void __launch_bounds__(128) k_csp(int n, const double* __restrict__ x, const uint8_t* __restrict__ ch,
-                                                const SysInfo* __restrict__ sys, const int* __restrict__ atom_sys,
-                                                const float4* __restrict__ s32, const int4* __restrict__ cunw,
-                                                const int* __restrict__ nbr, const int* __restrict__ off,
-                                                const int* __restrict__ cnt, int cap, float rsf2, double rs2,
-                                                double* __restrict__ csp, int* __restrict__ slow,
-                                                int* __restrict__ n_slow, const int* __restrict__ nin, float rpf2,
-                                                float stale2, int* __restrict__ n_stale) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n)
-    csp_atom<true>(i, x, ch, sys, atom_sys, s32, cunw, nbr, off, cnt, cap, rsf2, rs2, csp, slow, n_slow, nin, rpf2,
-                   stale2, n_stale);
-}
-
-__global__ void __launch_bounds__(128) k_csp_exact(const double* __restrict__ x, const uint8_t* __restrict__ ch,
-                                                   const SysInfo* __restrict__ sys, const int* __restrict__ atom_sys,
-                                                   const float4* __restrict__ s32, const int4* __restrict__ cunw,
-                                                   const int* __restrict__ nbr, const int* __restrict__ off,
-                                                   const int* __restrict__ cnt, int cap, float rsf2, double rs2,
-                                                   double* __restrict__ csp, const int* __restrict__ slow,
-                                                   const int* __restrict__ n_slow, float stale2,
-                                                   int* __restrict__ n_stale) {
-  const int m = *n_slow;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < m; t += gridDim.x * blockDim.x)
-    csp_atom<false>(slow[t], x, ch, sys, atom_sys, s32, cunw, nbr, off, cnt, cap, rsf2, rs2, csp, nullptr, nullptr,
-                    nullptr, 0.f, stale2, n_stale);
+    for (int u = 0; u < kKeep; ++u) {
+      const int t = lane + 32 * u;
+      ks[u] = t < c ? key(t) : none;
+      n_in += __popc(__ballot_sync(0xffffffffu, ks[u] != none));
+    }
+    for (int t0 = 32 * kKeep; t0 < c; t0 += 32) {
+      const int t = t0 + lane;
+      n_in += __popc(__ballot_sync(0xffffffffu, t < c && key(t) != none));
+    }
+    int mine = 0;   // lane a < 12: row position of the a-th neighbour
+    float r12 = INFINITY, r13 = INFINITY;
+    unsigned long long last = 0;
+    for (int a = 0; a <= kNN && a < n_in; ++a) {
+      unsigned long long best = none;
+#pragma unroll
+      for (int u = 0; u < kKeep; ++u)
+        if ((a == 0 || ks[u] > last) && ks[u] < best) best = ks[u];
+      for (int t = 32 * kKeep + lane; t < c; t += 32) {
+        const unsigned long long v = key(t);
+        if ((a == 0 || v > last) && v < best) best = v;
+      }
+      last = warp_min_key(best);
+      if (a == kNN - 1) r12 = __uint_as_float((unsigned)(last >> 32));
+      if (a == kNN) r13 = __uint_as_float((unsigned)(last >> 32));
+      if (lane == a) mine = (int)(unsigned)last;
+    }
+    // rows older than the positions: see csp_atom
+    if (A.stale2 > 0.f && !(n_in >= kNN && r12 + 2.f * kBand < A.stale2) && lane == 0) atomicAdd(A.n_stale, 1);
+    if (n_in < kNN) {
+      if (lane == 0) A.csp[i] = INFINITY;
+      continue;
+    }
+    if (n_in > kNN && r13 - r12 <= 2.f * kBand) {
+      // exact order: the next entry after (r_l, t_l) by (r^2, j, image), 12 times
+      double r_l = -1.0;
+      int t_l = -1;
+      for (int a = 0; a < kNN; ++a) {
+        double r_b = INFINITY;
+        int t_b = -1;
+        for (int t = lane; t < c; t += 32) {
+          double d[3];
+          int j, s[3];
+          exact_entry(A.x, S, i, ci, A.nbr, A.off, A.cunw, row, t, d, j, s);
+          const double r2 = norm2_exact(d);
+          if (!(r2 < A.rs2)) continue;
+          if (t_l >= 0 && (t == t_l || !entry_less(A.x, S, i, ci, A.nbr, A.off, A.cunw, row, r_l, t_l, r2, t))) continue;
+          if (t_b < 0 || entry_less(A.x, S, i, ci, A.nbr, A.off, A.cunw, row, r2, t, r_b, t_b)) {
+            r_b = r2;
+            t_b = t;
+          }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const double r_o = __shfl_xor_sync(0xffffffffu, r_b, o);
+          const int t_o = __shfl_xor_sync(0xffffffffu, t_b, o);
+          if (t_o >= 0 && (t_b < 0 || (t_o != t_b && entry_less(A.x, S, i, ci, A.nbr, A.off, A.cunw, row, r_o, t_o, r_b, t_b)))) {
+            r_b = r_o;
+            t_b = t_o;
+          }
+        }
+        r_l = r_b;
+        t_l = t_b;
+        if (lane == a) mine = t_b;
+      }
+    }
+    double d[3] = {0.0, 0.0, 0.0};
+    if (lane < kNN) {
+      int j, s[3];
+      exact_entry(A.x, S, i, ci, A.nbr, A.off, A.cunw, row, mine, d, j, s);
+    }
+    long long pv[3];
+#pragma unroll
+    for (int u = 0; u < 3; ++u) {
+      int p = lane + 32 * u, a = 0;   // pair p of the 66: (a, b), a < b
+      const bool have = p < kNN * (kNN - 1) / 2;
+      if (!have) p = 0;
+#pragma unroll
+      for (int e = kNN - 1; e > 0; --e)
+        if (a == kNN - 1 - e && p >= e) {
+          p -= e;
+          ++a;
+        }
+      const int b = a + 1 + p;
+      double s3[3];
+#pragma unroll
+      for (int e = 0; e < 3; ++e)
+        s3[e] = __dadd_rn(__shfl_sync(0xffffffffu, d[e], a), __shfl_sync(0xffffffffu, d[e], b));
+      pv[u] = have ? __double_as_longlong(norm2_exact(s3)) : 0x7fffffffffffffffll;
+    }
+    double sum = 0.0;
+    for (int t = 0; t < kHalf; ++t) {
+      const long long best = pv[0] < pv[1] ? (pv[0] < pv[2] ? pv[0] : pv[2]) : (pv[1] < pv[2] ? pv[1] : pv[2]);
+      const long long v = warp_min_key(best);
+      // one copy of the value is used up (equal values are taken one after the other)
+      const unsigned who = __ballot_sync(0xffffffffu, best == v);
+      if (lane == __ffs(who) - 1) {
+        if (pv[0] == v) pv[0] = 0x7fffffffffffffffll;
+        else if (pv[1] == v) pv[1] = 0x7fffffffffffffffll;
+        else pv[2] = 0x7fffffffffffffffll;
+      }
+      sum = t == 0 ? __longlong_as_double(v) : __dadd_rn(sum, __longlong_as_double(v));
+    }
+    if (lane == 0) A.csp[i] = sum;
+  }
 }
 
 // Canonical moving average over a ring buffer [ns][n]: oldest -> newest, then / ns.
@@ -710,14 +962,39 @@ void launch_csp(ap_ctx* c, const double* d_x, const uint8_t* d_ch, cudaStream_t 
     nin = c->d_split_eam;
     rpf2 = rp > 0.0 ? (float)(rp * rp) : 0.f;
   }
-  k_csp<<<nblk(c->n, 128), 128, 0, s>>>((int)c->n, d_x, d_ch, c->d_sys, c->d_atom_sys, c->d_sh32, c->d_cunw,
-                                              c->d_nbr_eam, off, c->d_cnt_eam, c->cap_eam, (float)rs2, rs2, c->d_csp,
-                                              c->d_csp_slow, n_slow, nin, rpf2, stale2, &c->d_sc->n_stale_bad);
-  // the handed-over atoms (a small fraction), grid-stride over the device-side count
-  k_csp_exact<<<c->num_sms * 4, 128, 0, s>>>(d_x, d_ch, c->d_sys, c->d_atom_sys, c->d_sh32, c->d_cunw, c->d_nbr_eam,
-                                             off, c->d_cnt_eam, c->cap_eam, (float)rs2, rs2, c->d_csp,
-                                             c->d_csp_slow, n_slow, stale2, &c->d_sc->n_stale_bad);
-  c->kernels += 2;
+  CspArgs A;
+  A.n = (int)c->n;
+  A.x = d_x;
+  A.ch = d_ch;
+  A.sys = c->d_sys;
+  A.atom_sys = c->d_atom_sys;
+  A.s32 = c->d_sh32;
+  A.cunw = c->d_cunw;
+  A.nbr = c->d_nbr_eam;
+  A.off = off;
+  A.cnt = c->d_cnt_eam;
+  A.cap = c->cap_eam;
+  A.rsf2 = (float)rs2;
+  A.rs2 = rs2;
+  A.csp = c->d_csp;
+  A.nin = nin;
+  A.rpf2 = rpf2;
+  A.stale2 = stale2;
+  A.n_stale = &c->d_sc->n_stale_bad;
+  // a few thousand atoms: a warp each at once (237 atoms 14 us; a thread each took 64 us, since
+  // one atom's chain is that long)
+  if (c->n <= 32 * c->num_sms) {
+    k_csp_exact<<<nblk(c->n, 4), 128, 0, s>>>(A, nullptr, nullptr, nullptr, nullptr);
+    c->kernels += 1;
+    return;
+  }
+  int* n_list = &c->d_sc->n_csp_list;
+  cudaMemsetAsync(n_list, 0, sizeof(int), s);
+  k_csp_near<<<nblk(c->n, 128), 128, 0, s>>>(A, c->d_csp_slow, n_list);
+  // the handed-over atoms, grid-stride over the device-side counts; d_det1 is free until the spread
+  if (c->n > kSortFrom) k_csp_sort<<<c->num_sms * 4, 128, 0, s>>>(A, c->d_csp_slow, n_list, c->d_det1, n_slow);
+  k_csp_exact<<<c->num_sms * 8, 128, 0, s>>>(A, c->d_csp_slow, n_list, c->d_det1, n_slow);
+  c->kernels += c->n > kSortFrom ? 3 : 2;
 }
 
 // d_score: the detection score pushed into the history (CSP, or the selector's p),
