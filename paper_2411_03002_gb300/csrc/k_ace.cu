@@ -14,9 +14,8 @@
 //   k_ace_basis    one warp per precise atom (persistent CTAs, atomic work counter):
 //                  row entries inside r_c compacted; G = g^T Y over 32-neighbour
 //                  shared tiles; A = (1/N0) W . G; nu = 1, 2 energy and gradient;
-//   k_ace_nu3      one lane per precise atom: the nu = 3 energy and gradient with A
-//                  and dE/dA in registers, straight-line code over the merged
-//                  monomials generated from the basis (ace_nu3.inc);
+//   k_ace_nu3      (k_ace_nu3.cu) the nu = 3 energy and gradient as straight-line code over
+//                  the merged monomials generated from the basis (ace_nu3.inc);
 //   k_ace_adjoint  8 or 16 lanes per precise atom: u = W^T dE/dA / N0; each lane evaluates
 //                  the pair force of one neighbour at a time from u (pair_force) and
 //                  scatters -w_i p_ij to neighbour j; +w_i sum p goes to i.
@@ -25,7 +24,7 @@
 #include <cstring>
 #include <cmath>
 
-#include "ap_internal.cuh"
+#include "ace_args.cuh"
 
 namespace ap {
 
@@ -52,21 +51,6 @@ constexpr int kTileWords = sizeof(R) == 4 ? 4 * kTyStep + 4 * kTgStep : kRows * 
 #endif
 template <typename R>
 constexpr int kWarps = sizeof(R) == 4 ? AP_ACE_WARPS : 4;
-
-template <typename R>
-struct V;
-template <>
-struct V<float> {
-  using S4 = float4;
-  using R4 = float4;
-  static __device__ inline int code(const float4& s) { return __float_as_int(s.w); }
-};
-template <>
-struct V<double> {
-  using S4 = double4_32a;
-  using R4 = double4_32a;
-  static __device__ inline int code(const double4_32a& s) { return (int)s.w; }
-};
 
 __device__ inline float rsqrt_(float v) { return rsqrtf(v); }
 __device__ inline double rsqrt_(double v) { return rsqrt(v); }
@@ -452,13 +436,6 @@ __device__ inline void lm_mix(const float (&in)[2][4], const float* __restrict__
   }
 }
 
-__device__ inline float pack_j(int j, float) { return __int_as_float(j); }
-__device__ inline double pack_j(int j, double) { return __longlong_as_double((long long)j); }
-__device__ inline int unpack_j(float v) { return __float_as_int(v); }
-__device__ inline float4 make_r4(float a, float b, float c, float d) { return make_float4(a, b, c, d); }
-__device__ inline double4_32a make_r4(double a, double b, double c, double d) { return make_double4_32a(a, b, c, d); }
-__device__ inline int unpack_j(double v) { return (int)__double_as_longlong(v); }
-
 constexpr int kListCap = 192;   // in-range records per precise atom cached in shared memory (FCC bulk: 134)
 #ifndef AP_ACE3_WARPS
 #define AP_ACE3_WARPS 6
@@ -468,58 +445,6 @@ constexpr int kListCap = 192;   // in-range records per precise atom cached in s
 #endif
 template <typename R>
 constexpr int kWarps3 = sizeof(R) == 4 ? AP_ACE3_WARPS : 4;   // warps per CTA of the adjoint kernel
-
-#include "ace_nu3.inc"
-
-// Arguments of the three ACE kernels.  Scratch indexed by the queue position q
-// carries the per-atom state from one kernel to the next.
-template <typename R>
-struct AceArgs {
-  const int* queue;
-  const int* count;        // queue length (device)
-  DevScalars* stats;
-  int* counter;
-  int* counter2;
-  const SysInfo* sys;
-  const int* atom_sys;
-  const typename V<R>::S4* sh;
-  const int* nbr;
-  const int* off;
-  const int* cnt;
-  int cap;
-  const double* lam;
-  const double* wgt;       // explicit weights w_i (NULL: w_i = 1 - lambda_i)
-  const R* W;
-  const R* M2;
-  const R* C1;
-  const R* M2b;      // phi^(2) tables of the Finnis-Sinclair form
-  const R* C1b;
-  R rc2, inv_rc, inv_n0;
-  int mode;
-  int fs_on;
-  double fs_eps;
-  double* e_prec;
-  float4* facc32;
-  double* facc64;
-  unsigned long long* faccfix;   // fixed-point accumulator [n][3], or NULL (float atomics)
-  typename V<R>::R4* list4;   // [q][rec] in-range (d, j) records in row order (kernel 1 -> 3)
-  int rec;                    // record slots per queue position (>= every ACE row's length)
-  int* nin;          // [q] their number
-  R* a48;            // [q][48] A entries with n <= 2, l <= 3 (input of nu = 3)
-  R* dA;             // [q][200] dE/dA of nu = 1, 2
-  double* e12;       // [q] E of nu = 1, 2
-  R* de3;            // [q][48] dE3/dA (Finnis-Sinclair form: of phi^(1) + F' phi^(2))
-  double* e3;        // [q] E3 (of phi^(1))
-  R* dAb;            // [q][200] dphi^(2)_12/dA                 (Finnis-Sinclair form only)
-  double* e12b;      // [q] phi^(2)_12                          (Finnis-Sinclair form only)
-  double* fs;        // [q][2] F(phi^(2)), F'(phi^(2))          (Finnis-Sinclair form only)
-};
-
-// nu = 3 coefficients, passed by value (kernel parameter space), in the order of kNu3Key.
-template <typename R>
-struct Nu3Coef {
-  R c[AP_NU3_N];
-};
 
 // Kernel 1, one warp per precise atom (persistent CTAs, atomic work counter):
 //   pass 0   row entries inside r_c compacted (displacement and j) into shared memory,
@@ -812,107 +737,6 @@ __global__ void __launch_bounds__(kWarps<R> * 32, sizeof(R) == 4 ? AP_ACE_MINB :
   }
 }
 
-// Kernel 2, one lane per precise atom: nu = 3 energy and gradient with the 48 A
-// entries and their gradient in registers, as straight-line code over the merged
-// monomials (ace_nu3.inc); coefficients are read from the parameter space.  E3
-// follows from Euler's identity for a homogeneous cubic, E3 = (1/3) sum A dE3/dA.
-// Finnis-Sinclair form (FS): a first pass gives the nu = 3 part of phi^(2), hence
-// phi^(2), F and F'; the gradient pass then uses the coefficients c1 + F' c2, and
-// E3 of phi^(1) is E3(c1 + F' c2) - F' E3(c2).
-#ifndef AP_NU3_MINB
-#define AP_NU3_MINB 0   // FP32: resident 128-thread blocks per SM the nu = 3 kernel is compiled for (0: no bound)
-#endif
-#if AP_NU3_MINB > 0
-#define AP_NU3_BOUNDS __launch_bounds__(sizeof(R) == 4 ? 128 : 64, sizeof(R) == 4 ? AP_NU3_MINB : 1)
-#else
-#define AP_NU3_BOUNDS __launch_bounds__(sizeof(R) == 4 ? 128 : 64)
-#endif
-#ifndef AP_NU3_VEC
-#define AP_NU3_VEC 1    // 4-wide loads of A and stores of dE3/dA
-#endif
-template <typename R, bool FS>
-__global__ void AP_NU3_BOUNDS k_ace_nu3(AceArgs<R> a, const Nu3Coef<R> P,
-                                                                       const Nu3Coef<R> Q) {
-  const int m = *a.count;
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < m; q += gridDim.x * blockDim.x) {
-    R A[48], dA[48];
-#if AP_NU3_VEC
-    // 4-wide loads (the rows of a48 are 48 entries, a multiple of 4)
-    const auto* src = reinterpret_cast<const typename V<R>::R4*>(a.a48 + (size_t)q * 48);
-#pragma unroll
-    for (int v = 0; v < 12; ++v) {
-      const auto t = src[v];
-      A[4 * v] = t.x;
-      A[4 * v + 1] = t.y;
-      A[4 * v + 2] = t.z;
-      A[4 * v + 3] = t.w;
-    }
-#else
-    const R* src = a.a48 + (size_t)q * 48;
-#pragma unroll
-    for (int v = 0; v < 48; ++v) A[v] = src[v];
-#endif
-#pragma unroll
-    for (int v = 0; v < 48; ++v) dA[v] = R(0);
-    R fp = R(0);
-    double e3b = 0.0, Fv = 0.0;
-    if constexpr (FS) {
-      R eb = R(0);
-#define NU3_GROUP_BEGIN(x, y) \
-  {                           \
-    const R p_ = A[x] * A[y]; \
-    R s_ = R(0);
-#define NU3_TERM(t, z) s_ = fma(Q.c[t], A[z], s_);
-#define NU3_GROUP_END(x, y) \
-  eb = fma(p_, s_, eb);     \
-  }
-      AP_NU3_BODY
-#undef NU3_GROUP_BEGIN
-#undef NU3_TERM
-#undef NU3_GROUP_END
-      e3b = (double)eb;
-      const double phi2 = a.e12b[q] + e3b;
-      const double sq = sqrt(fabs(phi2) + a.fs_eps * a.fs_eps);
-      Fv = phi2 > 0.0 ? sq - a.fs_eps : (phi2 < 0.0 ? a.fs_eps - sq : 0.0);
-      fp = (R)(0.5 / sq);
-    }
-#define NU3_GROUP_BEGIN(x, y) \
-  {                           \
-    const R p_ = A[x] * A[y]; \
-    R s_ = R(0);
-#define NU3_COEF(t) (FS ? fma(fp, Q.c[t], P.c[t]) : P.c[t])
-#define NU3_TERM(t, z)             \
-  s_ = fma(NU3_COEF(t), A[z], s_); \
-  dA[z] = fma(NU3_COEF(t), p_, dA[z]);
-#define NU3_GROUP_END(x, y)     \
-  dA[x] = fma(s_, A[y], dA[x]); \
-  dA[y] = fma(s_, A[x], dA[y]); \
-  }
-    AP_NU3_BODY
-#undef NU3_GROUP_BEGIN
-#undef NU3_COEF
-#undef NU3_TERM
-#undef NU3_GROUP_END
-    R e = R(0);
-#pragma unroll
-    for (int v = 0; v < 48; ++v) e = fma(A[v], dA[v], e);
-#if AP_NU3_VEC
-    auto* dst = reinterpret_cast<typename V<R>::R4*>(a.de3 + (size_t)q * 48);
-#pragma unroll
-    for (int v = 0; v < 12; ++v) dst[v] = make_r4(dA[4 * v], dA[4 * v + 1], dA[4 * v + 2], dA[4 * v + 3]);
-#else
-    R* dst = a.de3 + (size_t)q * 48;
-#pragma unroll
-    for (int v = 0; v < 48; ++v) dst[v] = dA[v];
-#endif
-    a.e3[q] = (double)e * (1.0 / 3.0) - (FS ? (double)fp * e3b : 0.0);
-    if (FS) {
-      a.fs[2 * (size_t)q] = Fv;
-      a.fs[2 * (size_t)q + 1] = (double)fp;
-    }
-  }
-}
-
 // Energies alone: E_i = E12 + E3 (+ F), one thread per precise atom.
 template <typename R, bool FS>
 __global__ void k_ace_energy(AceArgs<R> a) {
@@ -1111,11 +935,6 @@ void run_ace(ap_ctx* c, const double* d_lam, const double* d_wgt, const int* d_q
   a.e12 = c->d_ace_e12;
   a.de3 = reinterpret_cast<R*>(c->d_ace_de3);
   a.e3 = c->d_ace_e3;
-  static Nu3Coef<R> P, Q;
-  for (int t = 0; t < AP_NU3_N; ++t) {
-    P.c[t] = (R)c->ace.nu3_coef[t];
-    Q.c[t] = (R)c->ace.nu3_coef2[t];
-  }
   const bool fs = c->cfg.ace_fs_on != 0;
 
   const int pi = sizeof(R) == 4 ? 0 : 1;
@@ -1143,12 +962,8 @@ void run_ace(ap_ctx* c, const double* d_lam, const double* d_wgt, const int* d_q
   const int tb = prof_mark(c, s);
   k_ace_basis<R><<<persistent_grid(c->num_sms, b1[pi], kWarps<R>, m), kWarps<R> * 32, s1, s>>>(a);
   prof_add(c, AP_PHASE_ACE_BASIS, tb, prof_mark(c, s));
-  const int t2 = sizeof(R) == 4 ? 128 : 64;
-  if (fs)
-    k_ace_nu3<R, true><<<c->num_sms * (sizeof(R) == 4 ? 8 : 16), t2, 0, s>>>(a, P, Q);
-  else
-    k_ace_nu3<R, false><<<c->num_sms * (sizeof(R) == 4 ? 8 : 16), t2, 0, s>>>(a, P, Q);
-  c->kernels += 3;
+  c->kernels += launch_ace_nu3<R>(c, a, m, s);
+  c->kernels += 2;
   if (!forces) {
     auto ke = fs ? k_ace_energy<R, true> : k_ace_energy<R, false>;
     ke<<<std::max(1, std::min(c->num_sms * 8, (m + 127) / 128)), 128, 0, s>>>(a);
@@ -1160,14 +975,6 @@ void run_ace(ap_ctx* c, const double* d_lam, const double* d_wgt, const int* d_q
 }
 
 }  // namespace
-
-// The compiled nu = 3 code must match the host enumeration of the basis.
-bool ace_nu3_matches(const AceTables& t) {
-  if (t.nu3_key.size() != (size_t)AP_NU3_N) return false;
-  for (int k = 0; k < AP_NU3_N; ++k)
-    if (t.nu3_key[k] != kNu3Key[k]) return false;
-  return true;
-}
 
 void upload_ace_tables(ap_ctx* c) {
   const AceTables& t = c->ace;
