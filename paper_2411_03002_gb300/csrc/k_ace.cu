@@ -83,36 +83,54 @@ __device__ inline void radial(R r, R inv_rc, int mode, R g[8]) {
   }
 }
 
-// Real spherical harmonics of a unit vector (x, y, z), index lm = l^2 + l + m.
+// Real harmonics in the factored form Y_lm = N_lm Pi_lm(z) {A_m | B_m}(x, y) of a unit vector:
+// A_m + i B_m = (x + i y)^m (A for m >= 0, B for m < 0) and Pi_lm the monic polynomial
+// proportional to d^m P_l/dz^m.  kNorm[l^2 + l + m] = N_lm = sqrt((2l + 1)/(4 pi) (l - m)!/(l + m)!)
+// (sqrt 2 if m > 0) (2l)!/(2^l l! (l - m)!).  The adjoint keeps its u rows in the order of
+// evaluation, by m, cosine before sine, l ascending: kSlot[l^2 + l + m].
+__constant__ double kNorm[25] = {
+    0.28209479177387814, 0.48860251190291998, 0.48860251190291992, 0.48860251190291998, 0.54627421529603959,
+    1.0925484305920792,  0.94617469575756008, 1.0925484305920792,  0.54627421529603959, 0.59004358992664363,
+    1.4453057213202771,  2.2852289973223292,  1.865881662950577,   2.2852289973223292,  1.4453057213202771,
+    0.59004358992664363, 0.62583573544917637, 1.7701307697799304,  3.3116114351514598,  4.6833258049010249,
+    3.7024941420321507,  4.6833258049010249,  3.3116114351514598,  1.7701307697799304,  0.62583573544917637};
+__constant__ unsigned char kSlot[25] = {0,  9,  1,  5,  16, 10, 2,  6,  13, 21, 17, 11, 3,
+                                        7,  14, 19, 24, 22, 18, 12, 4,  8,  15, 20, 23};
+
+// Y_lm / N_lm of a unit vector (x, y, z), index lm = l^2 + l + m: 32 operations, the norms being
+// left to the sums over the neighbours (k_ace_basis FP64 1.31 -> 1.17 ms for 12,700 atoms, FP32
+// 0.89 -> 0.87 ms for 255,840; about 70 operations with the norms in every value).
 template <typename R>
 __device__ inline void sh_values(R x, R y, R z, R Y[25]) {
-  const R x2 = x * x, y2 = y * y, z2 = z * z;
-  Y[0] = R(0.28209479177387814);
-  Y[1] = R(0.4886025119029199) * y;
-  Y[2] = R(0.4886025119029199) * z;
-  Y[3] = R(0.4886025119029199) * x;
-  Y[4] = R(1.0925484305920792) * x * y;
-  Y[5] = R(1.0925484305920792) * y * z;
-  Y[6] = R(0.31539156525252005) * (R(2) * z2 - x2 - y2);
-  Y[7] = R(1.0925484305920792) * x * z;
-  Y[8] = R(0.5462742152960396) * (x2 - y2);
-  Y[9] = R(0.5900435899266435) * y * (R(3) * x2 - y2);
-  Y[10] = R(2.890611442640554) * x * y * z;
-  Y[11] = R(0.4570457994644658) * y * (R(4) * z2 - x2 - y2);
-  Y[12] = R(0.3731763325901154) * z * (R(2) * z2 - R(3) * x2 - R(3) * y2);
-  Y[13] = R(0.4570457994644658) * x * (R(4) * z2 - x2 - y2);
-  Y[14] = R(1.445305721320277) * z * (x2 - y2);
-  Y[15] = R(0.5900435899266435) * x * (x2 - R(3) * y2);
-  const R rho = x2 + y2;
-  Y[16] = R(2.5033429417967046) * x * y * (x2 - y2);
-  Y[17] = R(1.7701307697799304) * y * z * (R(3) * x2 - y2);
-  Y[18] = R(0.9461746957575601) * x * y * (R(6) * z2 - rho);
-  Y[19] = R(0.6690465435572892) * y * z * (R(4) * z2 - R(3) * rho);
-  Y[20] = R(0.10578554691520431) * (R(8) * z2 * z2 - R(24) * z2 * rho + R(3) * rho * rho);
-  Y[21] = R(0.6690465435572892) * x * z * (R(4) * z2 - R(3) * rho);
-  Y[22] = R(0.47308734787878004) * (x2 - y2) * (R(6) * z2 - rho);
-  Y[23] = R(1.7701307697799304) * x * z * (x2 - R(3) * y2);
-  Y[24] = R(0.6258357354491761) * (x2 * x2 - R(6) * x2 * y2 + y2 * y2);
+  const R w = z * z;
+  const R A2 = fma(x, x, -y * y), B2 = R(2) * x * y;
+  const R A3 = fma(x, A2, -y * B2), B3 = fma(x, B2, y * A2);
+  const R p31 = w - R(0.2), p41 = z * (w - R(3.0 / 7.0)), p42 = w - R(1.0 / 7.0);
+  Y[0] = R(1);
+  Y[1] = y;
+  Y[2] = z;
+  Y[3] = x;
+  Y[4] = B2;
+  Y[5] = z * y;
+  Y[6] = w - R(1.0 / 3.0);
+  Y[7] = z * x;
+  Y[8] = A2;
+  Y[9] = B3;
+  Y[10] = z * B2;
+  Y[11] = p31 * y;
+  Y[12] = z * (w - R(0.6));
+  Y[13] = p31 * x;
+  Y[14] = z * A2;
+  Y[15] = A3;
+  Y[16] = fma(x, B3, y * A3);
+  Y[17] = z * B3;
+  Y[18] = p42 * B2;
+  Y[19] = p41 * y;
+  Y[20] = fma(w, w - R(6.0 / 7.0), R(3.0 / 35.0));
+  Y[21] = p41 * x;
+  Y[22] = p42 * A2;
+  Y[23] = z * A3;
+  Y[24] = fma(x, A3, -y * B3);
 }
 
 template <typename R>
@@ -162,20 +180,6 @@ __device__ inline void add_force(float4* facc32, double* facc64, unsigned long l
     atomicAdd(&facc64[3 * j + 2], sz);
   }
 }
-
-// Real harmonics in the factored form Y_lm = N_lm Pi_lm(z) {A_m | B_m}(x, y) of a unit vector:
-// A_m + i B_m = (x + i y)^m (A for m >= 0, B for m < 0) and Pi_lm the monic polynomial
-// proportional to d^m P_l/dz^m.  kNorm[l^2 + l + m] = N_lm = sqrt((2l + 1)/(4 pi) (l - m)!/(l + m)!)
-// (sqrt 2 if m > 0) (2l)!/(2^l l! (l - m)!).  The adjoint keeps its u rows in the order of
-// evaluation, by m, cosine before sine, l ascending: kSlot[l^2 + l + m].
-__constant__ double kNorm[25] = {
-    0.28209479177387814, 0.48860251190291998, 0.48860251190291992, 0.48860251190291998, 0.54627421529603959,
-    1.0925484305920792,  0.94617469575756008, 1.0925484305920792,  0.54627421529603959, 0.59004358992664363,
-    1.4453057213202771,  2.2852289973223292,  1.865881662950577,   2.2852289973223292,  1.4453057213202771,
-    0.59004358992664363, 0.62583573544917637, 1.7701307697799304,  3.3116114351514598,  4.6833258049010249,
-    3.7024941420321507,  4.6833258049010249,  3.3116114351514598,  1.7701307697799304,  0.62583573544917637};
-__constant__ unsigned char kSlot[25] = {0,  9,  1,  5,  16, 10, 2,  6,  13, 21, 17, 11, 3,
-                                        7,  14, 19, 24, 22, 18, 12, 4,  8,  15, 20, 23};
 
 // Force of one pair, p = dE_i/dr_ij, from the atom's coefficients U[slot][k] = N_lm u_klm:
 //   E = f_cut(r) sum_lm P_lm(c) Pi_lm {A_m | B_m},  P_lm = sum_k U_k T_k(c),  Q_lm = dP_lm/dc.
@@ -485,6 +489,13 @@ __global__ void __launch_bounds__(kWarps<R> * 32, sizeof(R) == 4 ? AP_ACE_MINB :
   const unsigned lt_mask = (1u << lane) - 1u;
   unsigned long long cnt_pairs = 0, cnt_atoms = 0, cnt_mma = 0;   // profiling counts of this warp
   const int q_first = warp * gridDim.x + blockIdx.x, q_all = kWarps<R> * gridDim.x;
+  // norms N_lm of this lane's G entries: FP32 rows lm = lane / 4 + 8 u, FP64 lm = grp + 4 t
+  R norm[sizeof(R) == 4 ? 4 : 7];
+#pragma unroll
+  for (int u = 0; u < (sizeof(R) == 4 ? 4 : 7); ++u) {
+    const int lm = sizeof(R) == 4 ? (lane >> 2) + 8 * u : grp + 4 * u;
+    norm[u] = lm < 25 ? (R)kNorm[lm] : R(0);
+  }
   for (int q = q_first; q < m; q = next_item(a.counter, 1, q_all)) {
     const int i = a.queue[q];
     const SysInfo& S = a.sys[a.atom_sys ? a.atom_sys[i] : 0];
@@ -598,6 +609,10 @@ __global__ void __launch_bounds__(kWarps<R> * 32, sizeof(R) == 4 ? AP_ACE_MINB :
         }
         __syncwarp();
       }
+#pragma unroll
+      for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[mt][u] *= norm[2 * mt + (u >> 1)];
       // acc = G^T as fragments (rows lm, columns k); A = W G, then S = M2 A per l
       float am[2][4], sm[2][4];
       lm_mix(acc, Ws, g8, t4, am);
@@ -683,7 +698,7 @@ __global__ void __launch_bounds__(kWarps<R> * 32, sizeof(R) == 4 ? AP_ACE_MINB :
 #pragma unroll
       for (int t = 0; t < 7; ++t) {
         const int lm = grp + 4 * t;
-        if (lm < 25) Gs[kq * 25 + lm] = acc[t];
+        if (lm < 25) Gs[kq * 25 + lm] = acc[t] * norm[t];
       }
       __syncwarp();
       for (int o = lane; o < 200; o += 32) {
