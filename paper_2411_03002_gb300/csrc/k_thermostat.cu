@@ -130,9 +130,8 @@ __device__ inline T warp_sum(T v) {
 // Total mass and centre-of-mass velocity from the lanes' masses and momenta: four sums over the
 // warp in 6 additions per lane instead of 20 (FP64 additions issue at one per 16 cycles here):
 // the halves of the warp first split the four values among themselves, then every group of 8
-// lanes reduces one of them and divides it by the mass (a true division: a group of one atom
-// has no relative velocity).
-__device__ inline void warp_centre(double sm, double& px, double& py, double& pz) {
+// lanes reduces one of them and divides it by the mass.
+__device__ inline void warp_centre(double& sm, double& px, double& py, double& pz) {
   const int lane = threadIdx.x & 31;
   const bool hi = lane & 16, mid = lane & 8;
   double k0 = hi ? py : sm, k1 = hi ? pz : px;
@@ -142,7 +141,8 @@ __device__ inline void warp_centre(double sm, double& px, double& py, double& pz
   k += __shfl_xor_sync(0xffffffffu, mid ? k0 : k1, 8);
 #pragma unroll
   for (int o = 4; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
-  k = k / __shfl_sync(0xffffffffu, k, 0);
+  sm = __shfl_sync(0xffffffffu, k, 0);
+  k = k / sm;
   px = __shfl_sync(0xffffffffu, k, 8);
   py = __shfl_sync(0xffffffffu, k, 16);
   pz = __shfl_sync(0xffffffffu, k, 24);
@@ -291,6 +291,8 @@ __global__ void __launch_bounds__(32) k_th_rescale(
       }
     }
     k = warp_sum(k) * (0.5 / kAcc);
+    // a group of atom i alone has no relative velocity, whatever (m v) / m rounds to
+    if (sm == __shfl_sync(0xffffffffu, mi, 0)) k = 0.0;
     const double rad = k > 0.0 ? de / k + 1.0 : (de == 0.0 ? 1.0 : -1.0);
     if (rad < 0.0) {
       ++n_bad;
