@@ -242,6 +242,7 @@ ap_status ensure_capacity(ap_ctx* c, int64_t n) {
   CK(dalloc(c->d_cunw, m));
   CK(dalloc(c->d_cell_atoms, m));
   CK(dalloc(c->d_slot, m));
+  CK(dalloc(c->d_qpos, m));
   CK(dalloc(c->d_sh32, m));
   CK(dalloc(c->d_sh32c, m));
   CK(dalloc(c->d_sh64, m));
@@ -368,7 +369,10 @@ ap_status build_checked(ap_ctx* c, const double* d_x, const int32_t* d_species, 
 // ACE rows of a queue whose length is the device scalar d_count (a field of
 // c->d_sc), with the ACE storage sized for that length first and the pair records for
 // the longest row after; grows the row capacity once on overflow.  Synchronises.
-ap_status build_ace_checked(ap_ctx* c, const double* d_x, const int* d_queue, const int* d_count, cudaStream_t s) {
+// caller_queue: the queue was copied by k_copy_queue, which says whether it is strictly ascending;
+// the library's own queues are.
+ap_status build_ace_checked(ap_ctx* c, const double* d_x, const int* d_queue, const int* d_count, cudaStream_t s,
+                            bool caller_queue = false) {
   const size_t off = (size_t)((const char*)d_count - (const char*)c->d_sc);
   if (off + sizeof(int) > sizeof(DevScalars)) return fail(c, AP_ERR_ARG, "queue length outside the device scalars");
   for (int attempt = 0; attempt < 2; ++attempt) {
@@ -381,7 +385,7 @@ ap_status build_ace_checked(ap_ctx* c, const double* d_x, const int* d_queue, co
     std::memcpy(&m, (const char*)c->h_sc + off, sizeof(int));
     st = ensure_ace_queue(c, m);
     if (st) return st;
-    launch_build_ace(c, d_x, d_queue, d_count, s);
+    launch_build_ace(c, d_x, d_queue, d_count, m, !caller_queue || c->h_sc->queue_dup == 0, s);
     CK(cudaGetLastError());
     st = read_scalars(c, s);
     if (st) return st;
@@ -421,9 +425,11 @@ __global__ void k_copy_queue(const int* __restrict__ src, const int* __restrict_
   const int m = *count;
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < m; q += gridDim.x * blockDim.x) {
     int i = src[q];
+    if (q > 0 && src[q - 1] >= i) sc->queue_dup = 1;
     if (i < 0 || i >= n) {
       atomicOr(&sc->err, kErrArg);
       i = 0;
+      sc->queue_dup = 1;
     }
     dst[q] = i;
   }
@@ -653,7 +659,7 @@ void ap_destroy(ap_ctx* c) {
   if (!c) return;
   cudaDeviceSynchronize();
   void* ptrs[] = {c->d_sys, c->d_atom_sys, c->d_cell, c->d_cunw, c->d_cell_start, c->d_cell_count, c->d_cell_atoms,
-                  c->d_slot, c->d_sh32, c->d_sh32c, c->d_sh64, c->d_sh32b, c->d_sh32a, c->d_org, c->d_vscale, c->d_nbr_eam, c->d_off_eam, c->d_cnt_eam,
+                  c->d_slot, c->d_qpos, c->d_sh32, c->d_sh32c, c->d_sh64, c->d_sh32b, c->d_sh32a, c->d_org, c->d_vscale, c->d_nbr_eam, c->d_off_eam, c->d_cnt_eam,
                   c->d_lim_eam, c->d_split_eam, c->d_nbr_ace, c->d_off_ace, c->d_cnt_ace, c->d_csp, c->d_csp_slow, c->d_csp_avg, c->d_lam0, c->d_lam_min,
                   c->d_lam_avg, c->d_lam_prev, c->d_csp_hist, c->d_lam_hist, c->d_flag, c->d_scan, c->d_detected, c->d_vmin_f, c->d_det1,
                   c->d_precise, c->d_lam_int, c->d_q, c->d_xi, c->d_facc32, c->d_facc64, c->d_faccfix, c->d_efast, c->d_eprec,
@@ -883,8 +889,9 @@ ap_status ap_eval_ace(ap_ctx* c, int64_t n, const double* d_x, const double* d_l
   cudaStream_t s = S(stream);
   launch_shadow(c, d_x, s);
   k_set_count<<<1, 1, 0, s>>>((const long long*)d_n_precise, (int)n, &c->d_sc->n_precise, &c->d_sc->n_precise64);
+  CK(cudaMemsetAsync(&c->d_sc->queue_dup, 0, sizeof(int), s));
   k_copy_queue<<<c->num_sms * 4, 256, 0, s>>>(d_precise_idx, &c->d_sc->n_precise, (int)n, c->d_precise, c->d_sc);
-  ap_status st = build_ace_checked(c, d_x, c->d_precise, &c->d_sc->n_precise, s);
+  ap_status st = build_ace_checked(c, d_x, c->d_precise, &c->d_sc->n_precise, s, true);
   if (st) return st;
   CK(cudaMemsetAsync(d_e_prec, 0, sizeof(double) * (size_t)n, s));
   launch_ace(c, d_lam, c->d_precise, d_e_prec, d_f != nullptr, s);

@@ -108,6 +108,8 @@ struct DevScalars {
   int n_csp_list;     // atoms handed on by k_csp_near
   int ace_row_max;    // longest ACE row of the last ACE row build
   int n_stale_bad;    // atoms whose CSP the rows of an earlier build cannot decide (stale rows)
+  int n_ace_groups;   // cell groups with queued atoms (ACE row build)
+  int queue_dup;      // 1: the caller's queue is not strictly ascending (an atom may stand in it twice)
   int n_det1;         // detected atoms the lambda spread's second pass visits
   unsigned long long row_total;   // ap_neighbor_total's result
   unsigned int max_disp2_bits;  // float bits of the largest squared displacement
@@ -211,6 +213,7 @@ struct ap_ctx {
   int* d_cell_count = nullptr;   // [n_cells]
   int* d_cell_atoms = nullptr;   // [n]
   int* d_slot = nullptr;         // [n] slot inside cell
+  int* d_qpos = nullptr;         // [n] queue position of every atom (-1: none) during an ACE row build
   float4* d_sh32 = nullptr;      // FP32 cell-relative shadow
   float4* d_sh32c = nullptr;     // the same in cell order (the EAM row build's candidate stream)
   double4_32a* d_sh64 = nullptr;     // FP64 cell-relative shadow
@@ -349,7 +352,9 @@ void launch_cell_sort(ap_ctx* c, cudaStream_t s);
 void launch_shadow(ap_ctx* c, const double* d_x, cudaStream_t s);
 void launch_build_eam(ap_ctx* c, const double* d_x, cudaStream_t s);
 void launch_row_total(ap_ctx* c, int which, int rows, cudaStream_t s);   // -> c->d_sc->row_total
-void launch_build_ace(ap_ctx* c, const double* d_x, const int* d_queue, const int* d_nq, cudaStream_t s);
+// m: the queue's length; unique: no atom stands in the queue twice
+void launch_build_ace(ap_ctx* c, const double* d_x, const int* d_queue, const int* d_nq, int m, bool unique,
+                      cudaStream_t s);
 void launch_export_rows(ap_ctx* c, int which, int rows, int cap_out, int* d_cnt, int* d_idx, int* d_shift,
                         cudaStream_t s);
 void launch_wrap_positions(ap_ctx* c, double* d_x, cudaStream_t s);

@@ -328,7 +328,9 @@ __device__ inline int build_row_warp(int i, const double* __restrict__ x, const 
 // rows built at its own positions may stop after the first part.
 constexpr int kBuildWarps = 8;     // warps per block
 constexpr int kStage = 1024;       // staged candidates per block; a fuller stage is used up in rounds
-constexpr int kList = 416;         // listed candidates per warp (13 per lane), used up in turns likewise
+// listed candidates per warp (13 or 16 per lane), used up in turns likewise
+template <bool ACE>
+constexpr int kList = ACE ? 512 : 416;
 constexpr int kCentres = 3;        // atoms tested together against a listed candidate
 
 struct BuildArgs {
@@ -342,6 +344,15 @@ struct BuildArgs {
   float rcf2;
   double rc2;
   float rpf2, band;
+  // ACE rows only: the queue position of every atom (-1: none), the groups that hold queued atoms,
+  // the atoms' own shadows, the stencil's half-width and the atoms' displacement since the cells
+  // were built (build_row_warp)
+  const int* qpos;
+  const int* groups;
+  const int* n_list;
+  const float4* s32;
+  int sten, n_groups;
+  float margin;
   int cap;
   int* nbr;
   int* off;
@@ -377,22 +388,30 @@ __device__ inline float warp_max(float v) { return -warp_min(-v); }
 #endif
 // STORED: the box is narrower than five cells in a periodic dimension and rows carry the cell
 // offsets; otherwise they follow from the two atoms' cells.
-template <bool STORED>
+// ACE: the rows of the queued atoms, in queue order, at the ACE radius (no split).
+template <bool STORED, bool ACE>
 __global__ void __launch_bounds__(kBuildWarps * 32, AP_BUILD_MINB)
-    k_build_eam(const __grid_constant__ BuildArgs A) {
+    k_build_rows(const __grid_constant__ BuildArgs A) {
   constexpr int T = kBuildWarps * 32;
   __shared__ float4 s_pos[kStage];                      // position relative to the group's first cell, atom index
   __shared__ int s_cell[STORED ? kStage : 1];           // cell relative to the group's first cell (pack_off)
-  __shared__ unsigned short s_list[kBuildWarps][kList];
+  __shared__ unsigned short s_list[kBuildWarps][kList<ACE>];
   __shared__ int s_beg[T], s_pre[T + 1], s_run[T];      // runs: first slot, candidates before, cell (pack_off) and image
   __shared__ int s_sum[kBuildWarps + 1];
+  __shared__ int s_own[ACE ? kBuildWarps : 1][ACE ? 32 : 1];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
-  // the block's system and group of cells
+  const int sten = ACE ? A.sten : kStencil;
+  const float margin = ACE ? A.margin : 0.f;
+  const int n_work = ACE ? *A.n_list : A.n_groups;
+  for (int item = blockIdx.x; item < n_work; item += gridDim.x) {
+  const int group_id = ACE ? A.groups[item] : item;
+  __syncthreads();   // the shared arrays of the last item
+  // the system and the group of cells
   int sys = 0;
   for (int lo = 0, hi = A.n_sys - 1; lo <= hi;) {
     const int mid = (lo + hi) >> 1;
-    if (A.sys[mid].grp_base <= (int)blockIdx.x) {
+    if (A.sys[mid].grp_base <= group_id) {
       sys = mid;
       lo = mid + 1;
     } else {
@@ -403,7 +422,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32, AP_BUILD_MINB)
   const int nx = S.nc[0], ny = S.nc[1], nz = S.nc[2];
   const float hx = S.hf[0], hy = S.hf[1], hz = S.hf[2];
   const int gx = (nx + A.group - 1) / A.group, gy = (ny + A.group - 1) / A.group;
-  const int gid = blockIdx.x - S.grp_base;
+  const int gid = group_id - S.grp_base;
   const int x0 = gid % gx * A.group, y0 = gid / gx % gy * A.group, z0 = gid / (gx * gy) * A.group;
   const int mx = min(A.group, nx - x0), my = min(A.group, ny - y0), mz = min(A.group, nz - z0);
   const float reach2 = A.rcf2 + A.band, r_sure = A.rcf2 - A.band;
@@ -421,29 +440,32 @@ __global__ void __launch_bounds__(kBuildWarps * 32, AP_BUILD_MINB)
     b = A.cstart[cell];
     own = max(0, (A.cstart[cell + 1] - b - part + parts - 1) / parts);   // atoms part, part + parts, ...
   }
-  // ---- the runs of the group's stencil: pencil (dy, dz), periodic image ix along x
-  const int py = my + 2 * kStencil, pz = mz + 2 * kStencil;
-  const int ix_lo = S.periodic[0] ? floor_div(x0 - kStencil, nx) : 0;
-  const int n_im = S.periodic[0] ? floor_div(x0 + mx - 1 + kStencil, nx) - ix_lo + 1 : 1;
-  const int n_runs = py * pz * n_im;   // <= 36 * 2, or 25 * 5 for a single cell
-  const float gxh = (float)mx * hx + 1e-3f, gyh = (float)my * hy + 1e-3f, gzh = (float)mz * hz + 1e-3f;
+  // ---- the runs of the group's stencil: pencil (dy, dz), periodic image ix along x.  Cells are
+  // cut at the reach plus the margin of the group's box grown by the margin.
+  const int py = my + 2 * sten, pz = mz + 2 * sten;
+  const int ix_lo = S.periodic[0] ? floor_div(x0 - sten, nx) : 0;
+  const int n_im = S.periodic[0] ? floor_div(x0 + mx - 1 + sten, nx) - ix_lo + 1 : 1;
+  const int n_runs = py * pz * n_im;   // at most T (launch_build_eam, launch_build_ace)
+  const float blo = -margin - 1e-3f;
+  const float gxh = (float)mx * hx - blo, gyh = (float)my * hy - blo, gzh = (float)mz * hz - blo;
+  const float prune = sqrtf(A.rcf2) + margin, prune2 = prune * prune + A.band;
   int len = 0;
   if (threadIdx.x < n_runs) {
     const int pen = threadIdx.x / n_im, ix = ix_lo + threadIdx.x - pen * n_im;
-    const int dz = pen / py - kStencil, dy = pen % py - kStencil;
+    const int dz = pen / py - sten, dy = pen % py - sten;
     int ty = y0 + dy, tz = z0 + dz;
     bool valid = true;
     if (S.periodic[1]) ty -= floor_div(ty, ny) * ny;
     else valid = valid && ty >= 0 && ty < ny;
     if (S.periodic[2]) tz -= floor_div(tz, nz) * nz;
     else valid = valid && tz >= 0 && tz < nz;
-    const float ay = fmaxf(0.f, fmaxf((float)dy * hy - gyh, -1e-3f - (float)(dy + 1) * hy));
-    const float az = fmaxf(0.f, fmaxf((float)dz * hz - gzh, -1e-3f - (float)(dz + 1) * hz));
-    const float left = reach2 - ay * ay - az * az;
+    const float ay = fmaxf(0.f, fmaxf((float)dy * hy - gyh, blo - (float)(dy + 1) * hy));
+    const float az = fmaxf(0.f, fmaxf((float)dz * hz - gzh, blo - (float)(dz + 1) * hz));
+    const float left = prune2 - ay * ay - az * az;
     if (valid && left >= 0.f) {
       const float ax = sqrtf(left) + 2e-3f;   // cells that the reach along x touches, slack for the division
-      const int c0 = max(max(-kStencil, (int)floorf(-ax / hx)) + x0 - ix * nx, 0);
-      const int c1 = min(min(mx - 1 + kStencil, (int)floorf((gxh + ax) / hx)) + x0 - ix * nx, nx - 1);
+      const int c0 = max(max(-sten, (int)floorf((blo - ax) / hx)) + x0 - ix * nx, 0);
+      const int c1 = min(min(mx - 1 + sten, (int)floorf((gxh + ax) / hx)) + x0 - ix * nx, nx - 1);
       if (c0 <= c1) {
         const int row0 = S.cell_base + (tz * ny + ty) * nx;
         const int beg = A.cstart[row0 + c0];
@@ -475,7 +497,10 @@ __global__ void __launch_bounds__(kBuildWarps * 32, AP_BUILD_MINB)
   s_pre[threadIdx.x + 1] = pre + (warp ? s_sum[warp - 1] : 0);
   if (threadIdx.x == 0) s_pre[0] = 0;
   __syncthreads();
-  if (total == 0) return;   // no atom in the group either
+  if (total == 0) {   // no atom in the group either
+    if constexpr (ACE) continue;
+    else return;
+  }
 
   // ---- rounds: stage candidates (ordered), then test them against every warp's atoms
   int at = 0, staged = 0;   // uniform over the block
@@ -495,15 +520,15 @@ __global__ void __launch_bounds__(kBuildWarps * 32, AP_BUILD_MINB)
           else hi = mid - 1;
         }
         const int slot = s_beg[lo] + f - s_pre[lo], o = s_run[lo];
-        const float4 sj = A.s32c[slot];
         j = A.catoms[slot];
+        const float4 sj = ACE ? A.s32[j] : A.s32c[slot];
         const int kx = cell_x(__float_as_int(sj.w)) + (ix_lo + (o >> 24)) * nx - x0;
         ko = (o & 0xffffff) + kx;
         px = fmaf((float)kx, hx, sj.x);
         py_ = fmaf((float)off_y(o), hy, sj.y);
         pz_ = fmaf((float)off_z(o), hz, sj.z);
-        const float ax = fmaxf(0.f, fmaxf(-1e-3f - px, px - gxh)), ay = fmaxf(0.f, fmaxf(-1e-3f - py_, py_ - gyh)),
-                    az = fmaxf(0.f, fmaxf(-1e-3f - pz_, pz_ - gzh));
+        const float ax = fmaxf(0.f, fmaxf(blo - px, px - gxh)), ay = fmaxf(0.f, fmaxf(blo - py_, py_ - gyh)),
+                    az = fmaxf(0.f, fmaxf(blo - pz_, pz_ - gzh));
         keep = ax * ax + ay * ay + az * az <= reach2;
       }
       const unsigned mk = __ballot_sync(0xffffffffu, keep);
@@ -531,15 +556,25 @@ __global__ void __launch_bounds__(kBuildWarps * 32, AP_BUILD_MINB)
     }
     __syncthreads();
     for (int c0 = 0; c0 < own; c0 += 32) {   // up to 32 of the warp's atoms, one per lane
-      const int nc = min(32, own - c0);
-      const int slot = b + part + (c0 + min(lane, nc - 1)) * parts;
-      const float4 sm = A.s32c[slot];
+      int nc = min(32, own - c0);
+      int slot = b + part + (c0 + min(lane, nc - 1)) * parts;
+      if constexpr (ACE) {   // the queued ones of them
+        const unsigned queued = __ballot_sync(0xffffffffu, lane < nc && A.qpos[A.catoms[slot]] >= 0);
+        if (!queued) continue;
+        if (queued >> lane & 1) s_own[warp][__popc(queued & lt)] = slot;
+        nc = __popc(queued);
+        __syncwarp();
+        slot = s_own[warp][min(lane, nc - 1)];
+        __syncwarp();
+      }
       const int me_i = A.catoms[slot];
+      const int me_row = ACE ? A.qpos[me_i] : me_i;
+      const float4 sm = ACE ? A.s32[me_i] : A.s32c[slot];
       const float mex = fmaf((float)ux, hx, sm.x), mey = fmaf((float)uy, hy, sm.y), mez = fmaf((float)uz, hz, sm.z);
       int n_in = 0, n_skin = 0;   // entries found so far for this lane's atom
       if (!first_round) {
-        n_in = A.nin[me_i];
-        n_skin = A.cnt[me_i];
+        n_in = ACE ? A.cnt[me_row] : A.nin[me_row];
+        n_skin = ACE ? 0 : A.cnt[me_row];
       }
       const float xlo = warp_min(mex), xhi = warp_max(mex), ylo = warp_min(mey), yhi = warp_max(mey),
                   zlo = warp_min(mez), zhi = warp_max(mez);
@@ -559,7 +594,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32, AP_BUILD_MINB)
             keep = fmaf(ax, ax, fmaf(ay, ay, az * az)) <= reach2;
           }
           const unsigned mk = __ballot_sync(0xffffffffu, keep);
-          if (listed + __popc(mk) > kList) break;
+          if (listed + __popc(mk) > kList<ACE>) break;
           if (keep) list[listed + __popc(mk & lt)] = (unsigned short)t;
           listed += __popc(mk);
           from += 32;
@@ -621,7 +656,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32, AP_BUILD_MINB)
             // while more candidates are to come, from the end of its capacity
             int q_in = ni + (sum & 0xffff);
             int q_sk = (direct ? ni + (tot & 0xffff) + ns + (tot >> 16) : A.cap) - 1 - ns - (sum >> 16);
-            int* const row = A.nbr + (size_t)ci[u] * A.cap;
+            const size_t row = (size_t)(ACE ? __shfl_sync(0xffffffffu, me_row, u0 + u) : ci[u]) * A.cap;
             unsigned bits = m[u];
             while (bits) {
               const int k = __ffs(bits) - 1;
@@ -629,9 +664,8 @@ __global__ void __launch_bounds__(kBuildWarps * 32, AP_BUILD_MINB)
               const int q = k < 16 ? q_in++ : q_sk--;
               if (q >= 0 && q < A.cap) {
                 const int t = list[base + (k & 15)];
-                row[q] = __float_as_int(s_pos[t].w);
-                if (STORED)
-                  A.off[(size_t)ci[u] * A.cap + q] = s_cell[t] - (pack_off(ux, uy, uz) - pack_off(0, 0, 0));
+                A.nbr[row + q] = __float_as_int(s_pos[t].w);
+                if (STORED) A.off[row + q] = s_cell[t] - (pack_off(ux, uy, uz) - pack_off(0, 0, 0));
               }
             }
             if (lane == u0 + u) {
@@ -644,8 +678,8 @@ __global__ void __launch_bounds__(kBuildWarps * 32, AP_BUILD_MINB)
       } while (from < staged);
       if (full) {   // another round follows
         if (lane < nc) {
-          A.nin[me_i] = n_in;
-          A.cnt[me_i] = n_skin;
+          if (!ACE) A.nin[me_row] = n_in;
+          A.cnt[me_row] = ACE ? n_in : n_skin;
         }
         continue;
       }
@@ -654,7 +688,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32, AP_BUILD_MINB)
       // of the later runs.  An overflowing row holds cap valid entries (the capacity error makes
       // the caller rebuild or fail before any result is used).
       const int cnt = n_in + n_skin;
-      for (int u = 0; !direct && u < nc; ++u) {
+      for (int u = 0; !ACE && !direct && u < nc; ++u) {
         const int i = __shfl_sync(0xffffffffu, me_i, u), ni = __shfl_sync(0xffffffffu, n_in, u),
                   ns = __shfl_sync(0xffffffffu, n_skin, u);
         if (ni + ns >= A.cap) continue;
@@ -669,10 +703,13 @@ __global__ void __launch_bounds__(kBuildWarps * 32, AP_BUILD_MINB)
         }
       }
       if (lane < nc) {
-        A.cnt[me_i] = min(cnt, A.cap);
-        A.nin[me_i] = min(n_in, A.cap);   // the in-range part (read by the CSP on rows built at its positions)
+        A.cnt[me_row] = min(cnt, A.cap);
+        if constexpr (!ACE)
+          A.nin[me_row] = min(n_in, A.cap);   // the in-range part (read by the CSP on rows built at its positions)
+        else if (min(cnt, A.cap) > __ldcg(&A.sc->ace_row_max))   // only a new maximum takes the (same-address) atomic
+          atomicMax(&A.sc->ace_row_max, min(cnt, A.cap));
         if (cnt > A.cap) {
-          atomicMax(&A.sc->need_eam, cnt);
+          atomicMax(ACE ? &A.sc->need_ace : &A.sc->need_eam, cnt);
           atomicOr(&A.sc->err, kErrCapacity);
         }
       }
@@ -681,6 +718,26 @@ __global__ void __launch_bounds__(kBuildWarps * 32, AP_BUILD_MINB)
     first_round = false;
     staged = 0;
     __syncthreads();   // the stage is refilled
+  }
+  if constexpr (!ACE) return;   // one block per group
+  }
+}
+
+// qpos[i] = queue position of atom i (the others hold -1), and the list of the cell groups with
+// queued atoms (in any order: it only orders the work).  flag: one int per group, 0.
+__global__ void k_queue_groups(const int* __restrict__ queue, const int* __restrict__ nq, const SysInfo* __restrict__ sys,
+                               const int* __restrict__ atom_sys, const int4* __restrict__ cunw, int group,
+                               int* __restrict__ qpos, int* __restrict__ flag, int* __restrict__ list,
+                               int* __restrict__ n_list) {
+  const int m = *nq;
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < m; q += gridDim.x * blockDim.x) {
+    const int i = queue[q];
+    qpos[i] = q;
+    const SysInfo& S = sys_of(sys, atom_sys, i);
+    const int w = cunw[i].w;
+    const int gx = (S.nc[0] + group - 1) / group, gy = (S.nc[1] + group - 1) / group;
+    const int g = S.grp_base + (cell_z(w) / group * gy + cell_y(w) / group) * gx + cell_x(w) / group;
+    if (flag[g] == 0 && atomicExch(&flag[g], 1) == 0) list[atomicAdd(n_list, 1)] = g;
   }
 }
 
@@ -842,12 +899,18 @@ void launch_build_eam(ap_ctx* c, const double* d_x, cudaStream_t s) {
   A.cnt = c->d_cnt_eam;
   A.nin = c->d_lim_eam;
   A.sc = c->d_sc;
-  auto build = c->stored_off ? k_build_eam<true> : k_build_eam<false>;
+  A.qpos = A.groups = A.n_list = nullptr;
+  A.s32 = c->d_sh32;
+  A.sten = kStencil;
+  A.n_groups = c->n_groups;
+  A.margin = 0.f;
+  auto build = c->stored_off ? k_build_rows<true, false> : k_build_rows<false, false>;
   build<<<c->n_groups, kBuildWarps * 32, 0, s>>>(A);
   c->kernels += 1;
 }
 
-void launch_build_ace(ap_ctx* c, const double* d_x, const int* d_queue, const int* d_nq, cudaStream_t s) {
+void launch_build_ace(ap_ctx* c, const double* d_x, const int* d_queue, const int* d_nq, int m, bool unique,
+                      cudaStream_t s) {
   const double r = c->cfg.ace_rc + c->cfg.skin;
   // Cells older than the positions (ap_step kept the EAM lists): the atoms moved up to
   // m = stale_m since the cell build, so a cell is pruned only beyond r + m and the
@@ -861,6 +924,52 @@ void launch_build_ace(ap_ctx* c, const double* d_x, const int* d_queue, const in
       for (int d = 0; d < 3; ++d) sten = std::max(sten, (int)std::ceil((r + 2.0 * c->stale_m) / S.h[d]));
   }
   double rc2 = r * r;
+  // Cell groups, as for the EAM rows, for long queues in which every atom stands once, where the
+  // stencil's runs fit a block's threads (k_build_rows: 255,840 atoms at 8 A 0.59 ms, a warp per
+  // row 0.83; 240,000 of 4,000,000 at 7.7 A 0.76 and 0.97); a warp per row otherwise (12,700 atoms
+  // 43 us, by groups 51 and the list 5; 83,000 in narrow boxes 0.267 and 0.266 ms).
+  int runs = 0;
+  for (const SysInfo& S : c->h_sys) {
+    const int e = c->build_group + 2 * sten, im = S.periodic[0] ? (e + S.nc[0] - 1) / S.nc[0] + 1 : 1;
+    runs = std::max(runs, e * e * im);
+  }
+  if (m >= 400 * c->num_sms && unique && runs <= kBuildWarps * 32) {
+    int* flag = c->d_cell_count;   // free after the cell sort; n_groups <= n_cells
+    int* list = c->d_slot;         // free after the cell sort; at most one group per atom
+    int* n_list = &c->d_sc->n_ace_groups;
+    cudaMemsetAsync(flag, 0, sizeof(int) * (size_t)c->n_groups, s);
+    cudaMemsetAsync(n_list, 0, sizeof(int), s);
+    cudaMemsetAsync(c->d_qpos, 0xff, sizeof(int) * (size_t)c->n, s);
+    k_queue_groups<<<c->num_sms * 4, 256, 0, s>>>(d_queue, d_nq, c->d_sys, c->d_atom_sys, c->d_cunw, c->build_group,
+                                                  c->d_qpos, flag, list, n_list);
+    BuildArgs A = {};
+    A.x = d_x;
+    A.sys = c->d_sys;
+    A.n_sys = c->n_sys;
+    A.group = c->build_group;
+    A.cunw = c->d_cunw;
+    A.cstart = c->d_cell_start;
+    A.catoms = c->d_cell_atoms;
+    A.rcf2 = (float)rc2;
+    A.rc2 = rc2;
+    A.rpf2 = 3.4e38f;   // no split
+    A.band = kBand;
+    A.qpos = c->d_qpos;
+    A.groups = list;
+    A.n_list = n_list;
+    A.s32 = c->d_sh32;
+    A.sten = sten;
+    A.margin = margin;
+    A.cap = c->cap_ace;
+    A.nbr = c->d_nbr_ace;
+    A.off = c->stored_off ? c->d_off_ace : nullptr;
+    A.cnt = c->d_cnt_ace;
+    A.sc = c->d_sc;
+    auto build = c->stored_off ? k_build_rows<true, true> : k_build_rows<false, true>;
+    build<<<std::max(1, std::min(c->n_groups, c->num_sms * AP_BUILD_MINB * 2)), kBuildWarps * 32, 0, s>>>(A);
+    c->kernels += 2;
+    return;
+  }
   int grid = c->num_sms * 8;
   k_build_ace<<<grid, 256, 0, s>>>(d_queue, d_nq, d_x, c->d_sys, c->d_atom_sys, c->d_sh32, c->d_cunw,
                                    c->d_cell_start, c->d_cell_atoms, (float)rc2, rc2, kBand, c->cap_ace,
