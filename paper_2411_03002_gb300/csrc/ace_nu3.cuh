@@ -8,6 +8,7 @@
 #pragma once
 
 #include <algorithm>
+#include <cstring>
 
 #include "ace_args.cuh"
 
@@ -17,10 +18,17 @@ namespace {
 
 #include "ace_nu3.inc"
 
-// nu = 3 coefficients, passed by value (kernel parameter space), in the order of kNu3Key.
-template <typename R>
+// nu = 3 coefficients, passed by value (kernel parameter space), in the order of kNu3Key; the
+// ones of phi^(2) (second) only in the Finnis-Sinclair form.
+template <typename R, bool FS>
 struct Nu3Coef {
   R c[AP_NU3_N];
+  __device__ R second(int) const { return R(0); }
+};
+template <typename R>
+struct Nu3Coef<R, true> {
+  R c[AP_NU3_N], c2[AP_NU3_N];
+  __device__ R second(int t) const { return c2[t]; }
 };
 
 template <typename R>
@@ -50,10 +58,10 @@ __device__ inline void embed_fs(const AceArgs<R>& a, int q, double e3b, double& 
     const R p_ = A[x] * A[y]; \
     R s_ = R(0);
 // the energy part of the phi^(2) pass (ENERGY), or the gradient
-#define NU3_COEF(t) (FS ? fma(fp, Q.c[t], P.c[t]) : P.c[t])
+#define NU3_COEF(t) (FS ? fma(fp, P.second(t), P.c[t]) : P.c[t])
 #define NU3_TERM(t, z)                          \
   if constexpr (ENERGY) {                       \
-    s_ = fma(Q.c[t], A[z], s_);                 \
+    s_ = fma(P.second(t), A[z], s_);            \
   } else {                                      \
     s_ = fma(NU3_COEF(t), A[z], s_);            \
     dA[z] = fma(NU3_COEF(t), p_, dA[z]);        \
@@ -74,8 +82,7 @@ struct Int {
 
 // Part PART of the monomials (PART = -1: all of them).
 template <typename R, bool FS, bool ENERGY, int PART>
-__device__ __forceinline__ void nu3_body(const R A[48], R dA[48], R& eb, R fp, const Nu3Coef<R>& P,
-                                         const Nu3Coef<R>& Q) {
+__device__ __forceinline__ void nu3_body(const R A[48], R dA[48], R& eb, R fp, const Nu3Coef<R, FS>& P) {
   if constexpr (PART == -1) {
     AP_NU3_BODY
   } else if constexpr (PART == 0) {
@@ -105,9 +112,9 @@ static_assert(AP_NU3_PARTS == 8, "nu3_body and k_ace_nu3_parts take eight parts"
 // Long queues (FP32): one lane per atom.  The body is 6,000 FMAs of straight-line code, so this
 // takes 30 us (FP64: 235 us) however few the atoms are.
 template <typename R, bool FS>
-__global__ void __launch_bounds__(128) k_ace_nu3(AceArgs<R> a, const __grid_constant__ Nu3Coef<R> P,
-                                                 const __grid_constant__ Nu3Coef<R> Q) {
+__global__ void __launch_bounds__(128) k_ace_nu3(AceArgs<R> a, const __grid_constant__ Nu3Coef<R, FS> P) {
   const int m = *a.count;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *a.counter = *a.counter2 = 0;
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < m; q += gridDim.x * blockDim.x) {
     R A[48], dA[48];
     load48(a.a48 + (size_t)q * 48, A);
@@ -116,10 +123,10 @@ __global__ void __launch_bounds__(128) k_ace_nu3(AceArgs<R> a, const __grid_cons
     R fp = R(0), eb = R(0), e = R(0);
     double F = 0.0;
     if constexpr (FS) {
-      nu3_body<R, FS, true, -1>(A, dA, eb, fp, P, Q);
+      nu3_body<R, FS, true, -1>(A, dA, eb, fp, P);
       embed_fs(a, q, (double)eb, F, fp);
     }
-    nu3_body<R, FS, false, -1>(A, dA, e, fp, P, Q);
+    nu3_body<R, FS, false, -1>(A, dA, e, fp, P);
 #pragma unroll
     for (int v = 0; v < 48; ++v) e = fma(A[v], dA[v], e);
     auto* dst = reinterpret_cast<typename V<R>::R4*>(a.de3 + (size_t)q * 48);
@@ -139,13 +146,13 @@ __global__ void __launch_bounds__(128) k_ace_nu3(AceArgs<R> a, const __grid_cons
 // 235 -> 66 us, 12,700 atoms 236 -> 196 us) and by FP32 while the queue is one wave of its blocks,
 // two per SM: 155 atoms 33 -> 14 us, but 12,700 atoms 28 us with a lane per atom against 32.
 template <typename R, bool FS>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_ace_nu3_parts(AceArgs<R> a, const __grid_constant__ Nu3Coef<R> P,
-                                                       const __grid_constant__ Nu3Coef<R> Q) {
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_ace_nu3_parts(AceArgs<R> a, const __grid_constant__ Nu3Coef<R, FS> P) {
   extern __shared__ __align__(32) unsigned char smem_raw[];
   R* part = reinterpret_cast<R*>(smem_raw);   // [8][48][32] partial gradients
   __shared__ R s_e[8][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int m = *a.count;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *a.counter = *a.counter2 = 0;
   for (int q0 = blockIdx.x * 32; q0 < m; q0 += gridDim.x * 32) {
     const int q = q0 + lane;
     const R* src = a.a48 + (size_t)min(q, m - 1) * 48;
@@ -159,7 +166,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_ace_nu3_parts(A
 #pragma unroll
       for (int v = 0; v < 48; ++v) dA[v] = R(0);
       R e = R(0);
-      nu3_body<R, FS, ENERGY, PART>(A, dA, e, fp, P, Q);
+      nu3_body<R, FS, ENERGY, PART>(A, dA, e, fp, P);
       if (ENERGY) {
         s_e[PART][lane] = e;
       } else {
@@ -222,27 +229,31 @@ constexpr size_t kPartBytes = sizeof(R) * 8 * 48 * 32;
 #define AP_NU3_LONG 64   // atoms per SM from which FP32 queues take one lane per atom
 #endif
 
+template <typename R, bool FS>
+void run_nu3(ap_ctx* c, const AceArgs<R>& a, int m, cudaStream_t s) {
+  Nu3Coef<R, FS> P;
+  const R* src;
+  if constexpr (sizeof(R) == 4) src = c->ace.nu3_f32.data();
+  else src = c->ace.nu3_coef.data();
+  std::memcpy(P.c, src, sizeof(P.c));
+  if constexpr (FS) std::memcpy(P.c2, sizeof(R) == 4 ? src + AP_NU3_N : (const R*)c->ace.nu3_coef2.data(), sizeof(P.c2));
+  if constexpr (sizeof(R) == 4) {
+    if (m >= AP_NU3_LONG * c->num_sms) {
+      k_ace_nu3<R, FS><<<c->num_sms * 8, 128, 0, s>>>(a, P);
+      return;
+    }
+  }
+  cudaFuncSetAttribute(k_ace_nu3_parts<R, FS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPartBytes<R>);
+  const int blocks = std::max(1, std::min((m + 31) / 32, c->num_sms * (sizeof(R) == 4 ? 4 : 2)));
+  k_ace_nu3_parts<R, FS><<<blocks, 256, kPartBytes<R>, s>>>(a, P);
+}
+
 }  // namespace
 
 template <typename R>
 int launch_ace_nu3(ap_ctx* c, const AceArgs<R>& a, int m, cudaStream_t s) {
-  Nu3Coef<R> P, Q;
-  const bool fs = c->cfg.ace_fs_on != 0;
-  for (int t = 0; t < AP_NU3_N; ++t) {
-    P.c[t] = (R)c->ace.nu3_coef[t];
-    Q.c[t] = (R)c->ace.nu3_coef2[t];
-  }
-  if constexpr (sizeof(R) == 4) {
-    if (m >= AP_NU3_LONG * c->num_sms) {
-      auto k = fs ? k_ace_nu3<R, true> : k_ace_nu3<R, false>;
-      k<<<c->num_sms * 8, 128, 0, s>>>(a, P, Q);
-      return 1;
-    }
-  }
-  auto k = fs ? k_ace_nu3_parts<R, true> : k_ace_nu3_parts<R, false>;
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPartBytes<R>);
-  const int blocks = std::max(1, std::min((m + 31) / 32, c->num_sms * (sizeof(R) == 4 ? 4 : 2)));
-  k<<<blocks, 256, kPartBytes<R>, s>>>(a, P, Q);
+  if (c->cfg.ace_fs_on) run_nu3<R, true>(c, a, m, s);
+  else run_nu3<R, false>(c, a, m, s);
   return 1;
 }
 

@@ -276,9 +276,16 @@ ap_status ensure_capacity(ap_ctx* c, int64_t n) {
   if (q) cudaFree(q);
   CK(cudaMalloc(&c->d_q, 16 * (size_t)m));
   CK(dalloc(c->d_xi, m));
+  // the ACE force accumulators are zero between the evaluations (launch_ace_finalize clears
+  // what it has added)
   CK(dalloc(c->d_facc32, m));
+  CK(cudaMemset(c->d_facc32, 0, sizeof(float4) * (size_t)m));
   CK(dalloc(c->d_facc64, 3 * m));
-  if (c->cfg.ace_deterministic) CK(dalloc(c->d_faccfix, 3 * m));
+  CK(cudaMemset(c->d_facc64, 0, sizeof(double) * 3 * (size_t)m));
+  if (c->cfg.ace_deterministic) {
+    CK(dalloc(c->d_faccfix, 3 * m));
+    CK(cudaMemset(c->d_faccfix, 0, sizeof(unsigned long long) * 3 * (size_t)m));
+  }
   CK(dalloc(c->d_efast, m));
   CK(dalloc(c->d_eprec, m));
   CK(dalloc(c->d_eatom, m));
@@ -319,26 +326,21 @@ ap_status check_err_bits(ap_ctx* c) {
 }
 
 ap_status clear_err(ap_ctx* c, cudaStream_t s) {
-  CK(cudaMemsetAsync(&c->d_sc->err, 0, sizeof(int), s));
-  CK(cudaMemsetAsync(&c->d_sc->need_eam, 0, 2 * sizeof(int), s));
+  // err, need_eam, need_ace, ace_row_max, n_ace_groups
+  CK(cudaMemsetAsync(&c->d_sc->err, 0, 5 * sizeof(int), s));
   return AP_OK;
 }
 
-// Bin, sort, shadow and EAM rows at the given positions (asynchronous).
+// Bin (with the shadows), sort and EAM rows at the given positions (asynchronous).
 void build_async(ap_ctx* c, const double* d_x, const int32_t* d_species, cudaStream_t s) {
   launch_bin(c, d_x, d_species, s);
   launch_cell_sort(c, s);
-  launch_shadow(c, d_x, s);
   launch_build_eam(c, d_x, s);
   if (c->d_split_eam)   // the split of the rows, for a CSP on them after the atoms have moved
     cudaMemcpyAsync(c->d_split_eam, c->d_lim_eam, sizeof(int) * (size_t)c->n, cudaMemcpyDeviceToDevice, s);
   c->lim_valid = false;
   c->cells_stale = false;
   c->stale_m = 0.0;
-  cudaMemcpyAsync(c->d_sh32b, c->d_sh32, sizeof(float4) * (size_t)c->n, cudaMemcpyDeviceToDevice, s);
-  cudaMemsetAsync(&c->d_sc->max_disp2_bits, 0, sizeof(unsigned int), s);
-  // the ACE rows' reference shadows belong to the old cells: +3.4e38 until the next ACE build
-  cudaMemsetAsync(&c->d_sc->max_dispa2_bits, 0x7f, sizeof(unsigned int), s);
   c->rebuilds++;
 }
 
@@ -378,7 +380,6 @@ ap_status build_ace_checked(ap_ctx* c, const double* d_x, const int* d_queue, co
   for (int attempt = 0; attempt < 2; ++attempt) {
     ap_status st = clear_err(c, s);
     if (st) return st;
-    CK(cudaMemsetAsync(&c->d_sc->ace_row_max, 0, sizeof(int), s));
     st = read_scalars(c, s);
     if (st) return st;
     int m = 0;
@@ -411,10 +412,11 @@ void ace_ref(ap_ctx* c, cudaStream_t s) {
 }
 
 // Queue length from the caller's device int64, clamped to [0, n].
-__global__ void k_set_count(const long long* src, int n, int* dst32, long long* dst64) {
+__global__ void k_set_count(const long long* src, int n, int* dst32, long long* dst64, int* dup) {
   long long v = *src;
   v = v < 0 ? 0 : (v > n ? n : v);
   *dst32 = (int)v;
+  *dup = 0;
   if (dst64) *dst64 = v;
 }
 
@@ -641,6 +643,8 @@ ap_status ap_create(const ap_config* h_cfg, ap_ctx** out) {
     delete c;
     return AP_ERR_STATE;
   }
+  c->ace.nu3_f32.assign(c->ace.nu3_coef.begin(), c->ace.nu3_coef.end());
+  c->ace.nu3_f32.insert(c->ace.nu3_f32.end(), c->ace.nu3_coef2.begin(), c->ace.nu3_coef2.end());
   upload_ace_tables(c);
   e = cudaMalloc(&c->d_sc, sizeof(DevScalars));
   if (e == cudaSuccess) e = cudaMallocHost(&c->h_sc, sizeof(DevScalars));
@@ -888,8 +892,8 @@ ap_status ap_eval_ace(ap_ctx* c, int64_t n, const double* d_x, const double* d_l
   if (!d_x || !d_precise_idx || !d_n_precise || !d_e_prec) return fail(c, AP_ERR_ARG, "null argument");
   cudaStream_t s = S(stream);
   launch_shadow(c, d_x, s);
-  k_set_count<<<1, 1, 0, s>>>((const long long*)d_n_precise, (int)n, &c->d_sc->n_precise, &c->d_sc->n_precise64);
-  CK(cudaMemsetAsync(&c->d_sc->queue_dup, 0, sizeof(int), s));
+  k_set_count<<<1, 1, 0, s>>>((const long long*)d_n_precise, (int)n, &c->d_sc->n_precise, &c->d_sc->n_precise64,
+                            &c->d_sc->queue_dup);
   k_copy_queue<<<c->num_sms * 4, 256, 0, s>>>(d_precise_idx, &c->d_sc->n_precise, (int)n, c->d_precise, c->d_sc);
   ap_status st = build_ace_checked(c, d_x, c->d_precise, &c->d_sc->n_precise, s, true);
   if (st) return st;
@@ -1055,6 +1059,9 @@ ap_status ap_step(ap_ctx* c, int64_t n, double* d_x, double* d_v, double* d_f, c
         st = build_ace_checked(c, d_x, c->d_precise, &c->d_sc->n_precise, s);
         if (st) return st;
         ace_ref(c, s);
+        // E^p is 0 outside the queue: cleared when the queue may have changed, the atoms of the
+        // queue are written by every evaluation
+        CK(cudaMemsetAsync(c->d_eprec, 0, sizeof(double) * (size_t)n, s));
       }
     } else if (ace_only) {
       PhaseTimer t(c, s, AP_PHASE_NEIGHBORS);
@@ -1071,7 +1078,6 @@ ap_status ap_step(ap_ctx* c, int64_t n, double* d_x, double* d_v, double* d_f, c
     }
     {
       PhaseTimer t(c, s, AP_PHASE_ACE);
-      CK(cudaMemsetAsync(c->d_eprec, 0, sizeof(double) * (size_t)n, s));
       launch_ace(c, c->d_lam_int, c->d_precise, c->d_eprec, true, s);
     }
     {

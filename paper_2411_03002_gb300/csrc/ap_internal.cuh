@@ -100,15 +100,15 @@ struct DevScalars {
   int err;            // OR of error bits
   int need_eam;       // largest EAM row count seen
   int need_ace;       // largest ACE row count seen
+  int ace_row_max;    // longest ACE row of the last ACE row build
+  int n_ace_groups;   // cell groups with queued atoms (ACE row build); cleared with the four above
   int n_detected;     // |D|
   int n_precise;      // |P| (int32 copy used by kernels)
-  int work_counter;   // persistent-kernel work counter
-  int work_counter2;  // second persistent-kernel work counter (right after work_counter)
+  int work_counter;   // persistent-kernel work counters: 0 between the launches, k_ace_nu3 resets
+  int work_counter2;  // both (the first kernel has used the one, the third not yet the other)
   int n_csp_slow;     // atoms handed from k_csp_sort to k_csp_exact
   int n_csp_list;     // atoms handed on by k_csp_near
-  int ace_row_max;    // longest ACE row of the last ACE row build
   int n_stale_bad;    // atoms whose CSP the rows of an earlier build cannot decide (stale rows)
-  int n_ace_groups;   // cell groups with queued atoms (ACE row build)
   int queue_dup;      // 1: the caller's queue is not strictly ascending (an atom may stand in it twice)
   int n_det1;         // detected atoms the lambda spread's second pass visits
   unsigned long long row_total;   // ap_neighbor_total's result
@@ -147,6 +147,7 @@ struct AceTables {
   std::vector<double> nu3_coef;
   // second coefficient set phi^(2) of the Finnis-Sinclair form (zeros unless ace_fs_on)
   std::vector<double> c1b, m2b, nu3_coef2;
+  std::vector<float> nu3_f32;   // nu3_coef and nu3_coef2 in FP32, one after the other
 };
 void build_ace_tables(const ap_config& cfg, AceTables& t);
 
@@ -347,6 +348,7 @@ namespace ap {
 size_t scan_tmp_bytes(int n);
 // d_out has n+1 entries; returns the number of kernels launched
 int scan_exclusive(const int* d_in, int* d_out, int n, int* d_tmp, cudaStream_t s);
+// cells, cell-relative shadows, and the shadows kept for the displacement check (now 0)
 void launch_bin(ap_ctx* c, const double* d_x, const int32_t* d_species, cudaStream_t s);
 void launch_cell_sort(ap_ctx* c, cudaStream_t s);
 void launch_shadow(ap_ctx* c, const double* d_x, cudaStream_t s);

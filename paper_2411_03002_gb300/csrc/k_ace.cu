@@ -841,27 +841,35 @@ __global__ void __launch_bounds__(kWarps3<R> * 32, sizeof(R) == 4 ? AP_ACE3_MINB
   }
 }
 
-__global__ void k_ace_finalize32(int n, const float4* __restrict__ acc, double* __restrict__ f) {
+// The accumulated ACE forces join f and the accumulators are cleared for the next evaluation
+// (most atoms have no precise atom in reach and need neither).
+__global__ void k_ace_finalize32(int n, float4* __restrict__ acc, double* __restrict__ f) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   float4 v = acc[i];
-  if (v.x == 0.f && v.y == 0.f && v.z == 0.f) return;   // no precise atom in reach (most atoms)
+  if (v.x == 0.f && v.y == 0.f && v.z == 0.f) return;
+  acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
   f[3 * i + 0] += (double)v.x;
   f[3 * i + 1] += (double)v.y;
   f[3 * i + 2] += (double)v.z;
 }
 
-__global__ void k_ace_finalize_fix(int n, const unsigned long long* __restrict__ acc, double* __restrict__ f) {
+__global__ void k_ace_finalize_fix(int n, unsigned long long* __restrict__ acc, double* __restrict__ f) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= 3 * n) return;
   const long long v = (long long)acc[i];
-  if (v != 0) f[i] += (double)v * (1.0 / kFixScale);
+  if (v == 0) return;
+  acc[i] = 0;
+  f[i] += (double)v * (1.0 / kFixScale);
 }
 
-__global__ void k_ace_finalize64(int n, const double* __restrict__ acc, double* __restrict__ f) {
+__global__ void k_ace_finalize64(int n, double* __restrict__ acc, double* __restrict__ f) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= 3 * n) return;
-  f[i] += acc[i];
+  const double v = acc[i];
+  if (v == 0.0) return;
+  acc[i] = 0.0;
+  f[i] += v;
 }
 
 template <typename R>
@@ -965,15 +973,6 @@ void run_ace(ap_ctx* c, const double* d_lam, const double* d_wgt, const int* d_q
                        : (fs ? k_ace_adjoint<R, true, 32> : k_ace_adjoint<R, false, 32>);
   int& r3 = b3[pi][lanes == 8][fs];
   if (forces && !r3) r3 = resident_blocks(k3, kWarps3<R> * 32, s3);
-  if (forces) {
-    if (a.faccfix)
-      cudaMemsetAsync(c->d_faccfix, 0, sizeof(unsigned long long) * 3 * (size_t)c->n, s);
-    else if constexpr (sizeof(R) == 4)
-      cudaMemsetAsync(c->d_facc32, 0, sizeof(float4) * (size_t)c->n, s);
-    else
-      cudaMemsetAsync(c->d_facc64, 0, sizeof(double) * 3 * (size_t)c->n, s);
-  }
-  cudaMemsetAsync(a.counter, 0, 2 * sizeof(int), s);   // work_counter and work_counter2
   const int tb = prof_mark(c, s);
   k_ace_basis<R><<<persistent_grid(c->num_sms, b1[pi], kWarps<R>, m), kWarps<R> * 32, s1, s>>>(a);
   prof_add(c, AP_PHASE_ACE_BASIS, tb, prof_mark(c, s));

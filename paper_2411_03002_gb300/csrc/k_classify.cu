@@ -668,9 +668,12 @@ __device__ inline double ring_mean(const double* __restrict__ hist, int ns, int 
 __global__ void k_lambda0(int n, const uint8_t* __restrict__ ch, const double* __restrict__ csp,
                           double* __restrict__ hist, int ns, int pos, int fill, double csp_lo, double csp_hi,
                           int mode, double* __restrict__ csp_avg, double* __restrict__ lam0,
-                          double* __restrict__ lam_min, int* __restrict__ flag) {
+                          double* __restrict__ lam_min, int* __restrict__ flag, float* __restrict__ vmin_f,
+                          int* __restrict__ n_det1) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) *n_det1 = 0;   // for the spread that follows
   if (i >= n) return;
+  vmin_f[i] = 3.4e38f;       // the FP32 minima of the spread start above any estimate
   double c = csp[i];
   if (fill) {
     for (int q = 0; q < ns; ++q) hist[(size_t)q * n + i] = c;
@@ -946,7 +949,8 @@ void launch_csp(ap_ctx* c, const double* d_x, const uint8_t* d_ch, cudaStream_t 
   double rs2 = r * r;
   const int* off = c->stored_off ? c->d_off_eam : nullptr;
   int* n_slow = &c->d_sc->n_csp_slow;
-  cudaMemsetAsync(n_slow, 0, sizeof(int), s);
+  // n_csp_slow, n_csp_list and, for rows older than the positions, n_stale_bad
+  cudaMemsetAsync(n_slow, 0, (stale_disp > 0.0 ? 3 : 2) * sizeof(int), s);
   // Rows older than the positions: stale2 = the radius inside which they are complete.
   // The build's split still bounds the skin part from below: its entries were beyond r_c
   // at the build and are now beyond r_c - 2 m, the radius the in-range part is tested
@@ -957,7 +961,6 @@ void launch_csp(ap_ctx* c, const double* d_x, const uint8_t* d_ch, cudaStream_t 
   if (stale_disp > 0.0) {
     const double rin = r - 2.0 * stale_disp;
     stale2 = rin > 0.0 ? (float)(rin * rin) : 1e-30f;
-    cudaMemsetAsync(&c->d_sc->n_stale_bad, 0, sizeof(int), s);
     const double rp = std::sqrt((double)c->split_rpf2) - 2.0 * stale_disp;
     nin = c->d_split_eam;
     rpf2 = rp > 0.0 ? (float)(rp * rp) : 0.f;
@@ -989,7 +992,6 @@ void launch_csp(ap_ctx* c, const double* d_x, const uint8_t* d_ch, cudaStream_t 
     return;
   }
   int* n_list = &c->d_sc->n_csp_list;
-  cudaMemsetAsync(n_list, 0, sizeof(int), s);
   k_csp_near<<<nblk(c->n, 128), 128, 0, s>>>(A, c->d_csp_slow, n_list);
   // the handed-over atoms, grid-stride over the device-side counts; d_det1 is free until the spread
   if (c->n > kSortFrom) k_csp_sort<<<c->num_sms * 4, 128, 0, s>>>(A, c->d_csp_slow, n_list, c->d_det1, n_slow);
@@ -1005,7 +1007,8 @@ void launch_lambda0(ap_ctx* c, const uint8_t* d_ch, const double* d_score, doubl
   int pos = fill ? 0 : (c->csp_pos + 1) % ns;
   c->csp_pos = pos;
   k_lambda0<<<nblk(c->n, 256), 256, 0, s>>>((int)c->n, d_ch, d_score, c->d_csp_hist, ns, pos, fill, lo, hi,
-                                            c->cfg.fcut_mode, c->d_csp_avg, c->d_lam0, c->d_lam_min, c->d_flag);
+                                            c->cfg.fcut_mode, c->d_csp_avg, c->d_lam0, c->d_lam_min, c->d_flag,
+                                            c->d_vmin_f, &c->d_sc->n_det1);
   c->kernels += 2 + scan_exclusive(c->d_flag, c->d_scan, (int)c->n, c->d_scan_tmp, s);
   k_compact<<<nblk(c->n, 256), 256, 0, s>>>((int)c->n, c->d_flag, c->d_scan, c->d_detected, &c->d_sc->n_detected,
                                             nullptr);
@@ -1015,9 +1018,6 @@ void launch_spread(ap_ctx* c, const double* d_x, const uint8_t* d_ch, cudaStream
   int grid = c->num_sms * 8;
   const int* st = c->cells_stale ? c->sten_spread_stale : c->sten_spread;
   const float margin = c->cells_stale ? (float)c->stale_m : 0.f;
-  // +3.4e38 in every float: the FP32 minima start above any estimate
-  cudaMemsetAsync(c->d_vmin_f, 0x7f, sizeof(float) * (size_t)c->n, s);
-  cudaMemsetAsync(&c->d_sc->n_det1, 0, sizeof(int), s);
   k_spread<0><<<grid, kSpreadWarps * 32, 0, s>>>(c->d_detected, &c->d_sc->n_detected, d_x, d_ch, c->d_sys,
                                                  c->d_atom_sys, c->d_sh32, c->d_cunw, c->d_cell_start,
                                                  c->d_cell_atoms, c->d_lam0, c->cfg.r_lo, c->cfg.r_hi,

@@ -85,11 +85,18 @@ __device__ inline const SysInfo& sys_of(const SysInfo* sys, const int* atom_sys,
 }
 
 // ------------------------------------------------------------------ binning
+// Cell of every atom, its shadow (the k_shadow arithmetic) and the copy of it that the
+// displacement since this build is taken from.
 __global__ void k_bin(int n, const double* __restrict__ x, const int32_t* __restrict__ species,
                       const SysInfo* __restrict__ sys, const int* __restrict__ atom_sys, int* __restrict__ cell,
                       int* __restrict__ slot, int4* __restrict__ cunw, int* __restrict__ cell_count,
-                      DevScalars* sc) {
+                      const double* __restrict__ org, float4* __restrict__ s32, double4_32a* __restrict__ s64,
+                      float4* __restrict__ s32b, DevScalars* sc) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) {
+    sc->max_disp2_bits = 0;
+    sc->max_dispa2_bits = 0x7f7f7f7fu;   // the ACE rows' reference shadows belong to the old cells: until the next ACE build
+  }
   if (i >= n) return;
   const SysInfo& S = sys_of(sys, atom_sys, i);
   int cw[3], cu[3];
@@ -129,8 +136,16 @@ __global__ void k_bin(int n, const double* __restrict__ x, const int32_t* __rest
   if (bad) atomicOr(&sc->err, bad);
   int id = S.cell_base + (cw[2] * S.nc[1] + cw[1]) * S.nc[0] + cw[0];
   cell[i] = id;
-  cunw[i] = make_int4(cu[0], cu[1], cu[2], pack_cell(cw[0], cw[1], cw[2]));
+  const int4 c4 = make_int4(cu[0], cu[1], cu[2], pack_cell(cw[0], cw[1], cw[2]));
+  cunw[i] = c4;
   slot[i] = atomicAdd(&cell_count[id], 1);
+  const double xi[3] = {x[3 * i + 0], x[3 * i + 1], x[3 * i + 2]};
+  double sh[3];
+  cell_shadow(S, org, c4, xi, sh);
+  const float4 s4 = make_float4((float)sh[0], (float)sh[1], (float)sh[2], __int_as_float(c4.w));
+  s32[i] = s4;
+  s32b[i] = s4;
+  if (s64) s64[i] = make_double4_32a(sh[0], sh[1], sh[2], (double)c4.w);
 }
 
 __global__ void k_cell_scatter(int n, const int* __restrict__ cell, const int* __restrict__ slot,
@@ -831,7 +846,8 @@ void launch_wrap_positions(ap_ctx* c, double* d_x, cudaStream_t s) {
 void launch_bin(ap_ctx* c, const double* d_x, const int32_t* d_species, cudaStream_t s) {
   cudaMemsetAsync(c->d_cell_count, 0, sizeof(int) * (size_t)c->n_cells, s);
   k_bin<<<nblk(c->n, 256), 256, 0, s>>>((int)c->n, d_x, d_species, c->d_sys, c->d_atom_sys, c->d_cell, c->d_slot,
-                                        c->d_cunw, c->d_cell_count, c->d_sc);
+                                        c->d_cunw, c->d_cell_count, c->d_org, c->d_sh32,
+                                        c->cfg.precision == AP_PREC_FP64 ? c->d_sh64 : nullptr, c->d_sh32b, c->d_sc);
   c->kernels += 1;
 }
 
@@ -936,9 +952,8 @@ void launch_build_ace(ap_ctx* c, const double* d_x, const int* d_queue, const in
   if (m >= 400 * c->num_sms && unique && runs <= kBuildWarps * 32) {
     int* flag = c->d_cell_count;   // free after the cell sort; n_groups <= n_cells
     int* list = c->d_slot;         // free after the cell sort; at most one group per atom
-    int* n_list = &c->d_sc->n_ace_groups;
+    int* n_list = &c->d_sc->n_ace_groups;   // cleared by build_ace_checked
     cudaMemsetAsync(flag, 0, sizeof(int) * (size_t)c->n_groups, s);
-    cudaMemsetAsync(n_list, 0, sizeof(int), s);
     cudaMemsetAsync(c->d_qpos, 0xff, sizeof(int) * (size_t)c->n, s);
     k_queue_groups<<<c->num_sms * 4, 256, 0, s>>>(d_queue, d_nq, c->d_sys, c->d_atom_sys, c->d_cunw, c->build_group,
                                                   c->d_qpos, flag, list, n_list);
