@@ -355,7 +355,7 @@ ap_status build_checked(ap_ctx* c, const double* d_x, const int32_t* d_species, 
     if (st) return st;
     int e = c->h_sc->err;
     if ((e & kErrCapacity) && attempt == 0 && c->cfg.cap_eam == 0) {
-      c->cap_eam = c->h_sc->need_eam + 16;
+      c->cap_eam = (c->h_sc->need_eam + 19) & ~3;   // rows stay on 16-byte boundaries (row4)
       st = alloc_rows(c, true, false);
       if (st) return st;
       continue;

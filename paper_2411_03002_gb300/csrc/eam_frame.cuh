@@ -130,6 +130,18 @@ struct Frame {
   }
 };
 
+// Entries t .. t + 3 of a row (VEC: rows start on 16-byte boundaries, so one load; a thread that
+// reads its own row entry by entry costs the L1 one line per lane and entry: k_csp_near on
+// 4,000,000 atoms 1.98 -> 1.44 ms, k_sel_features and k_sel_rho on 130,944 atoms 223 -> 168 us).
+// The EAM passes, whose four lanes share a row, are faster with single entries (0.88 against
+// 0.96 ms for the density pass): their gathers are what counts.
+template <bool VEC>
+__device__ inline int4 row4(const int* __restrict__ row, int t, int c) {
+  if constexpr (VEC) return *reinterpret_cast<const int4*>(row + t);
+  return make_int4(row[t], t + 1 < c ? row[t + 1] : 0, t + 2 < c ? row[t + 2] : 0, t + 3 < c ? row[t + 3] : 0);
+}
+__device__ inline int pick(const int4& v, int u) { return u == 0 ? v.x : u == 1 ? v.y : u == 2 ? v.z : v.w; }
+
 template <typename T, int G>
 __device__ inline T group_sum(T v) {
 #pragma unroll

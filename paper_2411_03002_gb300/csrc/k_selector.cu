@@ -36,7 +36,7 @@ constexpr float kCspCap = 100.f;
 constexpr int kS2Max = 24;
 
 // ------------------------------------------------------------------ density pre-pass
-template <bool STORED>
+template <bool STORED, bool VEC>
 __global__ void __launch_bounds__(128) k_sel_rho(int n, const SysInfo* __restrict__ sys,
                                                  const int* __restrict__ atom_sys, const float4* __restrict__ sh,
                                                  const int* __restrict__ nbr, const int* __restrict__ off,
@@ -50,8 +50,11 @@ __global__ void __launch_bounds__(128) k_sel_rho(int n, const SysInfo* __restric
   const size_t row = (size_t)i * cap;
   const float rf2 = kRFeat * kRFeat;
   float rho = 0.f;
+  int4 jj;
+#pragma unroll 4
   for (int t = 0; t < c; ++t) {
-    const int j = nbr[row + t];
+    if ((t & 3) == 0) jj = row4<VEC>(nbr + row, t, c);
+    const int j = pick(jj, t & 3);
     float d[3];
     fr.disp(sh[j], off, row + t, d);
     const float r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
@@ -68,7 +71,7 @@ __global__ void __launch_bounds__(128) k_sel_rho(int n, const SysInfo* __restric
 }
 
 // ------------------------------------------------------------------ features
-template <bool STORED>
+template <bool STORED, bool VEC>
 __global__ void __launch_bounds__(128) k_sel_features(int n, const SysInfo* __restrict__ sys,
                                                       const int* __restrict__ atom_sys,
                                                       const float4* __restrict__ sh, const int* __restrict__ nbr,
@@ -88,8 +91,11 @@ __global__ void __launch_bounds__(128) k_sel_features(int n, const SysInfo* __re
   float v1[3] = {0.f, 0.f, 0.f}, v2[3] = {0.f, 0.f, 0.f}, va[3] = {0.f, 0.f, 0.f}, gz[3] = {0.f, 0.f, 0.f};
   int n_all = 0, n1 = 0, n2 = 0, n3 = 0;
   float s2v[kS2Max][3];
+  int4 jj;
+#pragma unroll 4
   for (int t = 0; t < c; ++t) {
-    const int j = nbr[row + t];
+    if ((t & 3) == 0) jj = row4<VEC>(nbr + row, t, c);
+    const int j = pick(jj, t & 3);
     float d[3];
     fr.disp(sh[j], off, row + t, d);
     const float r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
@@ -145,8 +151,10 @@ __global__ void __launch_bounds__(128) k_sel_features(int n, const SysInfo* __re
   const float mean = n_all ? sum_r / (float)n_all : 0.f;
   const float mean1 = n1 ? sum_r1 / (float)n1 : 0.f;
   float m2 = 0.f, m3 = 0.f, m4 = 0.f, m21 = 0.f;
+#pragma unroll 4
   for (int t = 0; t < c; ++t) {
-    const int j = nbr[row + t];
+    if ((t & 3) == 0) jj = row4<VEC>(nbr + row, t, c);
+    const int j = pick(jj, t & 3);
     float d[3];
     fr.disp(sh[j], off, row + t, d);
     const float r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
@@ -805,19 +813,15 @@ void launch_sel_features(ap_ctx* c, float* d_feat, cudaStream_t s) {
   if (n <= 0) return;
   EamP<float> p = make_params<float>(c->cfg);
   const int* off = c->stored_off ? c->d_off_eam : nullptr;
-  if (c->stored_off) {
-    k_sel_rho<true><<<nblk(n, 128), 128, 0, s>>>(n, c->d_sys, c->d_atom_sys, c->d_sh32, c->d_nbr_eam, off,
-                                                   c->d_cnt_eam, c->cap_eam, p, c->d_sel_rho);
-    k_sel_features<true><<<nblk(n, 128), 128, 0, s>>>(n, c->d_sys, c->d_atom_sys, c->d_sh32, c->d_nbr_eam, off,
-                                                        c->d_cnt_eam, c->cap_eam, p, c->d_sel_rho, c->d_csp,
-                                                        d_feat);
-  } else {
-    k_sel_rho<false><<<nblk(n, 128), 128, 0, s>>>(n, c->d_sys, c->d_atom_sys, c->d_sh32, c->d_nbr_eam, off,
-                                                    c->d_cnt_eam, c->cap_eam, p, c->d_sel_rho);
-    k_sel_features<false><<<nblk(n, 128), 128, 0, s>>>(n, c->d_sys, c->d_atom_sys, c->d_sh32, c->d_nbr_eam, off,
-                                                         c->d_cnt_eam, c->cap_eam, p, c->d_sel_rho, c->d_csp,
-                                                         d_feat);
-  }
+  const bool vec = c->cap_eam % 4 == 0;
+  auto rho = c->stored_off ? (vec ? k_sel_rho<true, true> : k_sel_rho<true, false>)
+                           : (vec ? k_sel_rho<false, true> : k_sel_rho<false, false>);
+  auto features = c->stored_off ? (vec ? k_sel_features<true, true> : k_sel_features<true, false>)
+                                : (vec ? k_sel_features<false, true> : k_sel_features<false, false>);
+  rho<<<nblk(n, 128), 128, 0, s>>>(n, c->d_sys, c->d_atom_sys, c->d_sh32, c->d_nbr_eam, off, c->d_cnt_eam, c->cap_eam, p,
+                                   c->d_sel_rho);
+  features<<<nblk(n, 128), 128, 0, s>>>(n, c->d_sys, c->d_atom_sys, c->d_sh32, c->d_nbr_eam, off, c->d_cnt_eam,
+                                        c->cap_eam, p, c->d_sel_rho, c->d_csp, d_feat);
   c->kernels += 2;
 }
 
