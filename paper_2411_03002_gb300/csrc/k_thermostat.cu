@@ -164,13 +164,14 @@ __device__ inline bool member(const int* __restrict__ row, int t, int i, const u
 }
 
 // One warp per cell of one colour; the corrections of a cell form a serial chain (each needs
-// the velocities that the last one left), so the latency of one correction is the cost.  The
-// members (row entry, mass) of the next atom are loaded while the current one is corrected,
-// each lane keeps up to kMem members' velocities in registers between the three sums, and
-// what is no member carries mass 0 at index i.  Rows beyond 32 kMem entries take the loop over
-// memory.  10 MD steps with one update of a 358,012-atom slab, a few hundred corrections a
-// cell: 170 -> 23.4 ms (the membership test over the whole row, for boxes that cannot need it,
-// was most of it).
+// the velocities that the last one left), so the latency of one correction is the cost.  Each
+// lane keeps up to kMem members' velocities in registers between the three sums, what is no
+// member carries mass 0 at index i, and what the chain needs of the coming atoms is loaded one
+// turn ahead (three turns of indices).  Rows beyond 32 kMem entries take the loop over memory.
+// 10 MD steps with one update of a 358,012-atom slab, a few hundred corrections a cell: 154 ms
+// with a membership test over the whole row for boxes that cannot need it, 19.9 ms without, 17.5
+// with the loads ahead; what is left is the FP64 chain of two divisions, a square root and
+// 11 dependent additions.
 constexpr int kMem = 6;   // 192 row entries: the default row capacity is 160
 template <bool DEDUP>
 __global__ void __launch_bounds__(32) k_th_rescale(
@@ -185,64 +186,83 @@ __global__ void __launch_bounds__(32) k_th_rescale(
   const int cx = 2 * (w % mx) + px, cy = 2 * ((w / mx) % my) + py, cz = 2 * (w / (mx * my)) + pz;
   const int cell = (cz * T.nc[1] + cy) * T.nc[0] + cx;
   const int a_end = start[cell + 1];
-  int a = start[cell];
-  if (a >= a_end) return;
+  const int a0 = start[cell];
+  if (a0 >= a_end) return;
   unsigned long long n_ok = 0, n_bad = 0;
   double e_sum = 0.0;
-  int i_n = atoms[a], c_n = cnt[i_n];
-  int j_n[kMem];
-  double m_n[kMem];
-  auto fetch = [&](int i, int c) {
-    const int* row = nbr + (size_t)i * cap;
+  // What the chain needs of the coming atoms is loaded a turn before it is used, without branches
+  // on loaded values: the atom of turn a + 4, the row length of a + 3, the row entries of a + 2,
+  // masses, fixed flags and Delta E of a + 1.
+  int i4 = -1, i3 = -1, c3 = 0, i2 = -1, c2 = 0, i1 = -1, c1 = 0;
+  int j2[kMem], j1[kMem];
+  double m1[kMem], de1 = 0.0;
+  unsigned f1[kMem];
 #pragma unroll
-    for (int u = 0; u < kMem; ++u) {
-      const int t = lane + 32 * u;
-      j_n[u] = i;
-      m_n[u] = 0.0;
-      if (t < c && member<DEDUP>(row, t, i, fixed)) {
-        j_n[u] = row[t];
-        m_n[u] = mass[j_n[u]];
-      }
-    }
-  };
-  if (c_n <= 32 * kMem) fetch(i_n, c_n);
-  for (; a < a_end; ++a) {
-    const int i = i_n, c = c_n;
-    const double de = dE[i];
+  for (int u = 0; u < kMem; ++u) {
+    j2[u] = j1[u] = -1;
+    m1[u] = 0.0;
+    f1[u] = 0;
+  }
+  for (int a = a0 - 4; a < a_end; ++a) {
+    const int i = i1, c = c1;
+    const double de = de1;
     const bool in_regs = c <= 32 * kMem;
     int j[kMem];
     double m[kMem], ux[kMem], uy[kMem], uz[kMem];
-    const int* row = nbr + (size_t)i * cap;
-    // total mass and momentum of Omega_i (atom i itself in lane 0)
-    double sm = 0.0, spx = 0.0, spy = 0.0, spz = 0.0, mi = 0.0, vx = 0.0, vy = 0.0, vz = 0.0;
-    if (lane == 0) {
-      mi = mass[i];
-      vx = v[3 * i];
-      vy = v[3 * i + 1];
-      vz = v[3 * i + 2];
-      sm = mi;
-      spx = mi * vx;
-      spy = mi * vy;
-      spz = mi * vz;
-    }
-    if (in_regs) {
+    double vx = 0.0, vy = 0.0, vz = 0.0, mi = 0.0;
+    if (a >= a0 && in_regs) {
 #pragma unroll
       for (int u = 0; u < kMem; ++u) {
-        j[u] = j_n[u];
-        m[u] = m_n[u];
+        const int t = lane + 32 * u;
+        bool is = t < c && j1[u] != i && f1[u] == 0;
+        if constexpr (DEDUP) is = is && member<DEDUP>(nbr + (size_t)i * cap, t, i, fixed);
+        j[u] = is ? j1[u] : i;
+        m[u] = is ? m1[u] : 0.0;
         ux[u] = uy[u] = uz[u] = 0.0;
-        if (m[u] != 0.0) {
+        if (is) {
           ux[u] = v[3 * j[u]];
           uy[u] = v[3 * j[u] + 1];
           uz[u] = v[3 * j[u] + 2];
         }
       }
     }
-    if (a + 1 < a_end) {   // the next atom's members do not depend on this correction
-      i_n = atoms[a + 1];
-      c_n = cnt[i_n];
-      if (c_n <= 32 * kMem) fetch(i_n, c_n);
+    if (a >= a0 && lane == 0) {
+      mi = mass[i];
+      vx = v[3 * i];
+      vy = v[3 * i + 1];
+      vz = v[3 * i + 2];
     }
+    // turn a + 1: the row entries have arrived
+    i1 = i2;
+    c1 = c2;
+    if (i1 >= 0) {
+      de1 = dE[i1];
+#pragma unroll
+      for (int u = 0; u < kMem; ++u) {
+        const bool in = lane + 32 * u < c1;
+        j1[u] = j2[u];
+        m1[u] = in ? mass[j2[u]] : 0.0;
+        f1[u] = in && fixed ? fixed[j2[u]] : 0u;
+      }
+    }
+    // turn a + 2: its row; turn a + 3: its length; turn a + 4: the atom
+    i2 = i3;
+    c2 = c3;
+    if (i2 >= 0) {
+      const int* row2 = nbr + (size_t)i2 * cap;
+#pragma unroll
+      for (int u = 0; u < kMem; ++u) {
+        const int t = lane + 32 * u;
+        j2[u] = t < c2 && c2 <= 32 * kMem ? row2[t] : i2;
+      }
+    }
+    i3 = i4;
+    c3 = i3 >= 0 ? cnt[i3] : 0;
+    i4 = a + 4 < a_end && a + 4 >= a0 ? atoms[a + 4] : -1;
+    if (a < a0) continue;
+    const int* row = nbr + (size_t)i * cap;
+    // total mass and momentum of Omega_i (atom i itself in lane 0)
+    double sm = mi, spx = mi * vx, spy = mi * vy, spz = mi * vz;
     if (in_regs) {
 #pragma unroll
       for (int u = 0; u < kMem; ++u) {
