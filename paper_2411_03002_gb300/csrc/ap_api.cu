@@ -971,11 +971,12 @@ ap_status ap_step(ap_ctx* c, int64_t n, double* d_x, double* d_v, double* d_f, c
     PhaseTimer t(c, s, AP_PHASE_OTHER);
     launch_vscale(c, d_mass, s);   // the half-kick factors of this call's masses
   }
+  bool finish = false;   // the step before left its ACE forces, indenter and second kick to the next drift
   for (int64_t k = 0; k < nsteps; ++k) {
     c->step++;
     {
       PhaseTimer t(c, s, AP_PHASE_OTHER);
-      launch_vv_first(c, d_x, d_v, d_f, d_mass, d_fixed, s);
+      launch_vv_first(c, d_x, d_v, d_f, d_mass, d_fixed, finish, (c->step - 1) * g.dt, s);
     }
     const bool lam_step = c->step % g.lambda_every == 0;
     bool build = false, keep = false, ace_only = false;
@@ -1080,6 +1081,8 @@ ap_status ap_step(ap_ctx* c, int64_t n, double* d_x, double* d_v, double* d_f, c
       PhaseTimer t(c, s, AP_PHASE_ACE);
       launch_ace(c, c->d_lam_int, c->d_precise, c->d_eprec, true, s);
     }
+    finish = k + 1 < nsteps && !(lam_step && thermo);
+    if (finish) continue;
     {
       PhaseTimer t(c, s, AP_PHASE_OTHER);
       launch_ace_finalize(c, d_f, s);

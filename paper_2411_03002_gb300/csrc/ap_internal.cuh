@@ -77,6 +77,9 @@ __device__ inline int wrap_off(int dc, int nc, int periodic) {
   return dc;
 }
 
+// Fixed-point ACE forces (ace_deterministic): multiples of 2^-36 eV/A.
+constexpr double kFixScale = 68719476736.0;
+
 // ------------------------------------------------------------------ error bits
 enum : int {
   kErrCapacity = 1 << AP_ERR_CAPACITY,
@@ -411,8 +414,10 @@ void launch_th_correct(ap_ctx* c, const int* d_q, const int* d_m, const double* 
 
 // k_md.cu
 void launch_vscale(ap_ctx* c, const double* d_mass, cudaStream_t s);
-void launch_vv_first(ap_ctx* c, double* d_x, double* d_v, const double* d_f, const double* d_mass,
-                     const uint8_t* d_fixed, cudaStream_t s);
+// finish: the forces in d_f lack the ACE accumulators and the indenter (at time t_ind), and the
+// velocities the second half kick of the step before; the kernel adds all three first.
+void launch_vv_first(ap_ctx* c, double* d_x, double* d_v, double* d_f, const double* d_mass, const uint8_t* d_fixed,
+                     bool finish, double t_ind, cudaStream_t s);
 void launch_vv_second(ap_ctx* c, double* d_v, const double* d_f, const double* d_mass, const uint8_t* d_fixed,
                       cudaStream_t s);
 void launch_indenter(ap_ctx* c, const double* d_x, double* d_f, double t, cudaStream_t s);

@@ -161,7 +161,6 @@ __device__ inline void pair_disp(const SysInfo& S, const typename V<R>::S4& si, 
 
 // Fixed-point force accumulation (ace_deterministic): contributions rounded to multiples
 // of 2^-36 eV/A, summed with exact, order-independent 64-bit integer atomics.
-constexpr double kFixScale = 68719476736.0;   // 2^36
 __device__ inline unsigned long long to_fix(double v) { return (unsigned long long)llrint(v * kFixScale); }
 
 template <typename R>
