@@ -286,6 +286,7 @@ ap_status ensure_capacity(ap_ctx* c, int64_t n) {
     CK(dalloc(c->d_faccfix, 3 * m));
     CK(cudaMemset(c->d_faccfix, 0, sizeof(unsigned long long) * 3 * (size_t)m));
   }
+  CK(cudaDeviceSynchronize());   // the clears are done before work on any stream
   CK(dalloc(c->d_efast, m));
   CK(dalloc(c->d_eprec, m));
   CK(dalloc(c->d_eatom, m));
@@ -649,6 +650,7 @@ ap_status ap_create(const ap_config* h_cfg, ap_ctx** out) {
   e = cudaMalloc(&c->d_sc, sizeof(DevScalars));
   if (e == cudaSuccess) e = cudaMallocHost(&c->h_sc, sizeof(DevScalars));
   if (e == cudaSuccess) e = cudaMemset(c->d_sc, 0, sizeof(DevScalars));
+  if (e == cudaSuccess) e = cudaDeviceSynchronize();   // before work on any stream
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {
     ap_destroy(c);
