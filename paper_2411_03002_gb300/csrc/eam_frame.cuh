@@ -77,6 +77,8 @@ struct Frame {
   int nx, ny, nz;
   int halfx, halfy, halfz;   // nc/2 in periodic dimensions, a huge value otherwise
   R sx, sy, sz;
+  int base;     // w_j - base = the cell offset + 4 in each 10-bit field, where nothing wraps
+  bool inner;   // no neighbour's cell lies across a periodic boundary
 
   template <typename S4>
   __device__ inline Frame(const SysInfo& S, const S4& si) {
@@ -102,6 +104,10 @@ struct Frame {
     sx = si.x;
     sy = si.y;
     sz = si.z;
+    base = w - pack_cell(4, 4, 4);
+    inner = (!S.periodic[0] || (cx >= kStencil && cx < nx - kStencil)) &&
+            (!S.periodic[1] || (cy >= kStencil && cy < ny - kStencil)) &&
+            (!S.periodic[2] || (cz >= kStencil && cz < nz - kStencil));
   }
 
   __device__ static inline int unwrap(int d, int n, int half) {
@@ -110,7 +116,8 @@ struct Frame {
     return d;
   }
 
-  template <typename S4>
+  // INNER: the atom is `inner` (its neighbours' cells, at most kStencil away, need no unwrapping)
+  template <bool INNER = false, typename S4>
   __device__ inline void disp(const S4& sj, const int* __restrict__ off, size_t e, R d[3]) const {
     int kx, ky, kz;
     if constexpr (STORED) {
@@ -118,6 +125,11 @@ struct Frame {
       kx = off_x(p);
       ky = off_y(p);
       kz = off_z(p);
+    } else if constexpr (INNER) {
+      const int t = Shadow<R>::code(sj) - base;
+      kx = cell_x(t) - 4;
+      ky = cell_y(t) - 4;
+      kz = cell_z(t) - 4;
     } else {
       int w = Shadow<R>::code(sj);
       kx = unwrap(cell_x(w) - cx, nx, halfx);
@@ -178,13 +190,15 @@ __device__ inline double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 //   zeta(r)                        density contribution,
 //   pair(r, dzeta, phi, dphi)      zeta'(r), Phi(r), Phi'(r),
 //   embed(rho, xi, dxi)            xi(rho), xi'(rho),
-// and kMinBlocks, the resident 256-thread blocks per SM its FP32 kernels are
-// compiled for (the register budget).
+// kMinBlocks, the resident 256-thread blocks per SM its FP32 kernels are compiled for
+// (the register budget), and kInnerForce, whether its FP32 force pass has a second walk for
+// atoms away from periodic boundaries.
 // PotSynth: the analytic synthetic EAM (zeta = exp(-beta (r/r0 - 1)) psi, Phi = Morse psi,
 // xi = -A sqrt(rho)).  PotMishin: the Mishin EAM2 forms of Appendix E.
 template <typename R>
 struct PotSynth {
   static constexpr int kMinBlocks = AP_EAM_MINB;
+  static constexpr bool kInnerForce = true;
   EamP<R> p;
   R rc2;
   __device__ inline R zeta(R r) const {
@@ -237,6 +251,7 @@ struct PotSynth {
 template <typename R>
 struct PotMishin {
   static constexpr int kMinBlocks = 4;   // <= 64 registers: the compensated terms fit unspilled
+  static constexpr bool kInnerForce = false;
   R E1, E2, delta, F0, xi0, xi2, inv_h, q1, q2, q3, q4, Q1, Q2, S1, S2, S3, a, a1, a2, b1, b2, r01, r02, r03, r04,
       rs1, rs2, rs3, rc;
   R E1l, E2l, a1l, a2l, r01l, r02l;      // low parts of the Morse constants
