@@ -39,17 +39,17 @@ METRIC = "atom-steps/s adaptive vs full-ACE on 1 GB300 at <=10 meV/A force error
 # The step's three largest kernels are instrumented (CUDA events around each launch);
 # `roofline` describes the one with the most measured time, `rooflines` all three.
 #
-# Algorithmic FLOPs of the ACE force stage k_ace_adjoint, per neighbour pair within r_c
-# and per precise atom (FMA = 2): per pair the radial functions and derivatives (~100),
-# the solid harmonics and gradients for l <= 4 (~400), the two 8-term contractions and
-# the accumulations for 25 (l, m) (~1040) and the scatter (~40); per atom
-# u = W^T dE/dA / N0 (~3300).
-ADJ_FLOP_PER_PAIR = 1580
+# FLOPs of the ACE force stage k_ace_adjoint, per neighbour pair within r_c and per precise
+# atom (FMA = 2): per pair T_k and T'_k (~28), the two contractions with u of 7 + 6 FMAs for 25
+# (l, m) (650), the sums over l per m (~82), value and gradient from them (~82), the
+# harmonics' factors (~35), cutoff, projection and scatter (~55); per atom u = W^T dE/dA / N0
+# (~3300).
+ADJ_FLOP_PER_PAIR = 930
 ADJ_FLOP_PER_ATOM = 3300
-# Algorithmic FLOPs of k_ace_basis: per pair g (~30), Y (~70), the normalisation (~10)
-# and the G = g^T Y accumulation over 8 x 25 (l, m, k) (400); per atom A = W G (3200)
-# and the nu = 1, 2 energy and gradient (~3800).
-BASIS_FLOP_PER_PAIR = 510
+# FLOPs of k_ace_basis: per pair g (~30), Y (~32), the normalisation (~10) and the G = g^T Y
+# accumulation over 8 x 25 (l, m, k) (400); per atom A = W G (3200) and the nu = 1, 2 energy
+# and gradient (~3800).
+BASIS_FLOP_PER_PAIR = 470
 BASIS_FLOP_PER_ATOM = 7000
 # The whole ACE evaluation (k_ace_basis + k_ace_nu3 + k_ace_adjoint): per atom add the
 # nu = 3 monomials (~11400).

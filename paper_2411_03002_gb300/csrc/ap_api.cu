@@ -649,14 +649,15 @@ ap_status ap_create(const ap_config* h_cfg, ap_ctx** out) {
   upload_ace_tables(c);
   e = cudaMalloc(&c->d_sc, sizeof(DevScalars));
   if (e == cudaSuccess) e = cudaMallocHost(&c->h_sc, sizeof(DevScalars));
-  if (e == cudaSuccess) e = cudaMemset(c->d_sc, 0, sizeof(DevScalars));
-  if (e == cudaSuccess) e = cudaDeviceSynchronize();   // before work on any stream
+  if (e == cudaSuccess) {   // a blocking copy: the scalars are 0 before work on any stream
+    std::memset(c->h_sc, 0, sizeof(DevScalars));
+    e = cudaMemcpy(c->d_sc, c->h_sc, sizeof(DevScalars), cudaMemcpyHostToDevice);
+  }
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {
     ap_destroy(c);
     return AP_ERR_CUDA;
   }
-  std::memset(c->h_sc, 0, sizeof(DevScalars));
   *out = c;
   return AP_OK;
 }

@@ -331,8 +331,8 @@ __device__ inline int build_row_warp(int i, const double* __restrict__ x, const 
 //     at a time, and keeps a bit per candidate and atom; a scan over the lanes' counts gives
 //     every accepted candidate its place in the row.
 // A thread per row walked all 560 candidates in one dependent chain and wrote 32 rows at once,
-// 4 bytes each: 999,180 atoms at 6.5 A 1.48 -> 1.30 ms, 32,000 atoms 206 -> 75 us, 237 atoms
-// 160 -> 25 us (the dependent chain was the cost there).  What binds it now is instruction
+// 4 bytes each: 999,180 atoms at 6.5 A 1.48 -> 1.28 ms, 32,000 atoms 206 -> 64 us, 237 atoms
+// 160 -> 13 us (the dependent chain was the cost there).  What binds it now is instruction
 // issue: the tests (about 35 % of the instructions) and the writes of the accepted entries.
 //
 // Row order: first the entries whose FP32 distance lies inside the potential cutoff
