@@ -441,6 +441,9 @@ __global__ void __launch_bounds__(kBuildWarps * 32, AP_BUILD_MINB)
   const int x0 = gid % gx * A.group, y0 = gid / gx % gy * A.group, z0 = gid / (gx * gy) * A.group;
   const int mx = min(A.group, nx - x0), my = min(A.group, ny - y0), mz = min(A.group, nz - z0);
   const float reach2 = A.rcf2 + A.band, r_sure = A.rcf2 - A.band;
+  // r_sure is rounded and may lie further from rcf2 than the guard band: the exact decision takes
+  // every pair that is not surely inside (the difference itself is exact)
+  const float band = fmaxf(A.band, A.rcf2 - r_sure);
   // this warp's cell of the group, or its share of the single cell's atoms
   const int parts = A.group == 1 ? kBuildWarps : 1, part = A.group == 1 ? warp : 0;
   const int wx = warp & 1, wy = (warp >> 1) & 1, wz = warp >> 2;
@@ -641,12 +644,12 @@ __global__ void __launch_bounds__(kBuildWarps * 32, AP_BUILD_MINB)
               const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
               const unsigned bit = r2 < A.rpf2 ? b_in : b_sk;
               if (r2 < r_sure) m[u] |= bit;
-              if (fabsf(r2 - A.rcf2) <= A.band || r2 < 1e-6f) {
+              if (fabsf(r2 - A.rcf2) <= band || r2 < 1e-6f) {
                 const int j = __float_as_int(p.w);
                 const int o = STORED ? s_cell[list[base + k]] - (pack_off(ux, uy, uz) - pack_off(0, 0, 0)) : 0;
                 if (r2 < 1e-6f && j == ci[u] && (!STORED || o == pack_off(0, 0, 0))) {
                   m[u] &= ~bit;   // the atom itself
-                } else if (fabsf(r2 - A.rcf2) <= A.band) {
+                } else if (fabsf(r2 - A.rcf2) <= band) {
                   m[u] &= ~bit;
                   if (decide(A, S, ci[u], j, o, STORED)) m[u] |= bit;
                 }
