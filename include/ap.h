@@ -361,6 +361,8 @@ ap_status ap_blend_forces(ap_ctx* ctx, int64_t n, const double* d_lam, const dou
  * error bits so far (an error ends the call), grows the EAM rows if one overflowed,
  * and reads the new precise queue's length to size the ACE storage for it.  With
  * rebuild_every = AP_REBUILD_SKIN it also synchronises after every drift.
+ * ap_classify and ap_eval_ace between two calls use the context's queue and ACE
+ * rows: the next call with nsteps > 0 rebuilds its own, and the lists, first.
  * Errors: as above plus AP_ERR_SKIN (an atom moved more than skin/2 before a
  * rebuild; never with AP_REBUILD_SKIN) and AP_ERR_NONFINITE. */
 ap_status ap_step(ap_ctx* ctx, int64_t n, double* d_x, double* d_v, double* d_f, const double* d_mass,

@@ -817,6 +817,7 @@ ap_status ap_classify(ap_ctx* c, int64_t n, const double* d_x, const uint8_t* d_
   }
   ap_status st = prep_detector(c);
   if (st) return st;
+  c->md_rows = false;   // n_precise is this queue's
   launch_shadow(c, d_x, s);
   classify_async(c, d_x, d_changeable, d_lam, d_precise_idx, d_n_precise, s);
   CK(cudaGetLastError());
@@ -894,6 +895,7 @@ ap_status ap_eval_ace(ap_ctx* c, int64_t n, const double* d_x, const double* d_l
   if (n == 0) return AP_OK;
   if (!d_x || !d_precise_idx || !d_n_precise || !d_e_prec) return fail(c, AP_ERR_ARG, "null argument");
   cudaStream_t s = S(stream);
+  c->md_rows = false;   // the caller's queue and its rows take the place of ap_step's
   launch_shadow(c, d_x, s);
   k_set_count<<<1, 1, 0, s>>>((const long long*)d_n_precise, (int)n, &c->d_sc->n_precise, &c->d_sc->n_precise64,
                             &c->d_sc->queue_dup);
@@ -961,7 +963,23 @@ ap_status ap_step(ap_ctx* c, int64_t n, double* d_x, double* d_v, double* d_f, c
     launch_ace_finalize(c, d_f, s);
     if (g.indenter_on) launch_indenter(c, d_x, d_f, c->step * g.dt, s);
     c->lam_ready = true;
-    c->md_ready = true;
+    c->md_ready = c->md_rows = true;
+  } else if (!c->md_rows) {
+    // A classification or an ACE evaluation between the calls, or an error in the last one, left
+    // another queue or its rows behind.  lambda determines the queue; the rows are built afresh,
+    // with their cells (rows at these positions on cells of older ones would be complete only
+    // for half the displacement that the skin check admits).
+    queue_from_lambda(c, s);
+    if (nsteps > 0) {
+      launch_wrap_positions(c, d_x, s);
+      st = build_checked(c, d_x, nullptr, s);
+      if (st) return st;
+      st = build_ace_checked(c, d_x, c->d_precise, &c->d_sc->n_precise, s);
+      if (st) return st;
+      ace_ref(c, s);
+      CK(cudaMemsetAsync(c->d_eprec, 0, sizeof(double) * (size_t)n, s));
+      c->md_rows = true;
+    }
   }
   st = clear_err(c, s);
   if (st) return st;
@@ -1010,6 +1028,7 @@ ap_status ap_step(ap_ctx* c, int64_t n, double* d_x, double* d_v, double* d_f, c
       build = lam_step || c->step % rb == 0;
     }
     if (build || lam_step) {
+      c->md_rows = false;   // until the new queue's rows stand: an error may end the call before
       if (build) {
         PhaseTimer t(c, s, AP_PHASE_NEIGHBORS);
         if (!skin_rule) {
@@ -1066,14 +1085,17 @@ ap_status ap_step(ap_ctx* c, int64_t n, double* d_x, double* d_v, double* d_f, c
         // E^p is 0 outside the queue: cleared when the queue may have changed, the atoms of the
         // queue are written by every evaluation
         CK(cudaMemsetAsync(c->d_eprec, 0, sizeof(double) * (size_t)n, s));
+        c->md_rows = true;
       }
     } else if (ace_only) {
       PhaseTimer t(c, s, AP_PHASE_NEIGHBORS);
       c->cells_stale = true;   // the atoms moved up to m since the cell build
       c->stale_m = m;
+      c->md_rows = false;
       st = build_ace_checked(c, d_x, c->d_precise, &c->d_sc->n_precise, s);
       if (st) return st;
       ace_ref(c, s);
+      c->md_rows = true;
       c->ace_rebuilds++;
     }
     {
