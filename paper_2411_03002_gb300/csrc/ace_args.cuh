@@ -50,6 +50,7 @@ struct AceArgs {
   const R* C1;
   const R* M2b;      // phi^(2) tables of the Finnis-Sinclair form
   const R* C1b;
+  const R* C1l;      // [16] what FP32 rounds off C1 and C1b
   R rc2, inv_rc, inv_n0;
   int mode;
   int fs_on;

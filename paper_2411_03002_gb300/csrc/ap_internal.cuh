@@ -270,7 +270,7 @@ struct ap_ctx {
   double* d_eext = nullptr;      // [n] indenter energy per atom (ap_step)
   uint8_t* d_changeable = nullptr;  // [n] complement of the fixed mask (ap_step)
   bool restart_pending = false;  // lambda state imported; next ap_step reuses it
-  float* d_W32 = nullptr;        // [W (320) | M2 (320) | C1 (8)]
+  float* d_W32 = nullptr;        // [W (320) | M2 (320) | C1 (8) | M2b (320) | C1b (8) | C1l (16)]
   double* d_W64 = nullptr;
   // ACE scratch per precise-queue position q < ace_q_cap (working precision)
   void* d_ace_list = nullptr;       // [q][ace_rec_cap] in-range (d_x, d_y, d_z, j) records

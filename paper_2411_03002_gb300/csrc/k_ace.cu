@@ -460,7 +460,7 @@ constexpr int kWarps3 = sizeof(R) == 4 ? AP_ACE3_WARPS : 4;   // warps per CTA o
 // FP64: SIMT loops, G with 4-wide vector loads along the neighbour axis.
 template <typename R>
 __global__ void __launch_bounds__(kWarps<R> * 32, sizeof(R) == 4 ? AP_ACE_MINB : 1) k_ace_basis(AceArgs<R> a) {
-  // Shared memory: W [320] | M2 [320] | C1 [8] | M2b [320] | C1b [8] | per warp: list
+  // Shared memory: W [320] | M2 [320] | C1 [8] | M2b [320] | C1b [8] | C1l [8] | C1bl [8] | per warp: list
   // [kListCap][4] | tile [kTileWords] (FP32: operand fragments of one batch; FP64: the
   // g/Y tile [kRows][kCols], which A and the G scratch alias after stage A).
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -469,7 +469,9 @@ __global__ void __launch_bounds__(kWarps<R> * 32, sizeof(R) == 4 ? AP_ACE_MINB :
   R* C1 = M2 + 320;
   R* M2b = C1 + 8;
   R* C1b = M2b + 320;
-  R* wbase = C1b + 8;
+  R* C1l = C1b + 8;    // what FP32 rounds off C1 and C1b (0 in FP64)
+  R* C1bl = C1l + 8;
+  R* wbase = C1bl + 8;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   R* list = wbase + warp * (4 * kListCap + kTileWords<R>);
   R* tile = list + 4 * kListCap;
@@ -481,6 +483,8 @@ __global__ void __launch_bounds__(kWarps<R> * 32, sizeof(R) == 4 ? AP_ACE_MINB :
   if (threadIdx.x < 8) {
     C1[threadIdx.x] = a.C1[threadIdx.x];
     C1b[threadIdx.x] = a.C1b[threadIdx.x];
+    C1l[threadIdx.x] = a.C1l[threadIdx.x];
+    C1bl[threadIdx.x] = a.C1l[8 + threadIdx.x];
   }
   __syncthreads();
   const int m = *a.count;
@@ -536,7 +540,7 @@ __global__ void __launch_bounds__(kWarps<R> * 32, sizeof(R) == 4 ? AP_ACE_MINB :
 
     // ---------------- stage A: G_klm = sum_j g_k Y_lm over the compacted neighbours,
     // then A = (1/N0) W . G and nu = 1, 2: E12 and dE12/dA
-    R e = R(0);
+    R e = R(0), e_lo = R(0);   // the nu = 1, 2 energy, and what FP32 rounds off its C1
     if constexpr (sizeof(R) == 4) {
       // Tensor cores, 3xTF32: per k-step of 8 neighbours, D[lm][k] += Y^T[lm][j] g[j][k]
       // for two m-tiles of 16 (l, m) rows.  Each lane evaluates g and Y of one neighbour
@@ -633,12 +637,16 @@ __global__ void __launch_bounds__(kWarps<R> * 32, sizeof(R) == 4 ? AP_ACE_MINB :
           if (lm < 25) {
             const float lin = lm == 0 ? C1[n] : 0.f;
             e += am[mt][u] * (0.5f * sm[mt][u] + lin);
+            // C1 to twice FP32's precision, in a sum of its own (e would round it off): its rounding
+            // shifts every energy the same way, by half of the mean error of bulk atoms (E of
+            // 255,840 atoms against FP64: mean 5.6e-6 -> 2.8e-6 eV, rms 2.84e-5 -> 2.80e-5 eV)
+            if (lm == 0) e_lo += am[mt][u] * C1l[n];
             a.dA[(size_t)q * 200 + n * 25 + lm] = sm[mt][u] + lin;
           }
         }
       if (a.fs_on) {   // the same products with the phi^(2) coefficients
         lm_mix(am, M2b, g8, t4, sm);
-        float eb = 0.f;
+        float eb = 0.f, eb_lo = 0.f;
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
@@ -647,10 +655,11 @@ __global__ void __launch_bounds__(kWarps<R> * 32, sizeof(R) == 4 ? AP_ACE_MINB :
             if (lm < 25) {
               const float lin = lm == 0 ? C1b[n] : 0.f;
               eb += am[mt][u] * (0.5f * sm[mt][u] + lin);
+              if (lm == 0) eb_lo += am[mt][u] * C1bl[n];
               a.dAb[(size_t)q * 200 + n * 25 + lm] = sm[mt][u] + lin;
             }
           }
-        const double Eb = warp_sum<double>((double)eb);
+        const double Eb = warp_sum<double>((double)eb + (double)eb_lo);
         if (lane == 0) a.e12b[q] = Eb;
       }
     } else {
@@ -736,7 +745,7 @@ __global__ void __launch_bounds__(kWarps<R> * 32, sizeof(R) == 4 ? AP_ACE_MINB :
         if (lane == 0) a.e12b[q] = Eb;
       }
     }
-    const double E = warp_sum<double>((double)e);
+    const double E = warp_sum<double>((double)e + (double)e_lo);
     if (lane == 0) a.e12[q] = E;
     cnt_pairs += nin;
     cnt_atoms += 1;
@@ -873,7 +882,7 @@ __global__ void k_ace_finalize64(int n, double* __restrict__ acc, double* __rest
 
 template <typename R>
 size_t basis_smem() {
-  return sizeof(R) * (320 + 320 + 8 + 320 + 8) + sizeof(R) * kWarps<R> * (4 * kListCap + kTileWords<R>);
+  return sizeof(R) * (320 + 320 + 8 + 320 + 3 * 8) + sizeof(R) * kWarps<R> * (4 * kListCap + kTileWords<R>);
 }
 
 template <typename R>
@@ -935,10 +944,11 @@ void run_ace(ap_ctx* c, const double* d_lam, const double* d_wgt, const int* d_q
   a.lam = d_lam;
   a.wgt = d_wgt;
   a.faccfix = c->cfg.ace_deterministic ? c->d_faccfix : nullptr;
-  a.M2 = a.W + 320;   // the parameter block is [W (320) | M2 (320) | C1 (8) | M2b (320) | C1b (8)]
+  a.M2 = a.W + 320;   // the parameter block is [W (320) | M2 (320) | C1 (8) | M2b (320) | C1b (8) | C1l (16)]
   a.C1 = a.W + 640;
   a.M2b = a.W + 648;
   a.C1b = a.W + 968;
+  a.C1l = a.W + 976;
   a.fs_on = c->cfg.ace_fs_on;
   a.fs_eps = c->cfg.ace_fs_eps;
   a.dAb = reinterpret_cast<R*>(c->d_ace_dAb);
@@ -997,6 +1007,11 @@ void upload_ace_tables(ap_ctx* c) {
   p64.insert(p64.end(), t.m2b.begin(), t.m2b.end());
   p64.insert(p64.end(), t.c1b.begin(), t.c1b.end());
   std::vector<float> p32(p64.begin(), p64.end());
+  for (const auto* c1 : {&t.c1, &t.c1b})   // the rest of C1 and C1b beyond FP32
+    for (double v : *c1) {
+      p64.push_back(0.0);
+      p32.push_back((float)(v - (double)(float)v));
+    }
   cudaMalloc(&c->d_W32, sizeof(float) * p32.size());
   cudaMalloc(&c->d_W64, sizeof(double) * p64.size());
   cudaMemcpy(c->d_W32, p32.data(), sizeof(float) * p32.size(), cudaMemcpyHostToDevice);
