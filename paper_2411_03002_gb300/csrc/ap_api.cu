@@ -327,7 +327,7 @@ ap_status check_err_bits(ap_ctx* c) {
 }
 
 ap_status clear_err(ap_ctx* c, cudaStream_t s) {
-  // err, need_eam, need_ace, ace_row_max, n_ace_groups
+  // err, need_eam, need_ace, ace_row_max, n_row_groups
   CK(cudaMemsetAsync(&c->d_sc->err, 0, 5 * sizeof(int), s));
   return AP_OK;
 }

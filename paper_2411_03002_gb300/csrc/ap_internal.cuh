@@ -104,7 +104,7 @@ struct DevScalars {
   int need_eam;       // largest EAM row count seen
   int need_ace;       // largest ACE row count seen
   int ace_row_max;    // longest ACE row of the last ACE row build
-  int n_ace_groups;   // cell groups with queued atoms (ACE row build); cleared with the four above
+  int n_row_groups;   // cell groups with (queued) atoms that a row build listed; cleared with the four above
   int n_detected;     // |D|
   int n_precise;      // |P| (int32 copy used by kernels)
   int work_counter;   // persistent-kernel work counters: 0 between the launches, k_ace_nu3 resets
