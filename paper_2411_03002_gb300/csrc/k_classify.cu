@@ -138,10 +138,6 @@ __device__ inline double sum_ascending(double v[kHalf]) {
 }
 
 // ------------------------------------------------------------------ CSP
-#ifndef AP_CSP_PREFETCH
-#define AP_CSP_PREFETCH 1   // software-pipelined row walk in the CSP selection (compile-time tuning)
-#endif
-
 // Three kernels share the atoms (launch_csp):
 //   k_csp_near   one thread per atom: the 12 nearest and the six smallest pair values found by
 //                thresholds, without sorting; in a crystal they stand apart.  Atoms where they
@@ -149,176 +145,11 @@ __device__ inline double sum_ascending(double v[kHalf]) {
 //   k_csp_sort   one thread per atom: sorted FP32 selections (insertion), for long lists only;
 //                what FP32 cannot decide is handed on again.
 //   k_csp_exact  one warp per atom, exact selections: what is left, short lists, small systems.
+// Structures without shells (a melt, a gas) take all three: updates of a gas of 50,000 / 100,000 /
+// 200,000 / 1,000,000 atoms 0.43 / 0.60 / 0.94 / 3.76 ms, where a sorting kernel for all atoms and a
+// thread for each of the rest took 0.92 / 0.97 / 1.32 / 3.71 ms.
 // FP64 arithmetic issues one warp instruction per 16 cycles and SM: a warp per atom for all
 // atoms would take 4 ms on 4,000,000 of them, the 89 FP64 operations of a thread 0.57 ms.
-
-// csp_atom: all selection arrays are indexed with compile-time indices (fully unrolled
-// insertion), so they live in registers.  An atom whose selection the FP32 values cannot
-// decide (an r_search band hit, an ambiguous 12/13 or 6/7 boundary) is appended to `slow`.
-// CSP of atom i (128-thread blocks: the shared arrays are indexed by threadIdx.x).
-// nin (rows built at these positions, else null): the row's first nin[i] entries
-// are the ones inside r_c^2 = rpf2 at the build (FP32), the rest lie beyond it.  When the
-// 13th smallest r^2 of that part lies more than two guard bands inside rpf2, no skin
-// entry can enter the 13 nearest or come within a band of the 12/13 boundary, and the
-// skin part is skipped; otherwise it is walked too.
-__device__ __forceinline__ void csp_atom(int i, const double* __restrict__ x, const uint8_t* __restrict__ ch,
-                                         const SysInfo* __restrict__ sys, const int* __restrict__ atom_sys,
-                                         const float4* __restrict__ s32, const int4* __restrict__ cunw,
-                                         const int* __restrict__ nbr, const int* __restrict__ off,
-                                         const int* __restrict__ cnt, int cap, float rsf2,
-                                         double* __restrict__ csp, int* __restrict__ slow, int* __restrict__ n_slow,
-                                         const int* __restrict__ nin = nullptr, float rpf2 = 0.f,
-                                         float stale2 = 0.f, int* __restrict__ n_stale = nullptr) {
-  static_assert(kNN <= 255, "neighbour slots are packed in 8 bits");
-  if (ch && !ch[i]) {
-    csp[i] = 0.0;
-    return;
-  }
-  const SysInfo& S = sys_of(sys, atom_sys, i);
-  const float4 si = s32[i];
-  const int4 ci = cunw[i];
-  const int c = cnt[i];
-  const size_t row = (size_t)i * cap;
-
-  // 1. the 13 smallest FP32 r^2 among candidates inside r_search
-  float tr[kNN + 1];
-  int tq[kNN + 1];
-#pragma unroll
-  for (int a = 0; a <= kNN; ++a) {
-    tr[a] = INFINITY;
-    tq[a] = -1;
-  }
-  int n_in = 0;
-  int q_end = nin ? nin[i] : c;
-#if AP_CSP_PREFETCH
-  // loads run ahead of the selection: the next entry's shadow and the entry after it
-  int j_a = c > 0 ? nbr[row] : 0;
-  float4 s_a = s32[j_a];
-  int j_b = c > 1 ? nbr[row + 1] : 0;
-#endif
-  for (int q = 0; q < c; ++q) {
-    if (q == q_end) {   // end of the in-range part
-      if (tr[kNN] + 2.f * kBand < rpf2) break;
-      q_end = c;
-    }
-#if AP_CSP_PREFETCH
-    const float4 sj = s_a;
-    j_a = j_b;
-    if (q + 1 < c) s_a = s32[j_a];
-    if (q + 2 < c) j_b = nbr[row + q + 2];
-#else
-    const float4 sj = s32[nbr[row + q]];
-#endif
-    int k[3];
-    entry_offset(off, row + q, S, ci.w, __float_as_int(sj.w), k);
-    const float dx = (float)k[0] * S.hf[0] + sj.x - si.x;
-    const float dy = (float)k[1] * S.hf[1] + sj.y - si.y;
-    const float dz = (float)k[2] * S.hf[2] + sj.z - si.z;
-    const float r2 = dx * dx + dy * dy + dz * dz;
-    if (r2 > rsf2 + kBand) continue;
-    if (r2 >= rsf2 - kBand) {
-      slow[atomicAdd(n_slow, 1)] = i;
-      return;
-    }
-    ++n_in;
-    if (r2 < tr[kNN]) {
-      tr[kNN] = r2;
-      tq[kNN] = q;
-#pragma unroll
-      for (int p = kNN; p > 0; --p) {
-        if (tr[p] < tr[p - 1]) {
-          const float t = tr[p];
-          tr[p] = tr[p - 1];
-          tr[p - 1] = t;
-          const int u = tq[p];
-          tq[p] = tq[p - 1];
-          tq[p - 1] = u;
-        }
-      }
-    }
-  }
-  // Rows older than the positions (stale2 > 0): every atom outside the row lies beyond
-  // r_search - 2 m (m the largest displacement since the build), stale2 = that radius
-  // squared.  The row's selection is exact when 12 candidates lie inside it with a
-  // guard band; otherwise (a nearly isolated atom) the atom is counted and the caller
-  // rebuilds the rows and computes the CSP again.
-  if (stale2 > 0.f && !(n_in >= kNN && tr[kNN - 1] + 2.f * kBand < stale2)) atomicAdd(n_stale, 1);
-  if (n_in < kNN) {
-    csp[i] = INFINITY;
-    return;
-  }
-  // 2. FP32 decides the 12 nearest unless the 12/13 boundary lies within the guard band
-  if (n_in > kNN && tr[kNN] - tr[kNN - 1] <= 2.f * kBand) {
-    slow[atomicAdd(n_slow, 1)] = i;
-    return;
-  }
-  // 3. FP32 vectors of the 12 and the 7 smallest pair values |r_a + r_b|^2.  The 12
-  // vectors and row positions live in shared memory, component-major (thread index
-  // fastest, conflict-free), not in registers.
-  __shared__ float s_v[3][kNN][128];
-  __shared__ int s_tq[kNN][128];
-  const int tx = threadIdx.x;
-#pragma unroll
-  for (int a = 0; a < kNN; ++a) {
-    const int q = tq[a];
-    s_tq[a][tx] = q;
-    const int j = nbr[row + q];
-    const float4 sj = s32[j];
-    int k[3];
-    entry_offset(off, row + q, S, ci.w, __float_as_int(sj.w), k);
-    s_v[0][a][tx] = (float)k[0] * S.hf[0] + sj.x - si.x;
-    s_v[1][a][tx] = (float)k[1] * S.hf[1] + sj.y - si.y;
-    s_v[2][a][tx] = (float)k[2] * S.hf[2] + sj.z - si.z;
-  }
-  float pv[kHalf + 1];
-  int pc[kHalf + 1];   // neighbour slots a | b << 8
-#pragma unroll
-  for (int a = 0; a <= kHalf; ++a) {
-    pv[a] = INFINITY;
-    pc[a] = 0;
-  }
-#pragma unroll
-  for (int a = 0; a < kNN; ++a) {
-    const float ax = s_v[0][a][tx], ay = s_v[1][a][tx], az = s_v[2][a][tx];
-#pragma unroll
-    for (int b = a + 1; b < kNN; ++b) {
-      const float sx = ax + s_v[0][b][tx], sy = ay + s_v[1][b][tx], sz = az + s_v[2][b][tx];
-      const float v = sx * sx + sy * sy + sz * sz;
-      if (v < pv[kHalf]) {
-        pv[kHalf] = v;
-        pc[kHalf] = a | (b << 8);
-#pragma unroll
-        for (int p = kHalf; p > 0; --p) {
-          if (pv[p] < pv[p - 1]) {
-            const float t = pv[p];
-            pv[p] = pv[p - 1];
-            pv[p - 1] = t;
-            const int u = pc[p];
-            pc[p] = pc[p - 1];
-            pc[p - 1] = u;
-          }
-        }
-      }
-    }
-  }
-  // 4. exact values of the six smallest pairs, unless the 6/7 boundary is ambiguous
-  double chosen[kHalf];
-  if (pv[kHalf] - pv[kHalf - 1] > 2.f * kBand) {
-#pragma unroll
-    for (int t = 0; t < kHalf; ++t) {
-      double da[3], db[3];
-      int ja, jb, sa[3], sb[3];
-      exact_entry(x, S, i, ci, nbr, off, cunw, row, s_tq[pc[t] & 0xff][tx], da, ja, sa);
-      exact_entry(x, S, i, ci, nbr, off, cunw, row, s_tq[pc[t] >> 8][tx], db, jb, sb);
-      const double s3[3] = {__dadd_rn(da[0], db[0]), __dadd_rn(da[1], db[1]), __dadd_rn(da[2], db[2])};
-      chosen[t] = norm2_exact(s3);
-    }
-  } else {
-    slow[atomicAdd(n_slow, 1)] = i;
-    return;
-  }
-  csp[i] = sum_ascending(chosen);
-}
 
 struct CspArgs {
   int n;
@@ -338,20 +169,178 @@ struct CspArgs {
   const int* nin;
   float rpf2, stale2;
   int* n_stale;
+  int sort_from;
 };
 
-// Atoms on k_csp_near's list up to which k_csp_exact takes them all (a warp each, about 2 ns);
-// beyond, k_csp_sort's threads (0.7 ns each, but 60 to 100 us however few).
-constexpr int kSortFrom = 48000;   // 965,000 atoms: 45,000 on the list took 0.43 ms sorted, 17,000 0.10 ms exactly
+// CSP of atom i by sorted FP32 selections; what FP32 cannot decide (an r_search band hit, an
+// ambiguous 12/13 or 6/7 boundary) is appended to `slow`.  All selection arrays are indexed with
+// compile-time indices (fully unrolled insertion), so they live in registers.  Rows four entries at
+// a time, and no exit but the end: with returns out of the loops the lanes of a warp, which go
+// on to the next atom here, no longer met again in the loops (1,000,000 atoms of a gas 10.5 ms,
+// 1.2 ms like this).
+// With A.nin (rows built at these positions) the row's first nin[i] entries are the ones inside
+// r_c^2 = rpf2 at the build (FP32), the rest lie beyond it: when the 13th smallest r^2 of that part
+// lies more than two guard bands inside rpf2, the skin part is skipped.  128-thread blocks: the
+// shared arrays are indexed by threadIdx.x.
+template <bool VEC>
+__device__ __forceinline__ void csp_atom(const CspArgs& A, int i, int* __restrict__ slow, int* __restrict__ n_slow) {
+  const SysInfo& S = sys_of(A.sys, A.atom_sys, i);
+  const float4 si = A.s32[i];
+  const int wi = __float_as_int(si.w);
+  const int c = A.cnt[i];
+  const size_t row = (size_t)i * A.cap;
+  const float rsf2 = A.rsf2;
 
+  // 1. the 13 smallest FP32 r^2 among candidates inside r_search
+  float tr[kNN + 1];
+  int tq[kNN + 1];
+#pragma unroll
+  for (int a = 0; a <= kNN; ++a) {
+    tr[a] = INFINITY;
+    tq[a] = -1;
+  }
+  int n_in = 0;
+  bool ok = true;
+  int q_end = A.nin ? A.nin[i] : c;
+  if (q_end == 0) q_end = c;
+  const int* const rowp = A.nbr + row;
+  int4 next = c > 0 ? row4<VEC>(rowp, 0, c) : make_int4(0, 0, 0, 0);
+  for (int q0 = 0; q0 < q_end; q0 += 4) {
+    // four entries at a time, the next four indices loaded ahead of their use
+    const int4 jj = next;
+    float4 sv[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) sv[u] = A.s32[q0 + u < c ? pick(jj, u) : i];
+    if (q0 + 4 < c) next = row4<VEC>(rowp, q0 + 4, c);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int q = q0 + u;
+      const float4 sj = sv[u];
+      int k[3];
+      entry_offset(A.off, row + min(q, c - 1), S, wi, __float_as_int(sj.w), k);
+      const float dx = (float)k[0] * S.hf[0] + sj.x - si.x;
+      const float dy = (float)k[1] * S.hf[1] + sj.y - si.y;
+      const float dz = (float)k[2] * S.hf[2] + sj.z - si.z;
+      const float r2 = dx * dx + dy * dy + dz * dz;
+      const bool in = q < c && r2 <= rsf2 + kBand;
+      ok = ok && !(in && r2 >= rsf2 - kBand);
+      n_in += in ? 1 : 0;
+      if (in && r2 < tr[kNN]) {
+        tr[kNN] = r2;
+        tq[kNN] = q;
+#pragma unroll
+        for (int p = kNN; p > 0; --p) {
+          const bool sw = tr[p] < tr[p - 1];
+          const float lo = fminf(tr[p], tr[p - 1]), hi = fmaxf(tr[p], tr[p - 1]);
+          const int ul = sw ? tq[p] : tq[p - 1], uh = sw ? tq[p - 1] : tq[p];
+          tr[p - 1] = lo;
+          tr[p] = hi;
+          tq[p - 1] = ul;
+          tq[p] = uh;
+        }
+      }
+    }
+    // the in-range part may end within a group of four: the entries after it only make the
+    // selection more complete
+    if (q0 + 4 >= q_end && q_end < c && !(tr[kNN] + 2.f * kBand < A.rpf2)) q_end = c;
+  }
+  // Rows older than the positions (stale2 > 0): every atom outside the row lies beyond
+  // r_search - 2 m (m the largest displacement since the build), stale2 = that radius
+  // squared.  The row's selection is exact when 12 candidates lie inside it with a
+  // guard band; otherwise (a nearly isolated atom) the atom is counted and the caller
+  // rebuilds the rows and computes the CSP again.
+  if (A.stale2 > 0.f && ok && !(n_in >= kNN && tr[kNN - 1] + 2.f * kBand < A.stale2)) atomicAdd(A.n_stale, 1);
+  const bool few = n_in < kNN;
+  // 2. FP32 decides the 12 nearest unless the 12/13 boundary lies within the guard band
+  ok = ok && (few || !(n_in > kNN && tr[kNN] - tr[kNN - 1] <= 2.f * kBand));
+  // 3. FP32 vectors of the 12 and the 7 smallest pair values |r_a + r_b|^2.  The 12
+  // vectors and row positions live in shared memory, component-major (thread index
+  // fastest, conflict-free), not in registers.
+  __shared__ float s_v[3][kNN][128];
+  __shared__ int s_tq[kNN][128];
+  const int tx = threadIdx.x;
+  double sum = INFINITY;
+  if (ok && !few) {
+#pragma unroll
+    for (int a = 0; a < kNN; ++a) {
+      const int q = tq[a];
+      s_tq[a][tx] = q;
+      const int j = A.nbr[row + q];
+      const float4 sj = A.s32[j];
+      int k[3];
+      entry_offset(A.off, row + q, S, wi, __float_as_int(sj.w), k);
+      s_v[0][a][tx] = (float)k[0] * S.hf[0] + sj.x - si.x;
+      s_v[1][a][tx] = (float)k[1] * S.hf[1] + sj.y - si.y;
+      s_v[2][a][tx] = (float)k[2] * S.hf[2] + sj.z - si.z;
+    }
+    float pv[kHalf + 1];
+    int pc[kHalf + 1];   // neighbour slots a | b << 8
+#pragma unroll
+    for (int a = 0; a <= kHalf; ++a) {
+      pv[a] = INFINITY;
+      pc[a] = 0;
+    }
+#pragma unroll 1
+    for (int a = 0; a < kNN - 1; ++a) {
+      const float ax = s_v[0][a][tx], ay = s_v[1][a][tx], az = s_v[2][a][tx];
+#pragma unroll 1
+      for (int b = a + 1; b < kNN; ++b) {
+        const float sx = ax + s_v[0][b][tx], sy = ay + s_v[1][b][tx], sz = az + s_v[2][b][tx];
+        const float v = sx * sx + sy * sy + sz * sz;
+        if (v < pv[kHalf]) {
+          pv[kHalf] = v;
+          pc[kHalf] = a | (b << 8);
+#pragma unroll
+          for (int p = kHalf; p > 0; --p) {
+            const bool sw = pv[p] < pv[p - 1];
+            const float lo = fminf(pv[p], pv[p - 1]), hi = fmaxf(pv[p], pv[p - 1]);
+            const int ul = sw ? pc[p] : pc[p - 1], uh = sw ? pc[p - 1] : pc[p];
+            pv[p - 1] = lo;
+            pv[p] = hi;
+            pc[p - 1] = ul;
+            pc[p] = uh;
+          }
+        }
+      }
+    }
+    // 4. exact values of the six smallest pairs, unless the 6/7 boundary is ambiguous
+    ok = pv[kHalf] - pv[kHalf - 1] > 2.f * kBand;
+    if (ok) {
+      const int4 ci = A.cunw[i];
+      double chosen[kHalf];
+#pragma unroll
+      for (int t = 0; t < kHalf; ++t) {
+        double da[3], db[3];
+        int ja, jb, sa[3], sb[3];
+        exact_entry(A.x, S, i, ci, A.nbr, A.off, A.cunw, row, s_tq[pc[t] & 0xff][tx], da, ja, sa);
+        exact_entry(A.x, S, i, ci, A.nbr, A.off, A.cunw, row, s_tq[pc[t] >> 8][tx], db, jb, sb);
+        const double s3[3] = {__dadd_rn(da[0], db[0]), __dadd_rn(da[1], db[1]), __dadd_rn(da[2], db[2])};
+        chosen[t] = norm2_exact(s3);
+      }
+      sum = sum_ascending(chosen);
+    }
+  }
+  if (ok) A.csp[i] = sum;
+  else slow[atomicAdd(n_slow, 1)] = i;
+}
+
+// Atoms per SM on k_csp_near's list up to which k_csp_exact takes them all.  A warp each takes 6 ns
+// an atom, the sort 75 us and 2.5 ns an atom; whole updates, sorted and by warps: a gas of 15,000
+// atoms 334 and 320 us, 20,000 355 and 347, 25,000 364 and 382, 40,000 404 and 475; 255,840 atoms
+// of disordered crystals with 15,500 on the list 975 and 965 us, with 39,000 1,076 and 1,157.
+constexpr int kSortFrom = 140;
+constexpr int kSortBlocks = 5;   // resident blocks of k_csp_sort per SM (92 registers)
+
+template <bool VEC>
 __global__ void __launch_bounds__(128) k_csp_sort(const CspArgs A, const int* __restrict__ list,
                                                   const int* __restrict__ n_list, int* __restrict__ slow,
                                                   int* __restrict__ n_slow) {
   const int m = *n_list;
-  if (m <= kSortFrom) return;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < m; t += gridDim.x * blockDim.x)
-    csp_atom(list[t], A.x, A.ch, A.sys, A.atom_sys, A.s32, A.cunw, A.nbr, A.off, A.cnt, A.cap, A.rsf2, A.csp, slow,
-             n_slow, A.nin, A.rpf2, A.stale2, A.n_stale);
+  if (m <= A.sort_from) return;
+  for (int t0 = blockIdx.x * blockDim.x; t0 < m; t0 += gridDim.x * blockDim.x) {
+    if (t0 + threadIdx.x < m) csp_atom<VEC>(A, list[t0 + threadIdx.x], slow, n_slow);
+    __syncwarp();
+  }
 }
 
 // Thread per atom, FP32 screening by thresholds.  The number of entries walked gives the density
@@ -521,7 +510,7 @@ __global__ void __launch_bounds__(128) k_csp_exact(const CspArgs A, const int* _
                                                    const int* __restrict__ n_list, const int* __restrict__ list2,
                                                    const int* __restrict__ n_list2) {
   const int lane = threadIdx.x & 31, warps = (gridDim.x * blockDim.x) >> 5;
-  const bool sorted = list && *n_list > kSortFrom;
+  const bool sorted = list && *n_list > A.sort_from;
   const int m = !list ? A.n : sorted ? *n_list2 : *n_list;
   const unsigned long long none = ~0ull;
   for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < m; w += warps) {
@@ -991,6 +980,7 @@ void launch_csp(ap_ctx* c, const double* d_x, const uint8_t* d_ch, cudaStream_t 
   A.rpf2 = rpf2;
   A.stale2 = stale2;
   A.n_stale = &c->d_sc->n_stale_bad;
+  A.sort_from = kSortFrom * c->num_sms;
   // a few thousand atoms: a warp each at once (237 atoms 14 us; a thread each took 64 us, since
   // one atom's chain is that long)
   if (c->n <= 32 * c->num_sms) {
@@ -1002,9 +992,10 @@ void launch_csp(ap_ctx* c, const double* d_x, const uint8_t* d_ch, cudaStream_t 
   auto near = c->cap_eam % 4 == 0 ? k_csp_near<true> : k_csp_near<false>;
   near<<<nblk(c->n, 128), 128, 0, s>>>(A, c->d_csp_slow, n_list);
   // the handed-over atoms, grid-stride over the device-side counts; d_det1 is free until the spread
-  if (c->n > kSortFrom) k_csp_sort<<<c->num_sms * 4, 128, 0, s>>>(A, c->d_csp_slow, n_list, c->d_det1, n_slow);
+  auto sort = c->cap_eam % 4 == 0 ? k_csp_sort<true> : k_csp_sort<false>;
+  if (c->n > A.sort_from) sort<<<c->num_sms * kSortBlocks, 128, 0, s>>>(A, c->d_csp_slow, n_list, c->d_det1, n_slow);
   k_csp_exact<<<c->num_sms * 8, 128, 0, s>>>(A, c->d_csp_slow, n_list, c->d_det1, n_slow);
-  c->kernels += c->n > kSortFrom ? 3 : 2;
+  c->kernels += c->n > A.sort_from ? 3 : 2;
 }
 
 // d_score: the detection score pushed into the history (CSP, or the selector's p),
