@@ -57,7 +57,8 @@ __device__ inline bool take_acc(const AceAcc& A, int i, double f[3]) {
   return any;
 }
 
-// Spherical indenter: F = k (R - r)^2 (x - c)/r, E = k (R - r)^3 / 3 for r < R.
+// Spherical indenter: F = k (R - r)^2 (x - c)/r, E = k (R - r)^3 / 3 for r < R.  Explicit fused
+// operations, so that the kernels that use it round alike.
 struct Indent {
   int on;
   double c[3], R, k;
@@ -67,13 +68,13 @@ __device__ inline bool indent_force(const Indent& I, const double x[3], double f
   e = 0.0;
   if (!(dz < I.R && dz > -I.R)) return false;   // r^2 < R^2 needs |dz| < R: most atoms stop here
   const double dx = x[0] - I.c[0], dy = x[1] - I.c[1];
-  const double r2 = dx * dx + dy * dy + dz * dz;
+  const double r2 = __fma_rn(dz, dz, __fma_rn(dy, dy, __dmul_rn(dx, dx)));
   if (!(r2 < I.R * I.R && r2 > 0.0)) return false;
   const double r = sqrt(r2);
   const double g = I.k * (I.R - r) * (I.R - r) / r;
-  f[0] += g * dx;
-  f[1] += g * dy;
-  f[2] += g * dz;
+  f[0] = __fma_rn(g, dx, f[0]);
+  f[1] = __fma_rn(g, dy, f[1]);
+  f[2] = __fma_rn(g, dz, f[2]);
   e = I.k * (I.R - r) * (I.R - r) * (I.R - r) / 3.0;
   return true;
 }
