@@ -301,6 +301,7 @@ ap_status ensure_capacity(ap_ctx* c, int64_t n) {
   c->hist_started = false;
   c->lam_ready = false;
   c->md_ready = false;
+  c->ace_rows = 0;
   return AP_OK;
 }
 
@@ -378,6 +379,7 @@ ap_status build_ace_checked(ap_ctx* c, const double* d_x, const int* d_queue, co
                             bool caller_queue = false) {
   const size_t off = (size_t)((const char*)d_count - (const char*)c->d_sc);
   if (off + sizeof(int) > sizeof(DevScalars)) return fail(c, AP_ERR_ARG, "queue length outside the device scalars");
+  c->ace_rows = 0;
   for (int attempt = 0; attempt < 2; ++attempt) {
     ap_status st = clear_err(c, s);
     if (st) return st;
@@ -399,6 +401,7 @@ ap_status build_ace_checked(ap_ctx* c, const double* d_x, const int* d_queue, co
     }
     st = check_err_bits(c);
     if (st) return st;
+    if (d_queue == c->d_precise) c->ace_rows = m;
     return ensure_ace_records(c, c->h_sc->ace_row_max);
   }
   return AP_OK;
@@ -733,6 +736,7 @@ ap_status ap_build_neighbors_batch(ap_ctx* c, int32_t n_sys, const int64_t* h_of
     c->hist_started = false;
     c->lam_ready = false;
     c->md_ready = false;
+    c->ace_rows = 0;
   }
   c->n = n;
   if (n == 0) {
@@ -757,7 +761,7 @@ ap_status ap_get_neighbors(ap_ctx* c, int32_t which, int32_t* d_cnt, int32_t* d_
   if (which != 0 && which != 1) return fail(c, AP_ERR_ARG, "which must be 0 (EAM) or 1 (ACE)");
   ap_status st = read_scalars(c, 0);
   if (st) return st;
-  int64_t rows = which == 0 ? c->n : c->h_sc->n_precise;
+  int64_t rows = which == 0 ? c->n : c->ace_rows;
   if (h_rows) *h_rows = rows;
   if (rows > 0 && (!d_cnt || !d_idx || !d_shift || cap <= 0)) return fail(c, AP_ERR_ARG, "null output or cap <= 0");
   launch_export_rows(c, which, (int)rows, (int)cap, d_cnt, d_idx, d_shift, 0);
@@ -783,7 +787,7 @@ ap_status ap_neighbor_total(ap_ctx* c, int32_t which, int64_t* h_total) {
   if (which == 2 && !c->lim_valid) return fail(c, AP_ERR_STATE, "no EAM evaluation on the current rows");
   ap_status st = read_scalars(c, 0);
   if (st) return st;
-  const int64_t rows = which == 1 ? c->h_sc->n_precise : c->n;
+  const int64_t rows = which == 1 ? c->ace_rows : c->n;
   launch_row_total(c, which, (int)rows, 0);
   unsigned long long t = 0;
   CK(cudaMemcpy(&t, &c->d_sc->row_total, sizeof(t), cudaMemcpyDeviceToHost));
@@ -945,6 +949,7 @@ ap_status ap_step(ap_ctx* c, int64_t n, double* d_x, double* d_v, double* d_f, c
     if (st) return st;
   }
   if (!c->md_ready) {
+    c->ace_rows = 0;
     launch_wrap_positions(c, d_x, s);
     st = build_checked(c, d_x, nullptr, s);
     if (st) return st;
@@ -969,6 +974,7 @@ ap_status ap_step(ap_ctx* c, int64_t n, double* d_x, double* d_v, double* d_f, c
     // another queue or its rows behind.  lambda determines the queue; the rows are built afresh,
     // with their cells (rows at these positions on cells of older ones would be complete only
     // for half the displacement that the skin check admits).
+    c->ace_rows = 0;
     queue_from_lambda(c, s);
     if (nsteps > 0) {
       launch_wrap_positions(c, d_x, s);
@@ -1029,6 +1035,7 @@ ap_status ap_step(ap_ctx* c, int64_t n, double* d_x, double* d_v, double* d_f, c
     }
     if (build || lam_step) {
       c->md_rows = false;   // until the new queue's rows stand: an error may end the call before
+      c->ace_rows = 0;
       if (build) {
         PhaseTimer t(c, s, AP_PHASE_NEIGHBORS);
         if (!skin_rule) {

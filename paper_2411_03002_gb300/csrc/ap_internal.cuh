@@ -329,6 +329,7 @@ struct ap_ctx {
   // MD
   int64_t step = 0;
   bool md_ready = false;
+  int ace_rows = 0;       // ACE rows of the queue in d_precise (0: none, or those of another queue)
   bool md_rows = false;   // d_precise, n_precise and the ACE rows are ap_step's own, at its positions and lambda
   int num_sms = 0;
 

@@ -76,3 +76,19 @@ def test_run_goes_on_with_its_own_queue(between, nxy, nz, before, after, rebuild
     assert (a.lam - b.lam).abs().max() < 1e-9
     assert abs(sa.e_pot - sb.e_pot) < 1e-7
     a.ctx.close(), b.ctx.close()
+
+
+def test_only_built_rows_are_exported():
+    """A classification makes a new queue; until its ACE rows are built there are none to export."""
+    r = Run(8, 10, 0)
+    s = r.step(2)
+    assert r.ctx.get_neighbors(1)[0].shape[0] == s.n_precise
+    fresh = ap.Context(r.ctx.cfg)
+    fresh.build_neighbors(r.x, ap.make_box((0, 0, -10.0), (8 * I.A_CU, 8 * I.A_CU, 10 * I.A_CU + 10.0), (True, True, False)))
+    lam, queue, count = fresh.classify(r.x)
+    assert int(count) > 0 and fresh.get_neighbors(1)[0].shape[0] == 0 and fresh.neighbor_total(1) == 0
+    fresh.eval_ace(r.x, lam, queue, count)
+    cnt = fresh.get_neighbors(1)[0]
+    assert cnt.shape[0] == int(count) and fresh.neighbor_total(1) == int(cnt.sum()) > 0
+    for c in (r.ctx, fresh):
+        c.close()
