@@ -359,8 +359,11 @@ struct BuildArgs {
   float rcf2;
   double rc2;
   float rpf2, band;
-  const int* groups;        // LIST: the groups that hold atoms (ACE rows: queued atoms)
+  // LIST: the groups that hold atoms (ACE rows: queued atoms); with more than list_max of them,
+  // thinly filled then, another kernel builds the rows (k_build_ace)
+  const int* groups;
   const int* n_list;
+  int list_max;
   // ACE rows only: the queue position of every atom (-1: none), the atoms' own shadows, the
   // stencil's half-width and the atoms' displacement since the cells were built (build_row_warp)
   const int* qpos;
@@ -420,6 +423,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32, AP_BUILD_MINB)
   const int sten = ACE ? A.sten : kStencil;
   const float margin = ACE ? A.margin : 0.f;
   const int n_work = LIST ? *A.n_list : A.n_groups;
+  if (LIST && n_work > A.list_max) return;
   for (int item = blockIdx.x; item < n_work; item += gridDim.x) {
   const int group_id = LIST ? A.groups[item] : item;
   __syncthreads();   // the shared arrays of the last item
@@ -464,7 +468,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32, AP_BUILD_MINB)
   const int py = my + 2 * sten, pz = mz + 2 * sten;
   const int ix_lo = S.periodic[0] ? floor_div(x0 - sten, nx) : 0;
   const int n_im = S.periodic[0] ? floor_div(x0 + mx - 1 + sten, nx) - ix_lo + 1 : 1;
-  const int n_runs = py * pz * n_im;   // at most T (launch_build_eam, launch_build_ace)
+  const int n_runs = py * pz * n_im;   // at most T: 36 x 5 for the EAM stencil; launch_build_ace checks
   const float blo = -margin - 1e-3f;
   const float gxh = (float)mx * hx - blo, gyh = (float)my * hy - blo, gzh = (float)mz * hz - blo;
   const float prune = sqrtf(A.rcf2) + margin, prune2 = prune * prune + A.band;
@@ -774,8 +778,10 @@ __global__ void __launch_bounds__(256) k_build_ace(const int* __restrict__ queue
                                                    const int4* __restrict__ cunw, const int* __restrict__ cstart,
                                                    const int* __restrict__ catoms, float rcf2, double rc2,
                                                    float band, int cap, int* __restrict__ nbr, int* __restrict__ off,
-                                                   int* __restrict__ cnt, DevScalars* sc, int sten, float margin) {
+                                                   int* __restrict__ cnt, DevScalars* sc, int sten, float margin,
+                                                   const int* __restrict__ n_list, int list_max) {
   __shared__ int4 s_buf[8][64];   // per warp: the stencil cells queued for the walk
+  if (n_list && *n_list <= list_max) return;   // k_build_rows has built them
   const int wib = threadIdx.x >> 5;
   const int m = *nq;
   const int warps = (gridDim.x * blockDim.x) >> 5;
@@ -921,6 +927,7 @@ void launch_build_eam(ap_ctx* c, const double* d_x, cudaStream_t s) {
   A.nin = c->d_lim_eam;
   A.sc = c->d_sc;
   A.qpos = A.groups = A.n_list = nullptr;
+  A.list_max = 0;
   A.s32 = c->d_sh32;
   A.sten = kStencil;
   A.n_groups = c->n_groups;
@@ -938,6 +945,7 @@ void launch_build_eam(ap_ctx* c, const double* d_x, cudaStream_t s) {
         (int)c->n, nullptr, nullptr, c->d_sys, c->d_atom_sys, c->d_cunw, c->build_group, nullptr, flag, list, n_list);
     A.groups = list;
     A.n_list = n_list;
+    A.list_max = c->n_groups;
     c->kernels += 1;
     auto build = c->stored_off ? k_build_rows<true, false, true> : k_build_rows<false, false, true>;
     build<<<std::min(c->n_groups, c->num_sms * AP_BUILD_MINB * 2), kBuildWarps * 32, 0, s>>>(A);
@@ -965,12 +973,17 @@ void launch_build_ace(ap_ctx* c, const double* d_x, const int* d_queue, const in
   // Cell groups, as for the EAM rows, for long queues in which every atom stands once, where the
   // stencil's runs fit a block's threads (k_build_rows: 255,840 atoms at 8 A 0.59 ms, a warp per
   // row 0.83; 240,000 of 4,000,000 at 7.7 A 0.76 and 0.97); a warp per row otherwise (12,700 atoms
-  // 43 us, by groups 51 and the list 5; 83,000 in narrow boxes 0.267 and 0.266 ms).
+  // 43 us, by groups 51 and the list 5; 83,000 in narrow boxes 0.267 and 0.266 ms), and where the
+  // list shows that the queue is scattered over groups with fewer than 20 of its atoms (energies of
+  // 500,000 atoms' random parts, by groups and by warps: 5.5 a group 0.86 and 0.61 ms, 18 a group 1.62
+  // and 1.60, 26 a group 2.13 and 2.31).
   int runs = 0;
   for (const SysInfo& S : c->h_sys) {
     const int e = c->build_group + 2 * sten, im = S.periodic[0] ? (e + S.nc[0] - 1) / S.nc[0] + 1 : 1;
     runs = std::max(runs, e * e * im);
   }
+  const int* listed = nullptr;
+  const int list_max = m / 20;
   if (m >= 400 * c->num_sms && unique && runs <= kBuildWarps * 32) {
     int* flag = c->d_cell_count;   // free after the cell sort; n_groups <= n_cells
     int* list = c->d_slot;         // free after the cell sort; at most one group per atom
@@ -993,7 +1006,8 @@ void launch_build_ace(ap_ctx* c, const double* d_x, const int* d_queue, const in
     A.band = kBand;
     A.qpos = c->d_qpos;
     A.groups = list;
-    A.n_list = n_list;
+    A.n_list = listed = n_list;
+    A.list_max = list_max;
     A.s32 = c->d_sh32;
     A.sten = sten;
     A.margin = margin;
@@ -1005,13 +1019,13 @@ void launch_build_ace(ap_ctx* c, const double* d_x, const int* d_queue, const in
     auto build = c->stored_off ? k_build_rows<true, true> : k_build_rows<false, true>;
     build<<<std::max(1, std::min(c->n_groups, c->num_sms * AP_BUILD_MINB * 2)), kBuildWarps * 32, 0, s>>>(A);
     c->kernels += 2;
-    return;
+    if (c->n_groups <= list_max) return;
   }
   int grid = c->num_sms * 8;
   k_build_ace<<<grid, 256, 0, s>>>(d_queue, d_nq, d_x, c->d_sys, c->d_atom_sys, c->d_sh32, c->d_cunw,
                                    c->d_cell_start, c->d_cell_atoms, (float)rc2, rc2, kBand, c->cap_ace,
                                    c->d_nbr_ace, c->stored_off ? c->d_off_ace : nullptr, c->d_cnt_ace, c->d_sc, sten,
-                                   margin);
+                                   margin, listed, list_max);
   c->kernels += 1;
 }
 

@@ -95,11 +95,11 @@ def test_rows_by_groups_in_narrow_boxes_of_several_systems():
     ctx.close()
 
 
-@pytest.mark.parametrize("name", ["part", "crowded", "crowded part"])
+@pytest.mark.parametrize("name", ["part", "scattered", "crowded", "crowded part"])
 def test_rows_by_groups(name):
     m = per_sm(401)
-    if name == "part":
-        c = int(np.ceil((2.0 * m / 4) ** (1 / 3)))
+    if name in ("part", "scattered"):   # 22 of a group's 44 atoms, or 6 (a warp per row after all)
+        c = int(np.ceil(((2.0 if name == "part" else 7.0) * m / 4) ** (1 / 3)))
         x, box = crystal(c, c, c, 0.08), ((0, 0, -4.0), (c * A, c * A, c * A + 4.0), (True, True, False))
     else:   # about five times the crystal's density; a block per cell, or per 2 x 2 x 2 cells
         n = m if name == "crowded" else 2 * m
@@ -108,7 +108,7 @@ def test_rows_by_groups(name):
     ctx, xt = context(x, box)
     n = x.shape[0]
     q = torch.randperm(n, generator=torch.Generator().manual_seed(2))[:m].sort().values.to(torch.int32).cuda()
-    a, b = both_builds(ctx, xt, q, 320 if name == "part" else 1400)
+    a, b = both_builds(ctx, xt, q, 1400 if "crowded" in name else 320)
     assert torch.equal(a, b)
     ctx.close()
 
