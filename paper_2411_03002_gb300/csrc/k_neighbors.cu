@@ -360,7 +360,7 @@ struct BuildArgs {
   double rc2;
   float rpf2, band;
   // LIST: the groups that hold atoms (ACE rows: queued atoms); with more than list_max of them,
-  // thinly filled then, another kernel builds the rows (k_build_ace)
+  // thinly filled then, another kernel builds the rows (k_build_thin, k_build_ace)
   const int* groups;
   const int* n_list;
   int list_max;
@@ -746,6 +746,91 @@ __global__ void __launch_bounds__(kBuildWarps * 32, AP_BUILD_MINB)
   }
 }
 
+// EAM rows where a group of cells holds a few atoms only (a dilute gas): one thread per row, in cell
+// order, with the row order of k_build_rows.  In-range entries fill the row from the front, skin
+// entries from the end of its capacity, and the gap is closed at the end.  Only if the list of groups
+// is longer than list_max.
+__global__ void __launch_bounds__(128, 9) k_build_thin(int n, const int* __restrict__ atom_sys,
+                                                       const __grid_constant__ BuildArgs A) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n || *A.n_list <= A.list_max) return;
+  const int i = A.catoms[t];
+  const SysInfo& S = sys_of(A.sys, atom_sys, i);
+  const float4 si = A.s32[i];
+  const int4 ci = A.cunw[i];
+  const int cw[3] = {cell_x(ci.w), cell_y(ci.w), cell_z(ci.w)};
+  const float reach2 = A.rcf2 + A.band, r_sure = A.rcf2 - A.band;
+  int* const row = A.nbr + (size_t)i * A.cap;
+  int* const offrow = A.off ? A.off + (size_t)i * A.cap : nullptr;
+  int n_in = 0, n_skin = 0;
+  for (int dz = -kStencil; dz <= kStencil; ++dz) {
+    int tz = cw[2] + dz, iz = 0;
+    if (S.periodic[2]) {
+      iz = floor_div(tz, S.nc[2]);
+      tz -= iz * S.nc[2];
+    } else if (tz < 0 || tz >= S.nc[2]) {
+      continue;
+    }
+    const float oz = (float)dz * S.hf[2] - si.z, gz = fmaxf(0.f, fmaxf(oz, -oz - S.hf[2]));
+    for (int dy = -kStencil; dy <= kStencil; ++dy) {
+      int ty = cw[1] + dy, iy = 0;
+      if (S.periodic[1]) {
+        iy = floor_div(ty, S.nc[1]);
+        ty -= iy * S.nc[1];
+      } else if (ty < 0 || ty >= S.nc[1]) {
+        continue;
+      }
+      const float oy = (float)dy * S.hf[1] - si.y, gy = fmaxf(0.f, fmaxf(oy, -oy - S.hf[1]));
+      if (gz * gz + gy * gy > reach2) continue;
+      const int row0 = S.cell_base + (tz * S.nc[1] + ty) * S.nc[0];
+      for (int dx = -kStencil; dx <= kStencil; ++dx) {
+        int tx = cw[0] + dx, ix = 0;
+        if (S.periodic[0]) {
+          ix = floor_div(tx, S.nc[0]);
+          tx -= ix * S.nc[0];
+        } else if (tx < 0 || tx >= S.nc[0]) {
+          continue;
+        }
+        const float ox = (float)dx * S.hf[0] - si.x, gx = fmaxf(0.f, fmaxf(ox, -ox - S.hf[0]));
+        if (gz * gz + gy * gy + gx * gx > reach2) continue;
+        const int b = A.cstart[row0 + tx], e = A.cstart[row0 + tx + 1];
+        for (int a = b; a < e; ++a) {
+          if (a == t && dx == 0 && dy == 0 && dz == 0) continue;   // the atom itself
+          const float4 sj = A.s32c[a];
+          const int j = A.catoms[a];
+          const float ddx = ox + sj.x, ddy = oy + sj.y, ddz = oz + sj.z;
+          const float r2 = ddx * ddx + ddy * ddy + ddz * ddz;
+          if (r2 > reach2) continue;
+          if (!(r2 < r_sure)) {
+            const int img[3] = {ix, iy, iz};
+            if (!exact_within(A.x, S, i, j, ci, A.cunw[j], img, A.rc2)) continue;
+          }
+          const bool in = r2 < A.rpf2;
+          if (n_in + n_skin < A.cap) {
+            const int pos = in ? n_in : A.cap - 1 - n_skin;
+            row[pos] = j;
+            if (offrow) offrow[pos] = pack_off(dx, dy, dz);
+          }
+          n_in += in ? 1 : 0;
+          n_skin += in ? 0 : 1;
+        }
+      }
+    }
+  }
+  const int cnt = n_in + n_skin;
+  if (cnt < A.cap)   // destinations lie below every later source
+    for (int k = 0; k < n_skin; ++k) {
+      row[n_in + k] = row[A.cap - n_skin + k];
+      if (offrow) offrow[n_in + k] = offrow[A.cap - n_skin + k];
+    }
+  A.cnt[i] = min(cnt, A.cap);
+  A.nin[i] = min(n_in, A.cap);
+  if (cnt > A.cap) {
+    atomicMax(&A.sc->need_eam, cnt);
+    atomicOr(&A.sc->err, kErrCapacity);
+  }
+}
+
 // The list of the cell groups with queued atoms (in any order: it only orders the work), and
 // qpos[i] = queue position of atom i (the others hold -1).  flag: one int per group, 0.  A null
 // queue stands for all n atoms (no qpos then).
@@ -933,10 +1018,15 @@ void launch_build_eam(ap_ctx* c, const double* d_x, cudaStream_t s) {
   A.n_groups = c->n_groups;
   A.margin = 0.f;
   c->kernels += 1;
-  // Mostly vacuum: the groups that hold atoms are listed first (about 6 us), since a block that
-  // finds its group empty costs 4.3 ns: builds of 108,000 atoms in a box of 400 A 0.74 -> 0.28 ms, of
-  // 800 A 4.57 -> 0.33 ms (a full group holds 44 atoms; 150 A, 16 a group, 0.25 ms without a list).
-  if (c->n_groups > 4096 && c->n < 8 * (int64_t)c->n_groups) {
+  // Fewer than 32 atoms a group on average (a crystal of copper's density fills one with 44): the
+  // groups that hold atoms are listed first (about 8 us), since a block that finds its group empty
+  // costs 4.3 ns, and the list's length decides.  A few thousand full groups in a large box are built
+  // from the list (whole builds of 10,976 atoms in 400 A 0.63 -> 0.13 ms, of 108,000 in 800 A
+  // 4.6 -> 0.34 ms); many groups, at 10 ns each however few their atoms, by a thread per row: a
+  // gas of a tenth of the crystal's density, 1,000,000 atoms 2.8 -> 0.86 ms, 100,000 0.34 -> 0.19, but
+  // 20,000 0.14 -> 0.18; a crystal of 0.6 of it, 1,000,000 atoms 1.44 -> 1.08 ms.  From 32 atoms a
+  // group on a block per group is as fast or faster (1,000,000 atoms at 0.8: 1.30 and 1.35 ms).
+  if (c->n_groups > 4096 && c->n < 32 * (int64_t)c->n_groups) {
     int* flag = c->d_cell_count;   // free after the cell sort, like d_slot; n_groups <= n_cells
     int* list = c->d_slot;
     int* n_list = &c->d_sc->n_row_groups;   // cleared by build_checked
@@ -945,10 +1035,14 @@ void launch_build_eam(ap_ctx* c, const double* d_x, cudaStream_t s) {
         (int)c->n, nullptr, nullptr, c->d_sys, c->d_atom_sys, c->d_cunw, c->build_group, nullptr, flag, list, n_list);
     A.groups = list;
     A.n_list = n_list;
-    A.list_max = c->n_groups;
+    A.list_max = 5000 + (int)c->n / 60;
     c->kernels += 1;
     auto build = c->stored_off ? k_build_rows<true, false, true> : k_build_rows<false, false, true>;
     build<<<std::min(c->n_groups, c->num_sms * AP_BUILD_MINB * 2), kBuildWarps * 32, 0, s>>>(A);
+    if (std::min<int64_t>(c->n, c->n_groups) > A.list_max) {
+      k_build_thin<<<nblk(c->n, 128), 128, 0, s>>>((int)c->n, c->d_atom_sys, A);
+      c->kernels += 1;
+    }
     return;
   }
   auto build = c->stored_off ? k_build_rows<true, false> : k_build_rows<false, false>;

@@ -75,10 +75,10 @@ def pair_sets(x, radius):
     return torch.sort(torch.cat(keys)).values
 
 
-# (list radius, atoms, box edge): a block per cell, a block per 2 x 2 x 2 cells, and enough atoms
-# for the ACE rows by groups of cells (400 per SM)
+# (list radius, atoms, box edge): a block per cell, a block per 2 x 2 x 2 cells, enough atoms for
+# the ACE rows by groups of cells (400 per SM), and a gas dilute enough for a thread per row
 @pytest.mark.parametrize("radius,n,edge", [(3.0, 2000, 15.0), (12.0, 1500, 60.0), (12.0, 20000, 120.0),
-                                           (12.0, 64000, 120.0)])
+                                           (12.0, 64000, 120.0), (12.0, 20000, 480.0)])
 def test_pairs_at_the_lower_bound_are_in_the_rows(radius, n, edge):
     x, pairs = workload(radius, n, edge, 64)
     r2 = f32(radius * radius)

@@ -1,5 +1,5 @@
 """EAM rows of bodies in boxes that are mostly vacuum, built from a list of the cell groups that
-hold atoms, against all pairs (needs a GPU)."""
+hold atoms, and of dilute gases, built by a thread per row, against all pairs (needs a GPU)."""
 import numpy as np
 import pytest
 import torch
@@ -51,4 +51,30 @@ def test_rows_of_bodies_in_several_boxes():
         i, j, code = k // 32768 // m, k // 32768 % m, k % 32768
         want.append(((i + int(a)) * n + j + int(a)) * 32768 + code)
     assert torch.equal(got, torch.sort(torch.cat(want)).values)
+    ctx.close()
+
+
+def dilute(n, box, seed, cluster=0):
+    lo, hi = np.asarray(box[0], float), np.asarray(box[1], float)
+    g = np.random.Generator(np.random.PCG64(seed))
+    x = g.uniform(lo, hi, (n, 3))
+    if cluster:   # rows beyond the default capacity
+        x[:cluster] = 0.5 * (lo + hi) + g.uniform(-3.0, 3.0, (cluster, 3))
+    return x, box
+
+
+GASES = {
+    "periodic": dilute(20000, ((0, 0, 0), (168, 170, 166), PERIODIC), 1),
+    "free": dilute(20000, ((-5, -5, -5), (163, 165, 161), (False, False, False)), 2, 300),
+    "narrow": dilute(20000, ((0, 0, 0), (3.4 * A, 620, 610), PERIODIC), 3),
+    "outside": (lambda x, b: (x + np.array([168.0, -170.0, 332.0]), b))(*dilute(20000, ((0, 0, 0), (168, 170, 166), PERIODIC), 4)),
+}
+
+
+@pytest.mark.parametrize("name", GASES)
+def test_rows_of_a_dilute_gas(name):
+    x, box = GASES[name]
+    ctx, xt = context(x, box)
+    n = x.shape[0]
+    assert torch.equal(row_keys(ctx, 0, torch.arange(n, device="cuda"), n), all_pairs(x, box, 6.5))
     ctx.close()
