@@ -425,324 +425,324 @@ __global__ void __launch_bounds__(kBuildWarps * 32, AP_BUILD_MINB)
   const int n_work = LIST ? *A.n_list : A.n_groups;
   if (LIST && n_work > A.list_max) return;
   for (int item = blockIdx.x; item < n_work; item += gridDim.x) {
-  const int group_id = LIST ? A.groups[item] : item;
-  __syncthreads();   // the shared arrays of the last item
-  // the system and the group of cells
-  int sys = 0;
-  for (int lo = 0, hi = A.n_sys - 1; lo <= hi;) {
-    const int mid = (lo + hi) >> 1;
-    if (A.sys[mid].grp_base <= group_id) {
-      sys = mid;
-      lo = mid + 1;
-    } else {
-      hi = mid - 1;
-    }
-  }
-  const SysInfo& S = A.sys[sys];
-  const int nx = S.nc[0], ny = S.nc[1], nz = S.nc[2];
-  const float hx = S.hf[0], hy = S.hf[1], hz = S.hf[2];
-  const int gx = (nx + A.group - 1) / A.group, gy = (ny + A.group - 1) / A.group;
-  const int gid = group_id - S.grp_base;
-  const int x0 = gid % gx * A.group, y0 = gid / gx % gy * A.group, z0 = gid / (gx * gy) * A.group;
-  const int mx = min(A.group, nx - x0), my = min(A.group, ny - y0), mz = min(A.group, nz - z0);
-  const float reach2 = A.rcf2 + A.band, r_sure = A.rcf2 - A.band;
-  // r_sure is rounded and may lie further from rcf2 than the guard band: the exact decision takes
-  // every pair that is not surely inside (the difference itself is exact)
-  const float band = fmaxf(A.band, A.rcf2 - r_sure);
-  // this warp's cell of the group, or its share of the single cell's atoms
-  const int parts = A.group == 1 ? kBuildWarps : 1, part = A.group == 1 ? warp : 0;
-  const int wx = warp & 1, wy = (warp >> 1) & 1, wz = warp >> 2;
-  int b = 0, own = 0, ux = 0, uy = 0, uz = 0;
-  if (A.group == 1 || (wx < mx && wy < my && wz < mz)) {
-    if (A.group != 1) {
-      ux = wx;
-      uy = wy;
-      uz = wz;
-    }
-    const int cell = S.cell_base + ((z0 + uz) * ny + y0 + uy) * nx + x0 + ux;
-    b = A.cstart[cell];
-    own = max(0, (A.cstart[cell + 1] - b - part + parts - 1) / parts);   // atoms part, part + parts, ...
-  }
-  // ---- the runs of the group's stencil: pencil (dy, dz), periodic image ix along x.  Cells are
-  // cut at the reach plus the margin of the group's box grown by the margin.
-  const int py = my + 2 * sten, pz = mz + 2 * sten;
-  const int ix_lo = S.periodic[0] ? floor_div(x0 - sten, nx) : 0;
-  const int n_im = S.periodic[0] ? floor_div(x0 + mx - 1 + sten, nx) - ix_lo + 1 : 1;
-  const int n_runs = py * pz * n_im;   // at most T: 36 x 5 for the EAM stencil; launch_build_ace checks
-  const float blo = -margin - 1e-3f;
-  const float gxh = (float)mx * hx - blo, gyh = (float)my * hy - blo, gzh = (float)mz * hz - blo;
-  const float prune = sqrtf(A.rcf2) + margin, prune2 = prune * prune + A.band;
-  int len = 0;
-  if (threadIdx.x < n_runs) {
-    const int pen = threadIdx.x / n_im, ix = ix_lo + threadIdx.x - pen * n_im;
-    const int dz = pen / py - sten, dy = pen % py - sten;
-    int ty = y0 + dy, tz = z0 + dz;
-    bool valid = true;
-    if (S.periodic[1]) ty -= floor_div(ty, ny) * ny;
-    else valid = valid && ty >= 0 && ty < ny;
-    if (S.periodic[2]) tz -= floor_div(tz, nz) * nz;
-    else valid = valid && tz >= 0 && tz < nz;
-    const float ay = fmaxf(0.f, fmaxf((float)dy * hy - gyh, blo - (float)(dy + 1) * hy));
-    const float az = fmaxf(0.f, fmaxf((float)dz * hz - gzh, blo - (float)(dz + 1) * hz));
-    const float left = prune2 - ay * ay - az * az;
-    if (valid && left >= 0.f) {
-      const float ax = sqrtf(left) + 2e-3f;   // cells that the reach along x touches, slack for the division
-      const int c0 = max(max(-sten, (int)floorf((blo - ax) / hx)) + x0 - ix * nx, 0);
-      const int c1 = min(min(mx - 1 + sten, (int)floorf((gxh + ax) / hx)) + x0 - ix * nx, nx - 1);
-      if (c0 <= c1) {
-        const int row0 = S.cell_base + (tz * ny + ty) * nx;
-        const int beg = A.cstart[row0 + c0];
-        len = A.cstart[row0 + c1 + 1] - beg;
-        s_beg[threadIdx.x] = beg;
-        s_run[threadIdx.x] = pack_off(0, dy, dz) | (ix - ix_lo) << 24;
+    const int group_id = LIST ? A.groups[item] : item;
+    __syncthreads();   // the shared arrays of the last item
+    // the system and the group of cells
+    int sys = 0;
+    for (int lo = 0, hi = A.n_sys - 1; lo <= hi;) {
+      const int mid = (lo + hi) >> 1;
+      if (A.sys[mid].grp_base <= group_id) {
+        sys = mid;
+        lo = mid + 1;
+      } else {
+        hi = mid - 1;
       }
     }
-  }
-  int pre = len;   // inclusive scan of the lengths over the block
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, pre, o);
-    if (lane >= o) pre += v;
-  }
-  if (lane == 31) s_sum[warp] = pre;
-  __syncthreads();
-  if (warp == 0) {
-    int v = lane < kBuildWarps ? s_sum[lane] : 0;
-#pragma unroll
-    for (int o = 1; o < kBuildWarps; o <<= 1) {
-      const int w = __shfl_up_sync(0xffffffffu, v, o);
-      if (lane >= o) v += w;
+    const SysInfo& S = A.sys[sys];
+    const int nx = S.nc[0], ny = S.nc[1], nz = S.nc[2];
+    const float hx = S.hf[0], hy = S.hf[1], hz = S.hf[2];
+    const int gx = (nx + A.group - 1) / A.group, gy = (ny + A.group - 1) / A.group;
+    const int gid = group_id - S.grp_base;
+    const int x0 = gid % gx * A.group, y0 = gid / gx % gy * A.group, z0 = gid / (gx * gy) * A.group;
+    const int mx = min(A.group, nx - x0), my = min(A.group, ny - y0), mz = min(A.group, nz - z0);
+    const float reach2 = A.rcf2 + A.band, r_sure = A.rcf2 - A.band;
+    // r_sure is rounded and may lie further from rcf2 than the guard band: the exact decision takes
+    // every pair that is not surely inside (the difference itself is exact)
+    const float band = fmaxf(A.band, A.rcf2 - r_sure);
+    // this warp's cell of the group, or its share of the single cell's atoms
+    const int parts = A.group == 1 ? kBuildWarps : 1, part = A.group == 1 ? warp : 0;
+    const int wx = warp & 1, wy = (warp >> 1) & 1, wz = warp >> 2;
+    int b = 0, own = 0, ux = 0, uy = 0, uz = 0;
+    if (A.group == 1 || (wx < mx && wy < my && wz < mz)) {
+      if (A.group != 1) {
+        ux = wx;
+        uy = wy;
+        uz = wz;
+      }
+      const int cell = S.cell_base + ((z0 + uz) * ny + y0 + uy) * nx + x0 + ux;
+      b = A.cstart[cell];
+      own = max(0, (A.cstart[cell + 1] - b - part + parts - 1) / parts);   // atoms part, part + parts, ...
     }
-    if (lane < kBuildWarps) s_sum[lane] = v;
-  }
-  __syncthreads();
-  const int total = s_sum[kBuildWarps - 1];
-  s_pre[threadIdx.x + 1] = pre + (warp ? s_sum[warp - 1] : 0);
-  if (threadIdx.x == 0) s_pre[0] = 0;
-  __syncthreads();
-  if (total == 0) {   // no atom in the group either
-    if constexpr (LIST) continue;
-    else return;
-  }
-
-  // ---- rounds: stage candidates (ordered), then test them against every warp's atoms
-  int at = 0, staged = 0;   // uniform over the block
-  bool first_round = true;
-  while (true) {
-    bool full = false;
-    while (at < total) {
-      const int f = at + threadIdx.x;
-      bool keep = false;
-      float px = 0.f, py_ = 0.f, pz_ = 0.f;
-      int j = 0, ko = 0;
-      if (f < total) {
-        int lo = 0, hi = n_runs - 1;   // the run of candidate f: the last one with s_pre <= f
-        while (lo < hi) {
-          const int mid = (lo + hi + 1) >> 1;
-          if (s_pre[mid] <= f) lo = mid;
-          else hi = mid - 1;
+    // ---- the runs of the group's stencil: pencil (dy, dz), periodic image ix along x.  Cells are
+    // cut at the reach plus the margin of the group's box grown by the margin.
+    const int py = my + 2 * sten, pz = mz + 2 * sten;
+    const int ix_lo = S.periodic[0] ? floor_div(x0 - sten, nx) : 0;
+    const int n_im = S.periodic[0] ? floor_div(x0 + mx - 1 + sten, nx) - ix_lo + 1 : 1;
+    const int n_runs = py * pz * n_im;   // at most T: 36 x 5 for the EAM stencil; launch_build_ace checks
+    const float blo = -margin - 1e-3f;
+    const float gxh = (float)mx * hx - blo, gyh = (float)my * hy - blo, gzh = (float)mz * hz - blo;
+    const float prune = sqrtf(A.rcf2) + margin, prune2 = prune * prune + A.band;
+    int len = 0;
+    if (threadIdx.x < n_runs) {
+      const int pen = threadIdx.x / n_im, ix = ix_lo + threadIdx.x - pen * n_im;
+      const int dz = pen / py - sten, dy = pen % py - sten;
+      int ty = y0 + dy, tz = z0 + dz;
+      bool valid = true;
+      if (S.periodic[1]) ty -= floor_div(ty, ny) * ny;
+      else valid = valid && ty >= 0 && ty < ny;
+      if (S.periodic[2]) tz -= floor_div(tz, nz) * nz;
+      else valid = valid && tz >= 0 && tz < nz;
+      const float ay = fmaxf(0.f, fmaxf((float)dy * hy - gyh, blo - (float)(dy + 1) * hy));
+      const float az = fmaxf(0.f, fmaxf((float)dz * hz - gzh, blo - (float)(dz + 1) * hz));
+      const float left = prune2 - ay * ay - az * az;
+      if (valid && left >= 0.f) {
+        const float ax = sqrtf(left) + 2e-3f;   // cells that the reach along x touches, slack for the division
+        const int c0 = max(max(-sten, (int)floorf((blo - ax) / hx)) + x0 - ix * nx, 0);
+        const int c1 = min(min(mx - 1 + sten, (int)floorf((gxh + ax) / hx)) + x0 - ix * nx, nx - 1);
+        if (c0 <= c1) {
+          const int row0 = S.cell_base + (tz * ny + ty) * nx;
+          const int beg = A.cstart[row0 + c0];
+          len = A.cstart[row0 + c1 + 1] - beg;
+          s_beg[threadIdx.x] = beg;
+          s_run[threadIdx.x] = pack_off(0, dy, dz) | (ix - ix_lo) << 24;
         }
-        const int slot = s_beg[lo] + f - s_pre[lo], o = s_run[lo];
-        j = A.catoms[slot];
-        const float4 sj = ACE ? A.s32[j] : A.s32c[slot];
-        const int kx = cell_x(__float_as_int(sj.w)) + (ix_lo + (o >> 24)) * nx - x0;
-        ko = (o & 0xffffff) + kx;
-        px = fmaf((float)kx, hx, sj.x);
-        py_ = fmaf((float)off_y(o), hy, sj.y);
-        pz_ = fmaf((float)off_z(o), hz, sj.z);
-        const float ax = fmaxf(0.f, fmaxf(blo - px, px - gxh)), ay = fmaxf(0.f, fmaxf(blo - py_, py_ - gyh)),
-                    az = fmaxf(0.f, fmaxf(blo - pz_, pz_ - gzh));
-        keep = ax * ax + ay * ay + az * az <= reach2;
       }
-      const unsigned mk = __ballot_sync(0xffffffffu, keep);
-      __syncthreads();
-      if (lane == 0) s_sum[warp] = __popc(mk);
-      __syncthreads();
-      int before = 0, sum = 0;
+    }
+    int pre = len;   // inclusive scan of the lengths over the block
 #pragma unroll
-      for (int w = 0; w < kBuildWarps; ++w) {
-        const int v = s_sum[w];
-        before += w < warp ? v : 0;
-        sum += v;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, pre, o);
+      if (lane >= o) pre += v;
+    }
+    if (lane == 31) s_sum[warp] = pre;
+    __syncthreads();
+    if (warp == 0) {
+      int v = lane < kBuildWarps ? s_sum[lane] : 0;
+#pragma unroll
+      for (int o = 1; o < kBuildWarps; o <<= 1) {
+        const int w = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += w;
       }
-      if (staged + sum > kStage) {   // uniform: no room, test what is staged first
-        full = true;
-        break;
-      }
-      if (keep) {
-        const int q = staged + before + __popc(mk & lt);
-        s_pos[q] = make_float4(px, py_, pz_, __int_as_float(j));
-        if (STORED) s_cell[q] = ko;
-      }
-      staged += sum;
-      at += T;
+      if (lane < kBuildWarps) s_sum[lane] = v;
     }
     __syncthreads();
-    for (int c0 = 0; c0 < own; c0 += 32) {   // up to 32 of the warp's atoms, one per lane
-      int nc = min(32, own - c0);
-      int slot = b + part + (c0 + min(lane, nc - 1)) * parts;
-      if constexpr (ACE) {   // the queued ones of them
-        const unsigned queued = __ballot_sync(0xffffffffu, lane < nc && A.qpos[A.catoms[slot]] >= 0);
-        if (!queued) continue;
-        if (queued >> lane & 1) s_own[warp][__popc(queued & lt)] = slot;
-        nc = __popc(queued);
-        __syncwarp();
-        slot = s_own[warp][min(lane, nc - 1)];
-        __syncwarp();
-      }
-      const int me_i = A.catoms[slot];
-      const int me_row = ACE ? A.qpos[me_i] : me_i;
-      const float4 sm = ACE ? A.s32[me_i] : A.s32c[slot];
-      const float mex = fmaf((float)ux, hx, sm.x), mey = fmaf((float)uy, hy, sm.y), mez = fmaf((float)uz, hz, sm.z);
-      int n_in = 0, n_skin = 0;   // entries found so far for this lane's atom
-      if (!first_round) {
-        n_in = ACE ? A.cnt[me_row] : A.nin[me_row];
-        n_skin = ACE ? 0 : A.cnt[me_row];
-      }
-      const float xlo = warp_min(mex), xhi = warp_max(mex), ylo = warp_min(mey), yhi = warp_max(mey),
-                  zlo = warp_min(mez), zhi = warp_max(mez);
-      unsigned short* const list = s_list[warp];
-      int from = 0;
-      bool first = first_round && !full, direct = false;
-      do {
-        // list the staged candidates within reach of this warp's atoms
-        int listed = 0;
-        while (from < staged) {
-          const int t = from + lane;
-          bool keep = false;
-          if (t < staged) {
-            const float4 p = s_pos[t];
-            const float ax = fmaxf(0.f, fmaxf(xlo - p.x, p.x - xhi)), ay = fmaxf(0.f, fmaxf(ylo - p.y, p.y - yhi)),
-                        az = fmaxf(0.f, fmaxf(zlo - p.z, p.z - zhi));
-            keep = fmaf(ax, ax, fmaf(ay, ay, az * az)) <= reach2;
+    const int total = s_sum[kBuildWarps - 1];
+    s_pre[threadIdx.x + 1] = pre + (warp ? s_sum[warp - 1] : 0);
+    if (threadIdx.x == 0) s_pre[0] = 0;
+    __syncthreads();
+    if (total == 0) {   // no atom in the group either
+      if constexpr (LIST) continue;
+      else return;
+    }
+
+    // ---- rounds: stage candidates (ordered), then test them against every warp's atoms
+    int at = 0, staged = 0;   // uniform over the block
+    bool first_round = true;
+    while (true) {
+      bool full = false;
+      while (at < total) {
+        const int f = at + threadIdx.x;
+        bool keep = false;
+        float px = 0.f, py_ = 0.f, pz_ = 0.f;
+        int j = 0, ko = 0;
+        if (f < total) {
+          int lo = 0, hi = n_runs - 1;   // the run of candidate f: the last one with s_pre <= f
+          while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (s_pre[mid] <= f) lo = mid;
+            else hi = mid - 1;
           }
-          const unsigned mk = __ballot_sync(0xffffffffu, keep);
-          if (listed + __popc(mk) > kList<ACE>) break;
-          if (keep) list[listed + __popc(mk & lt)] = (unsigned short)t;
-          listed += __popc(mk);
-          from += 32;
+          const int slot = s_beg[lo] + f - s_pre[lo], o = s_run[lo];
+          j = A.catoms[slot];
+          const float4 sj = ACE ? A.s32[j] : A.s32c[slot];
+          const int kx = cell_x(__float_as_int(sj.w)) + (ix_lo + (o >> 24)) * nx - x0;
+          ko = (o & 0xffffff) + kx;
+          px = fmaf((float)kx, hx, sj.x);
+          py_ = fmaf((float)off_y(o), hy, sj.y);
+          pz_ = fmaf((float)off_z(o), hz, sj.z);
+          const float ax = fmaxf(0.f, fmaxf(blo - px, px - gxh)), ay = fmaxf(0.f, fmaxf(blo - py_, py_ - gyh)),
+                      az = fmaxf(0.f, fmaxf(blo - pz_, pz_ - gzh));
+          keep = ax * ax + ay * ay + az * az <= reach2;
         }
-        __syncwarp();
-        direct = first && from >= staged;   // all candidates are in the list: rows are written in place
-        first = false;
-        // lane t takes candidates K t .. K t + K - 1 of the list
-        const int K = (listed + 31) >> 5, base = K * lane, nk = min(K, listed - base);
-        for (int u0 = 0; u0 < nc; u0 += kCentres) {
-          float cx[kCentres], cy[kCentres], cz[kCentres];
-          int ci[kCentres];
-          unsigned m[kCentres];   // bit k: candidate k is inside r_c; bit 16 + k: in the skin
+        const unsigned mk = __ballot_sync(0xffffffffu, keep);
+        __syncthreads();
+        if (lane == 0) s_sum[warp] = __popc(mk);
+        __syncthreads();
+        int before = 0, sum = 0;
 #pragma unroll
-          for (int u = 0; u < kCentres; ++u) {
-            const int src = min(u0 + u, nc - 1);
-            cx[u] = __shfl_sync(0xffffffffu, mex, src);
-            cy[u] = __shfl_sync(0xffffffffu, mey, src);
-            cz[u] = __shfl_sync(0xffffffffu, mez, src);
-            ci[u] = __shfl_sync(0xffffffffu, me_i, src);
-            m[u] = 0;
+        for (int w = 0; w < kBuildWarps; ++w) {
+          const int v = s_sum[w];
+          before += w < warp ? v : 0;
+          sum += v;
+        }
+        if (staged + sum > kStage) {   // uniform: no room, test what is staged first
+          full = true;
+          break;
+        }
+        if (keep) {
+          const int q = staged + before + __popc(mk & lt);
+          s_pos[q] = make_float4(px, py_, pz_, __int_as_float(j));
+          if (STORED) s_cell[q] = ko;
+        }
+        staged += sum;
+        at += T;
+      }
+      __syncthreads();
+      for (int c0 = 0; c0 < own; c0 += 32) {   // up to 32 of the warp's atoms, one per lane
+        int nc = min(32, own - c0);
+        int slot = b + part + (c0 + min(lane, nc - 1)) * parts;
+        if constexpr (ACE) {   // the queued ones of them
+          const unsigned queued = __ballot_sync(0xffffffffu, lane < nc && A.qpos[A.catoms[slot]] >= 0);
+          if (!queued) continue;
+          if (queued >> lane & 1) s_own[warp][__popc(queued & lt)] = slot;
+          nc = __popc(queued);
+          __syncwarp();
+          slot = s_own[warp][min(lane, nc - 1)];
+          __syncwarp();
+        }
+        const int me_i = A.catoms[slot];
+        const int me_row = ACE ? A.qpos[me_i] : me_i;
+        const float4 sm = ACE ? A.s32[me_i] : A.s32c[slot];
+        const float mex = fmaf((float)ux, hx, sm.x), mey = fmaf((float)uy, hy, sm.y), mez = fmaf((float)uz, hz, sm.z);
+        int n_in = 0, n_skin = 0;   // entries found so far for this lane's atom
+        if (!first_round) {
+          n_in = ACE ? A.cnt[me_row] : A.nin[me_row];
+          n_skin = ACE ? 0 : A.cnt[me_row];
+        }
+        const float xlo = warp_min(mex), xhi = warp_max(mex), ylo = warp_min(mey), yhi = warp_max(mey),
+                    zlo = warp_min(mez), zhi = warp_max(mez);
+        unsigned short* const list = s_list[warp];
+        int from = 0;
+        bool first = first_round && !full, direct = false;
+        do {
+          // list the staged candidates within reach of this warp's atoms
+          int listed = 0;
+          while (from < staged) {
+            const int t = from + lane;
+            bool keep = false;
+            if (t < staged) {
+              const float4 p = s_pos[t];
+              const float ax = fmaxf(0.f, fmaxf(xlo - p.x, p.x - xhi)), ay = fmaxf(0.f, fmaxf(ylo - p.y, p.y - yhi)),
+                          az = fmaxf(0.f, fmaxf(zlo - p.z, p.z - zhi));
+              keep = fmaf(ax, ax, fmaf(ay, ay, az * az)) <= reach2;
+            }
+            const unsigned mk = __ballot_sync(0xffffffffu, keep);
+            if (listed + __popc(mk) > kList<ACE>) break;
+            if (keep) list[listed + __popc(mk & lt)] = (unsigned short)t;
+            listed += __popc(mk);
+            from += 32;
           }
-          for (int k = 0; k < nk; ++k) {
-            const float4 p = s_pos[list[base + k]];
-            const unsigned b_in = 1u << k, b_sk = 0x10000u << k;
+          __syncwarp();
+          direct = first && from >= staged;   // all candidates are in the list: rows are written in place
+          first = false;
+          // lane t takes candidates K t .. K t + K - 1 of the list
+          const int K = (listed + 31) >> 5, base = K * lane, nk = min(K, listed - base);
+          for (int u0 = 0; u0 < nc; u0 += kCentres) {
+            float cx[kCentres], cy[kCentres], cz[kCentres];
+            int ci[kCentres];
+            unsigned m[kCentres];   // bit k: candidate k is inside r_c; bit 16 + k: in the skin
 #pragma unroll
             for (int u = 0; u < kCentres; ++u) {
-              const float dx = p.x - cx[u], dy = p.y - cy[u], dz = p.z - cz[u];
-              const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-              const unsigned bit = r2 < A.rpf2 ? b_in : b_sk;
-              if (r2 < r_sure) m[u] |= bit;
-              if (fabsf(r2 - A.rcf2) <= band || r2 < 1e-6f) {
-                const int j = __float_as_int(p.w);
-                const int o = STORED ? s_cell[list[base + k]] - (pack_off(ux, uy, uz) - pack_off(0, 0, 0)) : 0;
-                if (r2 < 1e-6f && j == ci[u] && (!STORED || o == pack_off(0, 0, 0))) {
-                  m[u] &= ~bit;   // the atom itself
-                } else if (fabsf(r2 - A.rcf2) <= band) {
-                  m[u] &= ~bit;
-                  if (decide(A, S, ci[u], j, o, STORED)) m[u] |= bit;
+              const int src = min(u0 + u, nc - 1);
+              cx[u] = __shfl_sync(0xffffffffu, mex, src);
+              cy[u] = __shfl_sync(0xffffffffu, mey, src);
+              cz[u] = __shfl_sync(0xffffffffu, mez, src);
+              ci[u] = __shfl_sync(0xffffffffu, me_i, src);
+              m[u] = 0;
+            }
+            for (int k = 0; k < nk; ++k) {
+              const float4 p = s_pos[list[base + k]];
+              const unsigned b_in = 1u << k, b_sk = 0x10000u << k;
+#pragma unroll
+              for (int u = 0; u < kCentres; ++u) {
+                const float dx = p.x - cx[u], dy = p.y - cy[u], dz = p.z - cz[u];
+                const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+                const unsigned bit = r2 < A.rpf2 ? b_in : b_sk;
+                if (r2 < r_sure) m[u] |= bit;
+                if (fabsf(r2 - A.rcf2) <= band || r2 < 1e-6f) {
+                  const int j = __float_as_int(p.w);
+                  const int o = STORED ? s_cell[list[base + k]] - (pack_off(ux, uy, uz) - pack_off(0, 0, 0)) : 0;
+                  if (r2 < 1e-6f && j == ci[u] && (!STORED || o == pack_off(0, 0, 0))) {
+                    m[u] &= ~bit;   // the atom itself
+                  } else if (fabsf(r2 - A.rcf2) <= band) {
+                    m[u] &= ~bit;
+                    if (decide(A, S, ci[u], j, o, STORED)) m[u] |= bit;
+                  }
                 }
+              }
+            }
+            __syncwarp();
+#pragma unroll
+            for (int u = 0; u < kCentres; ++u) {
+              if (u0 + u >= nc) break;
+              const int cnt = __popc(m[u] & 0xffffu) | (__popc(m[u] >> 16) << 16);
+              int sum = cnt;   // inclusive scan of both counts
+#pragma unroll
+              for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, sum, o);
+                if (lane >= o) sum += v;
+              }
+              const int tot = __shfl_sync(0xffffffffu, sum, 31);
+              const int ni = __shfl_sync(0xffffffffu, n_in, u0 + u), ns = __shfl_sync(0xffffffffu, n_skin, u0 + u);
+              sum -= cnt;
+              // in-range entries fill the row from the front; skin entries from the row's end, or,
+              // while more candidates are to come, from the end of its capacity
+              int q_in = ni + (sum & 0xffff);
+              int q_sk = (direct ? ni + (tot & 0xffff) + ns + (tot >> 16) : A.cap) - 1 - ns - (sum >> 16);
+              const size_t row = (size_t)(ACE ? __shfl_sync(0xffffffffu, me_row, u0 + u) : ci[u]) * A.cap;
+              unsigned bits = m[u];
+              while (bits) {
+                const int k = __ffs(bits) - 1;
+                bits &= bits - 1;
+                const int q = k < 16 ? q_in++ : q_sk--;
+                if (q >= 0 && q < A.cap) {
+                  const int t = list[base + (k & 15)];
+                  A.nbr[row + q] = __float_as_int(s_pos[t].w);
+                  if (STORED) A.off[row + q] = s_cell[t] - (pack_off(ux, uy, uz) - pack_off(0, 0, 0));
+                }
+              }
+              if (lane == u0 + u) {
+                n_in = ni + (tot & 0xffff);
+                n_skin = ns + (tot >> 16);
               }
             }
           }
           __syncwarp();
-#pragma unroll
-          for (int u = 0; u < kCentres; ++u) {
-            if (u0 + u >= nc) break;
-            const int cnt = __popc(m[u] & 0xffffu) | (__popc(m[u] >> 16) << 16);
-            int sum = cnt;   // inclusive scan of both counts
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-              const int v = __shfl_up_sync(0xffffffffu, sum, o);
-              if (lane >= o) sum += v;
-            }
-            const int tot = __shfl_sync(0xffffffffu, sum, 31);
-            const int ni = __shfl_sync(0xffffffffu, n_in, u0 + u), ns = __shfl_sync(0xffffffffu, n_skin, u0 + u);
-            sum -= cnt;
-            // in-range entries fill the row from the front; skin entries from the row's end, or,
-            // while more candidates are to come, from the end of its capacity
-            int q_in = ni + (sum & 0xffff);
-            int q_sk = (direct ? ni + (tot & 0xffff) + ns + (tot >> 16) : A.cap) - 1 - ns - (sum >> 16);
-            const size_t row = (size_t)(ACE ? __shfl_sync(0xffffffffu, me_row, u0 + u) : ci[u]) * A.cap;
-            unsigned bits = m[u];
-            while (bits) {
-              const int k = __ffs(bits) - 1;
-              bits &= bits - 1;
-              const int q = k < 16 ? q_in++ : q_sk--;
-              if (q >= 0 && q < A.cap) {
-                const int t = list[base + (k & 15)];
-                A.nbr[row + q] = __float_as_int(s_pos[t].w);
-                if (STORED) A.off[row + q] = s_cell[t] - (pack_off(ux, uy, uz) - pack_off(0, 0, 0));
-              }
-            }
-            if (lane == u0 + u) {
-              n_in = ni + (tot & 0xffff);
-              n_skin = ns + (tot >> 16);
+        } while (from < staged);
+        if (full) {   // another round follows
+          if (lane < nc) {
+            if (!ACE) A.nin[me_row] = n_in;
+            A.cnt[me_row] = ACE ? n_in : n_skin;
+          }
+          continue;
+        }
+        // rows of more than one turn: the skin entries move from [cap - n_skin, cap) to [n_in, cnt),
+        // each run of 32 read in full before it is written; its destinations lie below every source
+        // of the later runs.  An overflowing row holds cap valid entries (the capacity error makes
+        // the caller rebuild or fail before any result is used).
+        const int cnt = n_in + n_skin;
+        for (int u = 0; !ACE && !direct && u < nc; ++u) {
+          const int i = __shfl_sync(0xffffffffu, me_i, u), ni = __shfl_sync(0xffffffffu, n_in, u),
+                    ns = __shfl_sync(0xffffffffu, n_skin, u);
+          if (ni + ns >= A.cap) continue;
+          for (int which = 0; which < (STORED ? 2 : 1); ++which) {
+            int* r = (which ? A.off : A.nbr) + (size_t)i * A.cap;
+            for (int k0 = 0; k0 < ns; k0 += 32) {
+              const int k = k0 + lane;
+              const int v = k < ns ? r[A.cap - ns + k] : 0;
+              __syncwarp();
+              if (k < ns) r[ni + k] = v;
             }
           }
         }
-        __syncwarp();
-      } while (from < staged);
-      if (full) {   // another round follows
         if (lane < nc) {
-          if (!ACE) A.nin[me_row] = n_in;
-          A.cnt[me_row] = ACE ? n_in : n_skin;
-        }
-        continue;
-      }
-      // rows of more than one turn: the skin entries move from [cap - n_skin, cap) to [n_in, cnt),
-      // each run of 32 read in full before it is written; its destinations lie below every source
-      // of the later runs.  An overflowing row holds cap valid entries (the capacity error makes
-      // the caller rebuild or fail before any result is used).
-      const int cnt = n_in + n_skin;
-      for (int u = 0; !ACE && !direct && u < nc; ++u) {
-        const int i = __shfl_sync(0xffffffffu, me_i, u), ni = __shfl_sync(0xffffffffu, n_in, u),
-                  ns = __shfl_sync(0xffffffffu, n_skin, u);
-        if (ni + ns >= A.cap) continue;
-        for (int which = 0; which < (STORED ? 2 : 1); ++which) {
-          int* r = (which ? A.off : A.nbr) + (size_t)i * A.cap;
-          for (int k0 = 0; k0 < ns; k0 += 32) {
-            const int k = k0 + lane;
-            const int v = k < ns ? r[A.cap - ns + k] : 0;
-            __syncwarp();
-            if (k < ns) r[ni + k] = v;
+          A.cnt[me_row] = min(cnt, A.cap);
+          if constexpr (!ACE)
+            A.nin[me_row] = min(n_in, A.cap);   // the in-range part (read by the CSP on rows built at its positions)
+          else if (min(cnt, A.cap) > __ldcg(&A.sc->ace_row_max))   // only a new maximum takes the (same-address) atomic
+            atomicMax(&A.sc->ace_row_max, min(cnt, A.cap));
+          if (cnt > A.cap) {
+            atomicMax(ACE ? &A.sc->need_ace : &A.sc->need_eam, cnt);
+            atomicOr(&A.sc->err, kErrCapacity);
           }
         }
       }
-      if (lane < nc) {
-        A.cnt[me_row] = min(cnt, A.cap);
-        if constexpr (!ACE)
-          A.nin[me_row] = min(n_in, A.cap);   // the in-range part (read by the CSP on rows built at its positions)
-        else if (min(cnt, A.cap) > __ldcg(&A.sc->ace_row_max))   // only a new maximum takes the (same-address) atomic
-          atomicMax(&A.sc->ace_row_max, min(cnt, A.cap));
-        if (cnt > A.cap) {
-          atomicMax(ACE ? &A.sc->need_ace : &A.sc->need_eam, cnt);
-          atomicOr(&A.sc->err, kErrCapacity);
-        }
-      }
+      if (!full) break;
+      first_round = false;
+      staged = 0;
+      __syncthreads();   // the stage is refilled
     }
-    if (!full) break;
-    first_round = false;
-    staged = 0;
-    __syncthreads();   // the stage is refilled
-  }
-  if constexpr (!LIST) return;   // one block per group
+    if constexpr (!LIST) return;   // one block per group
   }
 }
 
