@@ -16,7 +16,7 @@
 //                  shared tiles; A = (1/N0) W . G; nu = 1, 2 energy and gradient;
 //   k_ace_nu3      (k_ace_nu3.cu) the nu = 3 energy and gradient as straight-line code over
 //                  the merged monomials generated from the basis (ace_nu3.inc);
-//   k_ace_adjoint  8 or 16 lanes per precise atom: u = W^T dE/dA / N0; each lane evaluates
+//   k_ace_adjoint  8 or 32 lanes per precise atom: u = W^T dE/dA / N0; each lane evaluates
 //                  the pair force of one neighbour at a time from u (pair_force) and
 //                  scatters -w_i p_ij to neighbour j; +w_i sum p goes to i.
 #include <complex>
