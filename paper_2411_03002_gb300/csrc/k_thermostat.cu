@@ -169,10 +169,10 @@ __device__ inline bool member(const int* __restrict__ row, int t, int i, const u
 // member carries mass 0 at index i, and what the chain needs of the coming atoms is loaded one
 // turn ahead (three turns of indices).  Rows beyond 32 kMem entries take the loop over memory.
 // The time of an update follows the number of corrections, few while a run is young.  On a slab of
-// 358,012 atoms with 405 / 5,970 / 21,750 / 32,700 of them (third, fourth, fifth and 48th update) the
-// thermostat takes 1.7 / 4.1 / 6.6 / 8.5 ms; 23 / 64 / 108 / 145 ms with a membership test over the
-// whole row for boxes that cannot need it, a tenth more without the loads ahead.  What is left is the
-// FP64 chain of two divisions, a square root and 11 dependent additions.
+// 358,012 atoms with 405 / 5,970 / 21,750 / 32,700 of them (third, fourth, fifth and 48th update)
+// the thermostat takes 1.7 / 4.1 / 6.6 / 8.5 ms; 23 / 64 / 108 / 145 ms with a membership test over
+// the whole row for boxes that cannot need it.  Loading ahead took 2.4 ms off an update of some
+// 28,000.  What is left is the FP64 chain of two divisions, a square root and 11 dependent additions.
 constexpr int kMem = 6;   // 192 row entries: the default row capacity is 160
 template <bool DEDUP>
 __global__ void __launch_bounds__(32) k_th_rescale(
