@@ -169,7 +169,6 @@ struct CspArgs {
   const int* nin;
   float rpf2, stale2;
   int* n_stale;
-  int sort_from;
 };
 
 // CSP of atom i by sorted FP32 selections; what FP32 cannot decide (an r_search band hit, an
@@ -334,9 +333,9 @@ constexpr int kSortBlocks = 5;   // resident blocks of k_csp_sort per SM (92 reg
 template <bool VEC>
 __global__ void __launch_bounds__(128) k_csp_sort(const CspArgs A, const int* __restrict__ list,
                                                   const int* __restrict__ n_list, int* __restrict__ slow,
-                                                  int* __restrict__ n_slow) {
+                                                  int* __restrict__ n_slow, int sort_from) {
   const int m = *n_list;
-  if (m <= A.sort_from) return;
+  if (m <= sort_from) return;
   for (int t0 = blockIdx.x * blockDim.x; t0 < m; t0 += gridDim.x * blockDim.x) {
     if (t0 + threadIdx.x < m) csp_atom<VEC>(A, list[t0 + threadIdx.x], slow, n_slow);
     __syncwarp();
@@ -508,9 +507,9 @@ __device__ inline K warp_min_key(K v) {
 // list2: what k_csp_sort handed on, when it ran.
 __global__ void __launch_bounds__(128) k_csp_exact(const CspArgs A, const int* __restrict__ list,
                                                    const int* __restrict__ n_list, const int* __restrict__ list2,
-                                                   const int* __restrict__ n_list2) {
+                                                   const int* __restrict__ n_list2, int sort_from) {
   const int lane = threadIdx.x & 31, warps = (gridDim.x * blockDim.x) >> 5;
-  const bool sorted = list && *n_list > A.sort_from;
+  const bool sorted = list && *n_list > sort_from;
   const int m = !list ? A.n : sorted ? *n_list2 : *n_list;
   const unsigned long long none = ~0ull;
   for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < m; w += warps) {
@@ -980,11 +979,11 @@ void launch_csp(ap_ctx* c, const double* d_x, const uint8_t* d_ch, cudaStream_t 
   A.rpf2 = rpf2;
   A.stale2 = stale2;
   A.n_stale = &c->d_sc->n_stale_bad;
-  A.sort_from = kSortFrom * c->num_sms;
+  const int sort_from = kSortFrom * c->num_sms;
   // a few thousand atoms: a warp each at once (237 atoms 14 us; a thread each took 64 us, since
   // one atom's chain is that long)
   if (c->n <= 32 * c->num_sms) {
-    k_csp_exact<<<nblk(c->n, 4), 128, 0, s>>>(A, nullptr, nullptr, nullptr, nullptr);
+    k_csp_exact<<<nblk(c->n, 4), 128, 0, s>>>(A, nullptr, nullptr, nullptr, nullptr, 0);
     c->kernels += 1;
     return;
   }
@@ -993,9 +992,10 @@ void launch_csp(ap_ctx* c, const double* d_x, const uint8_t* d_ch, cudaStream_t 
   near<<<nblk(c->n, 128), 128, 0, s>>>(A, c->d_csp_slow, n_list);
   // the handed-over atoms, grid-stride over the device-side counts; d_det1 is free until the spread
   auto sort = c->cap_eam % 4 == 0 ? k_csp_sort<true> : k_csp_sort<false>;
-  if (c->n > A.sort_from) sort<<<c->num_sms * kSortBlocks, 128, 0, s>>>(A, c->d_csp_slow, n_list, c->d_det1, n_slow);
-  k_csp_exact<<<c->num_sms * 8, 128, 0, s>>>(A, c->d_csp_slow, n_list, c->d_det1, n_slow);
-  c->kernels += c->n > A.sort_from ? 3 : 2;
+  if (c->n > sort_from)
+    sort<<<c->num_sms * kSortBlocks, 128, 0, s>>>(A, c->d_csp_slow, n_list, c->d_det1, n_slow, sort_from);
+  k_csp_exact<<<c->num_sms * 8, 128, 0, s>>>(A, c->d_csp_slow, n_list, c->d_det1, n_slow, sort_from);
+  c->kernels += c->n > sort_from ? 3 : 2;
 }
 
 // d_score: the detection score pushed into the history (CSP, or the selector's p),
