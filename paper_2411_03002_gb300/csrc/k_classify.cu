@@ -146,7 +146,7 @@ __device__ inline double sum_ascending(double v[kHalf]) {
 //                what FP32 cannot decide is handed on again.
 //   k_csp_exact  one warp per atom, exact selections: what is left, short lists, small systems.
 // Structures without shells (a melt, a gas) take all three: updates of a gas of 50,000 / 100,000 /
-// 200,000 / 1,000,000 atoms 0.43 / 0.60 / 0.94 / 3.76 ms, where a sorting kernel for all atoms and a
+// 200,000 / 1,000,000 atoms 0.43 / 0.60 / 0.93 / 3.73 ms, where a sorting kernel for all atoms and a
 // thread for each of the rest took 0.92 / 0.97 / 1.32 / 3.71 ms.
 // FP64 arithmetic issues one warp instruction per 16 cycles and SM: a warp per atom for all
 // atoms would take 4 ms on 4,000,000 of them, the 89 FP64 operations of a thread 0.57 ms.
